@@ -31,7 +31,7 @@ def sources():
 
 
 def _deps():
-    files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     files.append(os.path.join(os.path.dirname(HERE), "include", "chap.h"))
     return files
 

@@ -197,6 +197,67 @@ chap_status load_state(chap_bs *h, const double *x, const int *w, const int *tab
     return CHAP_OK;
 }
 
+// Device state of the kept-score search.  It is an extra over what the other
+// calls need: a handle whose device memory does not hold it runs the plain
+// iterations instead.
+void search_create(chap_bs *h, int bin_cols, int64_t nnz, double touched)
+{
+    Search &S = h->srch;
+    const int m = h->m;
+    S.bc = bin_cols;
+    S.nblk = (bin_cols + 255) / 256;
+    S.nvb = (m + 255) / 256;
+    if (!search_shape(S, touched <= kSrOneCtaTouched)) {
+        S = Search{};
+        return;
+    }
+    const size_t kept = h->allocs.size();
+    S.kS = dalloc<long long>(h, bin_cols);
+    S.kD = dalloc<int>(h, bin_cols);
+    S.bS = dalloc<long long>(h, S.nblk);
+    S.bV = dalloc<int2>(h, S.nblk);
+    S.bdirty = dalloc<int>(h, S.nblk);
+    S.vcnt = dalloc<int>(h, S.nvb);
+    S.epos = dalloc<int>(h, nnz);
+    S.eval = dalloc<long long>(h, nnz);
+    S.head = dalloc<int2>(h, (size_t)bin_cols * kSrHead);
+    S.rec = dalloc<SrRec>(h, m);
+    S.chunk = dalloc<int2>(h, search_chunks(S, m, nnz));
+    S.sc = dalloc<SrCtl>(h, 1);
+    if (S.kS && S.kD && S.bS && S.bV && S.bdirty && S.vcnt && S.epos && S.eval && S.head && S.rec && S.chunk && S.sc &&
+        launch_keep_entries(h->dev, S, h->st) == cudaSuccess) {
+        S.on = 1;
+        return;
+    }
+    cudaGetLastError();
+    while (h->allocs.size() > kept) {
+        cudaFree(h->allocs.back());
+        h->allocs.pop_back();
+    }
+    S = Search{};
+}
+
+// Iterations of chap_tabu_run on kept scores, from a state whose run has begun
+// (launch_begin_run): all kept values first, then launches of up to
+// kSrLaunchIters iterations.  A launch also ends early when a walk is left to
+// the whole GPU; then more launches are queued before the host looks again.
+chap_status search_run(chap_bs *h)
+{
+    CK(h, launch_keep_build(h->dev, h->plan, h->srch, h->st), "kept scores");
+    long long seen = h->h_ctl->iter;
+    for (int rounds = 1;;) {
+        for (int r = 0; r < rounds; ++r) CK(h, launch_search(h->dev, h->srch, kSrLaunchIters, h->st), "search");
+        const long long before = seen;
+        chap_status s = read_ctl(h);
+        if (s != CHAP_OK) return s;
+        if (h->h_ctl->done) return CHAP_OK;
+        seen = h->h_ctl->iter;
+        if (seen == before) return fail(h, CHAP_E_CUDA, "the search made no progress");
+        const bool early = seen - before < (long long)rounds * kSrLaunchIters;
+        rounds = early ? std::min(2 * rounds, 32) : 1;
+    }
+}
+
 }  // namespace
 
 namespace chap {
@@ -756,6 +817,11 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     }
     const int n_tb = bin_blk ? blk_nfin
                    : bin_rows ? rb_blocks * kRbCluster : (bin_cols > 0 ? bin_grid_size(bin_cols, bin_G) : 0);
+    // chap_tabu_run keeps the scores of a run (search.cuh) when every evaluated
+    // column is binary and no option asks for another evaluation; 2^31 scores
+    // of half weights are not assumed to fit: the kept sums are int64
+    const bool all_bin = bin_cols > 0 && bin_cols == kind_base[T_NUM_KINDS] && m > 0 && !lazy_bin && !bin_rows &&
+                         h->opt.bin_kernel != 3 && h->shard_count == 1;
     const int n_tc = (int)tiles_cta.size();
     const int slot_hist = n_tb + n_tn + n_tc;
     for (size_t q = 0; q < hcols.size(); ++q) hcols[q].slot = slot_hist + (int)q;
@@ -835,9 +901,11 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         rbvf_d = dalloc<double>(h, rb_vf.size());
     }
     BinBlk bbd{};
-    if (bin_blk) {
+    if (bin_blk || all_bin) {
         d.bup = dalloc<unsigned char>(h, bin_cols);
         d.n_bup = bin_cols;
+    }
+    if (bin_blk) {
         bbd.nblk = nblk;
         bbd.rows = blk_rows;
         bbd.n_items = (int)blk_items.size();
@@ -850,8 +918,8 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         bbd.acc_s = dalloc<long long>(h, bin_cols);
         bbd.acc_dc = dalloc<int>(h, bin_cols);
     }
-    const bool blk_ok = !bin_blk || (d.bup && bbd.items && bbd.metaI && bbd.metaF && bbd.valI && bbd.valF &&
-                                     bbd.acc_s && bbd.acc_dc);
+    const bool blk_ok = (d.bup || !(bin_blk || all_bin)) && (!bin_blk || ( bbd.items && bbd.metaI && bbd.metaF && bbd.valI && bbd.valF &&
+                                     bbd.acc_s && bbd.acc_dc));
     LongCol *lc_d = dalloc<LongCol>(h, lcols.size());
     Tile *tlg_d = dalloc<Tile>(h, tiles_lgen.size()), *tls_d = dalloc<Tile>(h, tiles_lscan.size());
     d.n_long = (int)lcols.size();
@@ -958,6 +1026,15 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         free_all(h);
         delete h;
         return CHAP_E_CUDA;
+    }
+    if (all_bin) {
+        // mean entries a move's walk meets: sum of len^2 over the rows, per column
+        double touched = 0.0;
+        for (int i = 0; i < m; ++i) {
+            const double len = (double)(p->row_ptr[i + 1] - p->row_ptr[i]);
+            touched += len * len;
+        }
+        search_create(h, bin_cols, p->nnz, touched / std::max(1, n));
     }
     pl.apply_blocks = (int)std::min<int64_t>(304, std::max<int64_t>(1, ((int64_t)m + kApplyThreads - 1) / kApplyThreads));
     pl.apply_move_blocks = (int)std::min<int64_t>(152, std::max<int64_t>(1, ((int64_t)max_col + kApplyMoveThreads - 1) / kApplyMoveThreads));
@@ -1344,6 +1421,10 @@ chap_status chap_tabu_run(chap_bs *h, const chap_options *opts, chap_tabu_result
         return fail(h, CHAP_E_UNSUPPORTED, "iteration counter would exceed the 32-bit tabu stamps");
     Dev &d = h->dev;
     CK(h, launch_begin_run(d, o.max_iters, o.stop_at_feasible, h->st), "begin run");
+    if (h->srch.on && !h->h_ctl->cut_on) {
+        s = search_run(h);
+        if (s != CHAP_OK) return s;
+    } else {
     if (!h->gexec || h->g_iters != o.graph_iters) {
         if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }
         cudaGraph_t g = nullptr;
@@ -1369,6 +1450,7 @@ chap_status chap_tabu_run(chap_bs *h, const chap_options *opts, chap_tabu_result
         s = read_ctl(h);
         if (s != CHAP_OK) return s;
         if (h->h_ctl->done) break;
+    }
     }
     auto t1 = std::chrono::steady_clock::now();
     const Ctl c = *h->h_ctl;

@@ -23,6 +23,7 @@ struct chap_bs {
     std::vector<void *> allocs;
     Dev dev{};
     LaunchPlan plan{};
+    chap::Search srch{};        // kept-score search of chap_tabu_run (srch.on: in use)
     // device scratch for host-memory outputs
     double *t_xhat = nullptr;
     long long *t_s = nullptr;

@@ -312,6 +312,46 @@ struct Dev {
 
 
 
+// Kept-score search of chap_tabu_run (search.cuh).  A changed row as the walk
+// needs it: residual before and after the change, weights before it and which
+// of them it raises (inc: bit 0 first half, bit 1 second), the row's CSR
+// entries.
+struct __align__(16) SrRec {
+    long long r0, r1;
+    double eps;              // 0 on integral rows
+    long long p0;
+    int len, w1, w2, inc;
+    int integral, pad[3];
+};
+
+struct __align__(16) SrCtl {
+    unsigned nchunks, nrec;  // walk chunks and records of the current iteration
+    int pending;             // a walk is left to k_search_walk
+    int moved;               // position of the moved column (-1: a weight update)
+};
+
+struct Search {
+    int on;                  // chap_tabu_run uses the kept-score search
+    int nct;                 // CTAs of k_search (1, or one cluster)
+    int bc;                  // binary positions [0, bc)
+    int nblk;                // summary blocks of the binary positions
+    int nvb;                 // blocks of physical rows with a violation count
+    int flip_words;          // words of the flip bits in k_search's shared memory (0: d.bup is read)
+    int smem;                // dynamic shared memory of k_search
+    long long *kS;           // flip score and violation change of every binary position
+    int *kD;
+    long long *bS;           // per summary block: best score, (variable, position), dirty flag
+    int2 *bV;
+    int *bdirty;
+    int *vcnt;               // violated normalised rows per row block
+    int *epos;               // per CSR entry: position of its column, coefficient
+    long long *eval;
+    int2 *head;              // first kSrHead integral entries (row, coefficient) of every binary position
+    SrRec *rec;              // [m]
+    int2 *chunk;             // (record, part) of the walk
+    SrCtl *sc;
+};
+
 // Optional per-variable outputs of a best-shift pass (device pointers, may be null).
 struct VarOut {
     double *xhat;
@@ -386,6 +426,15 @@ cudaError_t launch_move_record(const Dev &d, chap_move_record *rec, cudaStream_t
 cudaError_t launch_subset_nb(const Dev &d, const LaunchPlan &p, const int *list, int k, double *xh,
                              unsigned long long *key, int gate, cudaStream_t st);
 cudaError_t launch_apply_records(const Dev &d, const chap_move_record *recs, int k, cudaStream_t st);
+// Kept-score search: the row entries by position (once per handle), the kept
+// values of a run, up to max_launch iterations with the walk they may leave.
+cudaError_t launch_keep_entries(const Dev &d, const Search &S, cudaStream_t st);
+cudaError_t launch_keep_build(const Dev &d, const LaunchPlan &p, const Search &S, cudaStream_t st);
+cudaError_t launch_search(const Dev &d, const Search &S, int max_launch, cudaStream_t st);
+// Chooses S.nct (one CTA, or the largest cluster that fits the current device)
+// and the shared memory of k_search; false when no shape fits.
+bool search_shape(Search &S, bool one_cta);
+size_t search_chunks(const Search &S, int m, long long nnz);  // capacity of the chunk list
 
 // Sizes used by both sides.
 constexpr int kEvalThreads = 256;
@@ -412,6 +461,11 @@ constexpr int kBlkFinThreads = 256;
 constexpr int kBlkMaxBlocks = 32;       // the library picks the row-blocked flips up to this many row blocks,
 constexpr int kBlkMinCols = 16384;      // from this many binary columns,
 constexpr double kBlkMinSeg = 2.0;      // and from this many entries per (block, column) on average
+// Entries a move changes on average up to which one CTA runs the search (16
+// chunks of 256, one per warp: a cluster would add its barriers and save nothing).
+constexpr double kSrOneCtaTouched = 4096.0;
+constexpr int kSrHead = 8;              // integral column entries addressed by position
+constexpr int kSrLaunchIters = 2048;    // iterations of one launch of the search
 constexpr int kApplyThreads = 256;
 constexpr int kApplyMoveThreads = 1024;
 constexpr int kLazyMaxRows = 2048;      // longer moved columns re-evaluate every kept binary score

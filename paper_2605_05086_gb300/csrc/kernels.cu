@@ -3066,6 +3066,8 @@ __global__ void k_widen(int n, const int *a, long long *b)
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) b[j] = a[j];
 }
 
+#include "search.cuh"
+
 // ---------------------------------------------------------------- launchers
 
 static int grid_for(long long n, int threads, int cap = 152 * 8)
@@ -3162,7 +3164,7 @@ cudaError_t static_hist_scratch(HBin **bins, HistAcc **acc)
 // largest size any handle launches with), under a mutex.
 static cudaError_t raise_smem_limit(const void *fn, int slot, int bytes)
 {
-    constexpr int kMaxDevices = 64, kSlots = 8;
+    constexpr int kMaxDevices = 64, kSlots = 9;
     static std::mutex s_mu;
     static int s_set[kMaxDevices][kSlots] = {};
     int dev = 0;
@@ -3411,6 +3413,84 @@ cudaError_t launch_objective(const Dev &d, double *out, double *partial, cudaStr
 cudaError_t launch_tabu_convert(int n, const int *a, long long *b, cudaStream_t st)
 {
     k_widen<<<grid_for(n, 256), 256, 0, st>>>(n, a, b);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_keep_entries(const Dev &d, const Search &S, cudaStream_t st)
+{
+    if (d.m > 0) k_keep_entries<<<grid_for((long long)d.m * 32, 256, 152 * 16), 256, 0, st>>>(d, S.epos, S.eval);
+    if (S.bc > 0) k_keep_heads<<<grid_for((long long)S.bc * kSrHead, 256, 152 * 16), 256, 0, st>>>(d, S);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_keep_build(const Dev &d, const LaunchPlan &p, const Search &S, cudaStream_t st)
+{
+    // every summary block is stale (any non-zero word marks it)
+    cudaError_t e = cudaMemsetAsync(S.bdirty, 1, sizeof(int) * (size_t)S.nblk, st);
+    if (e != cudaSuccess) return e;
+    k_keep_rows<<<S.nvb, kSrBlk, 0, st>>>(d, S);
+    if (S.bc > 0) {
+        const int grid = bin_grid_size(S.bc, p.bin_G);
+        switch (p.bin_G) {
+        case 2: k_keep_bin<2><<<grid, kEvalThreads, 0, st>>>(d, S); break;
+        case 4: k_keep_bin<4><<<grid, kEvalThreads, 0, st>>>(d, S); break;
+        case 16: k_keep_bin<16><<<grid, kEvalThreads, 0, st>>>(d, S); break;
+        default: k_keep_bin<8><<<grid, kEvalThreads, 0, st>>>(d, S); break;
+        }
+    }
+    return cudaGetLastError();
+}
+
+size_t search_chunks(const Search &, int m, long long nnz) { return (size_t)(nnz / kSrChunk) + (size_t)m + 1; }
+
+static void search_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, const Search &S, cudaStream_t st)
+{
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(S.nct);
+    cfg.blockDim = dim3(kSrThreads);
+    cfg.dynamicSmemBytes = S.smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    if (S.nct > 1) {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = S.nct;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.numAttrs = 1;
+    }
+}
+
+bool search_shape(Search &S, bool one_cta)
+{
+    // clusters of more than 8 CTAs are a size the device may or may not offer
+    if (cudaFuncSetAttribute((const void *)k_search, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        cudaGetLastError();
+    const int words = (S.bc + 31) / 32;
+    S.flip_words = words <= kSrFlipWords ? words : 0;
+    for (S.nct = one_cta && S.nblk <= kSrMaxTops ? 1 : kSrMaxCluster; S.nct >= 1; S.nct >>= 1) {
+        const int nl = (S.nblk + S.nct - 1) / S.nct;
+        if (nl > kSrMaxTops) return false;
+        S.smem = sr_smem_bytes(nl, S.flip_words);
+        if (raise_smem_limit((const void *)k_search, 8, S.smem) == cudaSuccess) {
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute at[1];
+            search_config(cfg, at, S, nullptr);
+            int n = 0;
+            if (S.nct == 1 || (cudaOccupancyMaxActiveClusters(&n, k_search, &cfg) == cudaSuccess && n >= 1)) return true;
+        }
+        cudaGetLastError();
+    }
+    return false;
+}
+
+cudaError_t launch_search(const Dev &d, const Search &S, int max_launch, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    search_config(cfg, at, S, st);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_search, d, S, S.nct, max_launch);
+    if (e != cudaSuccess) return e;
+    k_search_walk<<<152, kSrThreads, 0, st>>>(d, S);
     return cudaGetLastError();
 }
 
