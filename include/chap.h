@@ -334,12 +334,14 @@ CHAP_API chap_status chap_bs_step(struct chap_bs *h, chap_move *out);
 /*
  * Run the tabu search from the current state until no row is violated (when
  * stop_at_feasible) or opts->max_iters iterations have run in this call.
- * Instances whose evaluated columns are all binary run on scores kept from
- * iteration to iteration inside the call (evaluated from scratch at its start,
- * then updated on the rows a move changes; the same moves), in launches of
- * many iterations.  Otherwise, and under an objective cutoff, iterations are
- * recorded into a CUDA graph of opts->graph_iters iterations (Sec. 3.1,
- * "Kernel Specialization", last point) and replayed.
+ * Iterations run on scores kept from one to the next inside the call
+ * (evaluated from scratch at its start, then updated on the rows a move
+ * changes; the same moves), in launches of many iterations.  Instances with
+ * CTA- or merge-sorted columns, handles created with lazy_binary, bin_kernel 2
+ * or 3 or static_scratch_only, handles whose device memory did not hold the
+ * kept state, and runs under an objective cutoff evaluate every iteration from
+ * scratch, recorded into a CUDA graph of opts->graph_iters iterations
+ * (Sec. 3.1, "Kernel Specialization", last point) and replayed.
  * opts may be NULL (the create options).  result (host) is filled on success.
  */
 CHAP_API chap_status chap_tabu_run(struct chap_bs *h, const chap_options *opts, chap_tabu_result *result);

@@ -200,13 +200,25 @@ chap_status load_state(chap_bs *h, const double *x, const int *w, const int *tab
 // Device state of the kept-score search.  It is an extra over what the other
 // calls need: a handle whose device memory does not hold it runs the plain
 // iterations instead.
-void search_create(chap_bs *h, int bin_cols, int64_t nnz, double touched)
+void search_create(chap_bs *h, int bin_cols, int nb_cols, const std::vector<int> &hist_vars, int64_t nnz, double touched)
 {
     Search &S = h->srch;
     const int m = h->m;
     S.bc = bin_cols;
     S.nblk = (bin_cols + 255) / 256;
     S.nvb = (m + 255) / 256;
+    S.nnb = nb_cols;
+    const int hist_cols = (int)hist_vars.size();
+    S.nhist = hist_cols;
+    S.nnblk = (nb_cols + 255) / 256;
+    S.mix = nb_cols + hist_cols > 0 ? 1 : 0;
+    // kept bins: an even number per column, so that pairs are 16-byte aligned
+    std::vector<long long> hoff(hist_cols);
+    for (int k = 0; k < hist_cols; ++k) {
+        hoff[k] = S.hist_bins;
+        const int j = hist_vars[k];
+        S.hist_bins += ((int64_t)(h->ub[j] - h->lb[j]) + 2) & ~1LL;
+    }
     if (!search_shape(S, touched <= kSrOneCtaTouched)) {
         S = Search{};
         return;
@@ -218,13 +230,32 @@ void search_create(chap_bs *h, int bin_cols, int64_t nnz, double touched)
     S.bV = dalloc<int2>(h, S.nblk);
     S.bdirty = dalloc<int>(h, S.nblk);
     S.vcnt = dalloc<int>(h, S.nvb);
+    S.rowinfo = dalloc<SrRow>(h, m);
     S.epos = dalloc<int>(h, nnz);
     S.eval = dalloc<long long>(h, nnz);
     S.head = dalloc<int2>(h, (size_t)bin_cols * kSrHead);
-    S.rec = dalloc<SrRec>(h, m);
-    S.chunk = dalloc<int2>(h, search_chunks(S, m, nnz));
     S.sc = dalloc<SrCtl>(h, 1);
-    if (S.kS && S.kD && S.bS && S.bV && S.bdirty && S.vcnt && S.epos && S.eval && S.head && S.rec && S.chunk && S.sc &&
+    bool mix_ok = true;
+    if (S.mix) {
+        const size_t nx = (size_t)nb_cols + hist_cols;
+        S.kL = dalloc<long long>(h, nb_cols);
+        S.kR = dalloc<long long>(h, nb_cols);
+        S.nctx = dalloc<NbCtx>(h, nb_cols);
+        S.side = dalloc<unsigned char>(h, nb_cols);
+        S.clean = dalloc<unsigned char>(h, nx);
+        S.kU = dalloc<long long>(h, nx);
+        S.cX = dalloc<double>(h, nx);
+        S.cD = dalloc<int>(h, nx);
+        S.hb = dalloc<HBin>(h, S.hist_bins);
+        S.ha = dalloc<HistAcc>(h, hist_cols);
+        S.hctx = dalloc<KeepCtx>(h, hist_cols);
+        long long *ho = dalloc<long long>(h, hist_cols);
+        S.hoff = ho;
+        mix_ok = S.kL && S.kR && S.nctx && S.side && S.clean && S.kU && S.cX && S.cD && S.hb && S.ha && S.hctx && ho &&
+                 h2d(ho, hoff.data(), hoff.size(), h->st) == cudaSuccess &&
+                 cudaStreamSynchronize(h->st) == cudaSuccess;
+    }
+    if (mix_ok && S.kS && S.kD && S.bS && S.bV && S.bdirty && S.vcnt && S.rowinfo && S.epos && S.eval && S.head && S.sc &&
         launch_keep_entries(h->dev, S, h->st) == cudaSuccess) {
         S.on = 1;
         return;
@@ -245,16 +276,18 @@ chap_status search_run(chap_bs *h)
 {
     CK(h, launch_keep_build(h->dev, h->plan, h->srch, h->st), "kept scores");
     long long seen = h->h_ctl->iter;
+    int idle = 0;
     for (int rounds = 1;;) {
         for (int r = 0; r < rounds; ++r) CK(h, launch_search(h->dev, h->srch, kSrLaunchIters, h->st), "search");
-        const long long before = seen;
         chap_status s = read_ctl(h);
         if (s != CHAP_OK) return s;
         if (h->h_ctl->done) return CHAP_OK;
+        const long long n = h->h_ctl->iter - seen;
+        // an iteration left to the whole GPU is counted by the next launch
+        idle = n > 0 ? 0 : idle + 1;
+        if (idle > 2) return fail(h, CHAP_E_CUDA, "the search made no progress");
+        rounds = n < (long long)rounds * kSrLaunchIters ? std::min(2 * rounds, 32) : 1;
         seen = h->h_ctl->iter;
-        if (seen == before) return fail(h, CHAP_E_CUDA, "the search made no progress");
-        const bool early = seen - before < (long long)rounds * kSrLaunchIters;
-        rounds = early ? std::min(2 * rounds, 32) : 1;
     }
 }
 
@@ -817,11 +850,11 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     }
     const int n_tb = bin_blk ? blk_nfin
                    : bin_rows ? rb_blocks * kRbCluster : (bin_cols > 0 ? bin_grid_size(bin_cols, bin_G) : 0);
-    // chap_tabu_run keeps the scores of a run (search.cuh) when every evaluated
-    // column is binary and no option asks for another evaluation; 2^31 scores
-    // of half weights are not assumed to fit: the kept sums are int64
-    const bool all_bin = bin_cols > 0 && bin_cols == kind_base[T_NUM_KINDS] && m > 0 && !lazy_bin && !bin_rows &&
-                         h->opt.bin_kernel != 3 && h->shard_count == 1;
+    // chap_tabu_run keeps the scores of a run (search.cuh) when no column needs
+    // the CTA or merge sort and no option asks for another evaluation
+    const bool keep = kind_base[T_NUM_KINDS] > 0 && kind_base[T_NB_CTA] == kind_base[T_NB_CTA + 1] &&
+                      kind_base[T_NB_LONG] == kind_base[T_NB_LONG + 1] && m > 0 && h->opt.lazy_binary == 0 &&
+                      h->opt.bin_kernel < 2 && h->opt.static_scratch_only == 0 && h->shard_count == 1;
     const int n_tc = (int)tiles_cta.size();
     const int slot_hist = n_tb + n_tn + n_tc;
     for (size_t q = 0; q < hcols.size(); ++q) hcols[q].slot = slot_hist + (int)q;
@@ -901,7 +934,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         rbvf_d = dalloc<double>(h, rb_vf.size());
     }
     BinBlk bbd{};
-    if (bin_blk || all_bin) {
+    if (bin_blk || keep) {
         d.bup = dalloc<unsigned char>(h, bin_cols);
         d.n_bup = bin_cols;
     }
@@ -918,7 +951,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         bbd.acc_s = dalloc<long long>(h, bin_cols);
         bbd.acc_dc = dalloc<int>(h, bin_cols);
     }
-    const bool blk_ok = (d.bup || !(bin_blk || all_bin)) && (!bin_blk || ( bbd.items && bbd.metaI && bbd.metaF && bbd.valI && bbd.valF &&
+    const bool blk_ok = (d.bup || !(bin_blk || keep)) && (!bin_blk || ( bbd.items && bbd.metaI && bbd.metaF && bbd.valI && bbd.valF &&
                                      bbd.acc_s && bbd.acc_dc));
     LongCol *lc_d = dalloc<LongCol>(h, lcols.size());
     Tile *tlg_d = dalloc<Tile>(h, tiles_lgen.size()), *tls_d = dalloc<Tile>(h, tiles_lscan.size());
@@ -1027,14 +1060,15 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         delete h;
         return CHAP_E_CUDA;
     }
-    if (all_bin) {
+    if (keep) {
+        const std::vector<int> hist_vars(var_list.begin() + kind_base[T_NB_HIST], var_list.begin() + kind_base[T_NB_HIST + 1]);
         // mean entries a move's walk meets: sum of len^2 over the rows, per column
         double touched = 0.0;
         for (int i = 0; i < m; ++i) {
             const double len = (double)(p->row_ptr[i + 1] - p->row_ptr[i]);
             touched += len * len;
         }
-        search_create(h, bin_cols, p->nnz, touched / std::max(1, n));
+        search_create(h, bin_cols, nb_cols, hist_vars, p->nnz, touched / std::max(1, n));
     }
     pl.apply_blocks = (int)std::min<int64_t>(304, std::max<int64_t>(1, ((int64_t)m + kApplyThreads - 1) / kApplyThreads));
     pl.apply_move_blocks = (int)std::min<int64_t>(152, std::max<int64_t>(1, ((int64_t)max_col + kApplyMoveThreads - 1) / kApplyMoveThreads));

@@ -312,22 +312,52 @@ struct Dev {
 
 
 
-// Kept-score search of chap_tabu_run (search.cuh).  A changed row as the walk
-// needs it: residual before and after the change, weights before it and which
-// of them it raises (inc: bit 0 first half, bit 1 second), the row's CSR
-// entries.
+// Kept-score search of chap_tabu_run (search.cuh).  Entries of a physical row
+// in the search's order: first entry, binary and other entries, how far one
+// entry of each kind can move the row's residual (rounded up).
+struct __align__(16) SrRow {
+    long long p0;
+    int nbin, nother;
+    float reach_bin, reach_other;
+    int pad0, pad1;
+};
+
+// A changed row as the walk needs it: residual before and after the change,
+// weights before it and which of them it raises (inc: bit 0 first half, bit 1
+// second), the entries to visit (lenB binary ones from p0, lenN others from
+// p0 + offN).
 struct __align__(16) SrRec {
     long long r0, r1;
     double eps;              // 0 on integral rows
     long long p0;
-    int len, w1, w2, inc;
-    int integral, pad[3];
+    int w1, w2, inc, integral;
+    int lenB, lenN, offN, pad;
 };
 
+// Context of a short non-binary column for the bounds of its halves: distances
+// to the bounds (infinite when unbounded), rounding margin of a breakpoint.
+struct __align__(16) NbCtx {
+    float dl, dh, tol;
+    int isint;
+};
+
+// Context of a counting-sorted (integer) column: bounds relative to its value.
+struct __align__(16) KeepCtx {
+    long long lo, hi, xbi, pad;
+};
+
+// Contexts of a moved non-binary column before and after the move.
+struct SrMovedCtx {
+    NbCtx n[2];
+    KeepCtx h[2];
+};
+
+// State between the launches of a search.
 struct __align__(16) SrCtl {
-    unsigned nchunks, nrec;  // walk chunks and records of the current iteration
-    int pending;             // a walk is left to k_search_walk
+    int pending;             // the iteration's move or weight update is left to k_search_big / k_search_put
     int moved;               // position of the moved column (-1: a weight update)
+    long long dnv;           // change of the violation count by k_search_put
+    SrMovedCtx mc;
 };
 
 struct Search {
@@ -338,17 +368,31 @@ struct Search {
     int nvb;                 // blocks of physical rows with a violation count
     int flip_words;          // words of the flip bits in k_search's shared memory (0: d.bup is read)
     int smem;                // dynamic shared memory of k_search
+    // non-binary columns: place p = position - bc, short ones [0, nnb), then
+    // nhist counting-sorted ones
+    int mix, nnb, nhist, nnblk;
+    long long hist_bins;     // bins of hb
+    long long *kL, *kR;      // short: bound of the score left and right of xbar
+    NbCtx *nctx;
+    unsigned char *side;     // bit 0: x above its lower bound, bit 1: below its upper
+    unsigned char *clean;    // kU, cX, cD are the column's best shift regardless of tabu
+    long long *kU;           // its score, or since then a bound of it
+    double *cX;
+    int *cD;
+    HBin *hb;                // counting-sorted: kept bins (column k from hoff[k], an even number), scalars, contexts
+    const long long *hoff;
+    HistAcc *ha;
+    KeepCtx *hctx;
     long long *kS;           // flip score and violation change of every binary position
     int *kD;
     long long *bS;           // per summary block: best score, (variable, position), dirty flag
     int2 *bV;
     int *bdirty;
     int *vcnt;               // violated normalised rows per row block
-    int *epos;               // per CSR entry: position of its column, coefficient
+    SrRow *rowinfo;
+    int *epos;               // row entries: position of the column, coefficient
     long long *eval;
     int2 *head;              // first kSrHead integral entries (row, coefficient) of every binary position
-    SrRec *rec;              // [m]
-    int2 *chunk;             // (record, part) of the walk
     SrCtl *sc;
 };
 
@@ -434,7 +478,6 @@ cudaError_t launch_search(const Dev &d, const Search &S, int max_launch, cudaStr
 // Chooses S.nct (one CTA, or the largest cluster that fits the current device)
 // and the shared memory of k_search; false when no shape fits.
 bool search_shape(Search &S, bool one_cta);
-size_t search_chunks(const Search &S, int m, long long nnz);  // capacity of the chunk list
 
 // Sizes used by both sides.
 constexpr int kEvalThreads = 256;

@@ -155,6 +155,15 @@ __device__ __forceinline__ unsigned long long global_ns()
 
 __device__ __forceinline__ int4 ld_row16(const RowState *p) { return __ldg(reinterpret_cast<const int4 *>(p)); }
 
+// Half `k` of a row state; LIVE: row states change inside the calling kernel
+// (read through L2, not the read-only path).
+template <bool LIVE>
+__device__ __forceinline__ int4 ld_rowx(const RowState *p, int k)
+{
+    const int4 *v = reinterpret_cast<const int4 *>(p) + k;
+    return LIVE ? __ldcg(v) : __ldg(v);
+}
+
 // The whole 32-byte row state in one 256-bit load: one L1 wavefront per lane
 // instead of one for each 16-byte half (the per-nonzero gathers of the
 // evaluation kernels are bound by these wavefronts).  Row states are 32-byte
@@ -1306,6 +1315,7 @@ __device__ __forceinline__ void fp_half(double r, double a, double m, double mo,
 }
 
 // Both halves of the v-th nonzero of the column (integral part first).
+template <bool LIVE = false>
 __device__ __forceinline__ void gen_entry(const Dev &d, const ColCtx &c, int v, Acc &acc, Half &h1, Half &h2)
 {
     h1.type = 0; h1.mark = 0;
@@ -1314,7 +1324,7 @@ __device__ __forceinline__ void gen_entry(const Dev &d, const ColCtx &c, int v, 
         const int e = c.ci0 + v;
         const int i = __ldg(d.ci_row + e);
         const long long a = __ldg(d.ci_val + e);
-        const int4 st = ld_row16(d.rs + i);
+        const int4 st = ld_rowx<LIVE>(d.rs + i, 0);
         const long long r = row_r(st);
         int_half(r, a, st.z, c, acc, h1);
         if (st.w >= 0) int_half(-r, -a, st.w, c, acc, h2);
@@ -1322,8 +1332,7 @@ __device__ __forceinline__ void gen_entry(const Dev &d, const ColCtx &c, int v, 
         const int e = c.cf0 + (v - c.nI);
         const int i = __ldg(d.cf_row + e);
         const double a = __ldg(d.cf_val + e);
-        const int4 *p = reinterpret_cast<const int4 *>(d.rs + i);
-        const int4 s0 = __ldg(p), s1 = __ldg(p + 1);
+        const int4 s0 = ld_rowx<LIVE>(d.rs + i, 0), s1 = ld_rowx<LIVE>(d.rs + i, 1);
         const double r = i4_double_lo(s0), m1 = i4_double_lo(s1), m2 = i4_double_hi(s1);
         fp_half(r, a, m1, m2, s0.z, c, acc, h1);
         if (s0.w >= 0) fp_half(dflip(r), dflip(a), m2, m1, s0.w, c, acc, h2);
@@ -1677,14 +1686,14 @@ __device__ __forceinline__ VCand group_sort_scan(const ColCtx &c, const Acc &a, 
     return vb;
 }
 
-// Whole-warp evaluation of one column with up to kWarpListMax list entries
-// (columns whose list outgrew the group path; stage holds that many).  Exact
-// breakpoints inline.
-__device__ __noinline__ void column_warp(const Dev &d, const VarOut &o, int q, SEnt *stage, long long iter,
-                                         long long nviol, long long bestnv, Cand &best)
+// The breakpoint list of one column (up to kWarpListMax entries, bounds
+// included) into stage by the calling warp, exact breakpoints inline; acc: the
+// column's scalars in every lane.  Returns the number of entries.  LIVE: row
+// states change inside the calling kernel.
+template <bool LIVE>
+__device__ __forceinline__ int column_list(const Dev &d, const ColCtx &c, SEnt *stage, Acc &acc)
 {
     const int lane = threadIdx.x & 31;
-    const ColCtx c = make_col(d, q, iter);
     const int nv = c.nI + c.nF;
     int cnt;
     {
@@ -1695,12 +1704,12 @@ __device__ __noinline__ void column_warp(const Dev &d, const VarOut &o, int q, S
         }
         cnt = (int)fl + (int)fu;
     }
-    Acc acc{0, 0, 0, 0};
+    acc = Acc{0, 0, 0, 0};
     for (int v = lane; v - lane < nv; v += 32) {
         Half h1, h2;
         h1.type = 0; h1.mark = 0;
         h2.type = 0; h2.mark = 0;
-        if (v < nv) gen_entry(d, c, v, acc, h1, h2);
+        if (v < nv) gen_entry<LIVE>(d, c, v, acc, h1, h2);
 #pragma unroll
         for (int hh = 0; hh < 4; ++hh) {
             const Half &h = (hh & 1) ? h2 : h1;
@@ -1714,6 +1723,18 @@ __device__ __noinline__ void column_warp(const Dev &d, const VarOut &o, int q, S
     }
     warp_allreduce_acc(acc);
     __syncwarp();
+    return cnt;
+}
+
+// Whole-warp evaluation of one column (columns whose list outgrew the group
+// path; stage holds kWarpListMax entries).
+__device__ __noinline__ void column_warp(const Dev &d, const VarOut &o, int q, SEnt *stage, long long iter,
+                                         long long nviol, long long bestnv, Cand &best)
+{
+    const int lane = threadIdx.x & 31;
+    const ColCtx c = make_col(d, q, iter);
+    Acc acc;
+    const int cnt = column_list<false>(d, c, stage, acc);
     VCand vb;
     if (cnt <= 32) vb = group_sort_scan<1, 32>(c, acc, stage, cnt, nviol, bestnv);
     else if (cnt <= 64) vb = group_sort_scan<2, 32>(c, acc, stage, cnt, nviol, bestnv);
@@ -1721,6 +1742,43 @@ __device__ __noinline__ void column_warp(const Dev &d, const VarOut &o, int q, S
     else vb = group_sort_scan<8, 32>(c, acc, stage, cnt, nviol, bestnv);
     if (lane == 0) finish_column(d, o, c, vb, best);
     __syncwarp();
+}
+
+// The best candidate of the column at position q in every lane, and its value,
+// without sorting: each lane takes candidates of the list and sums the deltas
+// that count at its value (pre entries at or left of it, post entries left of
+// it).  n^2 / 32 steps of a short loop instead of a sorting network: for the
+// few columns a search evaluates at a time, whose warps wait for the network's
+// code (15 to 115 KB unrolled) longer than for its arithmetic.
+__device__ __noinline__ VCand column_best(const Dev &d, int q, SEnt *stage, long long iter, long long nviol,
+                                          long long bestnv, double &xh)
+{
+    const int lane = threadIdx.x & 31;
+    const ColCtx c = make_col(d, q, iter);
+    Acc acc;
+    const int cnt = column_list<true>(d, c, stage, acc);
+    VCand vb{0, 0ull, 0, 0};
+#pragma unroll 1
+    for (int k = lane; k - lane < cnt; k += 32) {
+        const SEnt me = k < cnt ? stage[k] : SEnt{c.kxb, 0, make_aux(kClsPostDelta, 0)};
+        const unsigned cls = aux_cls(me.aux);
+        const bool right = me.key > c.kxb;
+        long long s = acc.beta + (right ? acc.alpha : 0);
+        int dc = acc.beta_c + (right ? acc.alpha_c : 0);
+#pragma unroll 4
+        for (int e = 0; e < cnt; ++e) {
+            const SEnt t = stage[e];
+            if (t.key < me.key || (t.key == me.key && aux_post(t.aux) == 0)) {
+                s += t.del;
+                dc += aux_dc(t.aux);
+            }
+        }
+        if (cls == kClsPre || cls == kClsPost) consider(vb, c, me.key, s, dc, nviol, bestnv);
+    }
+    warp_reduce_vc(vb, c);
+    __syncwarp();
+    xh = vb.valid ? key_value(c, vb.key) : c.xb;
+    return vb;
 }
 
 // Classification context of a lane's column (thresholds of the side tests).
@@ -3164,7 +3222,7 @@ cudaError_t static_hist_scratch(HBin **bins, HistAcc **acc)
 // largest size any handle launches with), under a mutex.
 static cudaError_t raise_smem_limit(const void *fn, int slot, int bytes)
 {
-    constexpr int kMaxDevices = 64, kSlots = 9;
+    constexpr int kMaxDevices = 64, kSlots = 11;
     static std::mutex s_mu;
     static int s_set[kMaxDevices][kSlots] = {};
     int dev = 0;
@@ -3186,6 +3244,7 @@ cudaError_t setup_kernel_attributes(const LaunchPlan &p)
                         : raise_smem_limit((const void *)k_eval_nb<8>, 1, nb_smem<8>());
     if (e == cudaSuccess && p.cta_smem > 0) e = raise_smem_limit((const void *)k_eval_cta, 2, p.cta_smem);
     if (e == cudaSuccess && p.hist_smem > 0) e = raise_smem_limit((const void *)k_eval_hist, 3, p.hist_smem);
+    if (e == cudaSuccess && p.hist_smem > 0) e = raise_smem_limit((const void *)k_keep_hist, 9, p.hist_smem);
     if (e == cudaSuccess && p.n_lgen > 0) e = raise_smem_limit((const void *)k_long_gen, 4, long_gen_smem());
     if (e == cudaSuccess && p.bin_rows) e = raise_smem_limit((const void *)k_eval_bin_rows, 5, kRbSmem);
     if (e == cudaSuccess && p.bin_blk) e = raise_smem_limit((const void *)k_eval_bin_blk, 7, blk_smem(p.bb.rows));
@@ -3418,7 +3477,7 @@ cudaError_t launch_tabu_convert(int n, const int *a, long long *b, cudaStream_t 
 
 cudaError_t launch_keep_entries(const Dev &d, const Search &S, cudaStream_t st)
 {
-    if (d.m > 0) k_keep_entries<<<grid_for((long long)d.m * 32, 256, 152 * 16), 256, 0, st>>>(d, S.epos, S.eval);
+    if (d.m > 0) k_keep_entries<<<grid_for((long long)d.m * 32, 256, 152 * 16), 256, 0, st>>>(d, S);
     if (S.bc > 0) k_keep_heads<<<grid_for((long long)S.bc * kSrHead, 256, 152 * 16), 256, 0, st>>>(d, S);
     return cudaGetLastError();
 }
@@ -3429,6 +3488,13 @@ cudaError_t launch_keep_build(const Dev &d, const LaunchPlan &p, const Search &S
     cudaError_t e = cudaMemsetAsync(S.bdirty, 1, sizeof(int) * (size_t)S.nblk, st);
     if (e != cudaSuccess) return e;
     k_keep_rows<<<S.nvb, kSrBlk, 0, st>>>(d, S);
+    if (S.nnb > 0) k_keep_nb<<<grid_for((long long)S.nnb * 8, kEvalThreads, 152 * 8), kEvalThreads, 0, st>>>(d, S);
+    if (S.nhist > 0) {
+        e = cudaMemsetAsync(S.hb, 0, sizeof(HBin) * (size_t)S.hist_bins, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(S.ha, 0, sizeof(HistAcc) * (size_t)S.nhist, st);
+        if (e != cudaSuccess) return e;
+        k_keep_hist<<<p.n_hist_tiles, kHistThreads, p.hist_smem, st>>>(d, S, p.tiles_hist);
+    }
     if (S.bc > 0) {
         const int grid = bin_grid_size(S.bc, p.bin_G);
         switch (p.bin_G) {
@@ -3440,8 +3506,6 @@ cudaError_t launch_keep_build(const Dev &d, const LaunchPlan &p, const Search &S
     }
     return cudaGetLastError();
 }
-
-size_t search_chunks(const Search &, int m, long long nnz) { return (size_t)(nnz / kSrChunk) + (size_t)m + 1; }
 
 static void search_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, const Search &S, cudaStream_t st)
 {
@@ -3462,21 +3526,25 @@ static void search_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, cons
 
 bool search_shape(Search &S, bool one_cta)
 {
+    const void *fn = S.mix ? (const void *)k_search<true> : (const void *)k_search<false>;
     // clusters of more than 8 CTAs are a size the device may or may not offer
-    if (cudaFuncSetAttribute((const void *)k_search, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-        cudaGetLastError();
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
     const int words = (S.bc + 31) / 32;
     S.flip_words = words <= kSrFlipWords ? words : 0;
+    if (S.nhist > kSrMaxHist) return false;
     for (S.nct = one_cta && S.nblk <= kSrMaxTops ? 1 : kSrMaxCluster; S.nct >= 1; S.nct >>= 1) {
-        const int nl = (S.nblk + S.nct - 1) / S.nct;
-        if (nl > kSrMaxTops) return false;
-        S.smem = sr_smem_bytes(nl, S.flip_words);
-        if (raise_smem_limit((const void *)k_search, 8, S.smem) == cudaSuccess) {
+        SrLocal L;
+        S.smem = sr_layout(S, S.nct, nullptr, L);
+        if (L.nl > kSrMaxTops || L.nnl > 0xffff / kSrBlk) return false;   // 16-bit places inside a CTA
+        if (raise_smem_limit(fn, S.mix ? 10 : 8, S.smem) == cudaSuccess) {
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute at[1];
             search_config(cfg, at, S, nullptr);
             int n = 0;
-            if (S.nct == 1 || (cudaOccupancyMaxActiveClusters(&n, k_search, &cfg) == cudaSuccess && n >= 1)) return true;
+            const cudaError_t e = S.nct == 1 ? cudaSuccess
+                                  : S.mix ? cudaOccupancyMaxActiveClusters(&n, k_search<true>, &cfg)
+                                          : cudaOccupancyMaxActiveClusters(&n, k_search<false>, &cfg);
+            if (S.nct == 1 || (e == cudaSuccess && n >= 1)) return true;
         }
         cudaGetLastError();
     }
@@ -3488,9 +3556,13 @@ cudaError_t launch_search(const Dev &d, const Search &S, int max_launch, cudaStr
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
     search_config(cfg, at, S, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_search, d, S, S.nct, max_launch);
+    cudaError_t e = S.mix ? cudaLaunchKernelEx(&cfg, k_search<true>, d, S, S.nct, max_launch)
+                          : cudaLaunchKernelEx(&cfg, k_search<false>, d, S, S.nct, max_launch);
     if (e != cudaSuccess) return e;
-    k_search_walk<<<152, kSrThreads, 0, st>>>(d, S);
+    const int hist = S.nhist * (int)sizeof(HistAcc);
+    if (S.mix) k_search_big<true><<<152 * 4, kSrBigThreads, hist, st>>>(d, S);
+    else k_search_big<false><<<152 * 4, kSrBigThreads, 0, st>>>(d, S);
+    k_search_put<<<152, kSrBigThreads, 0, st>>>(d, S);
     return cudaGetLastError();
 }
 

@@ -54,6 +54,47 @@ INSTANCES = {
 }
 
 
+def integers_long_columns(seed, n_hub=5, rows_per=200, dom=300, n_other=120):
+    """Integer hubs of more than 128 entries (counting-sorted columns) beside
+    short binary, integer and continuous columns, an unbounded integer among
+    them; integral and N(0,1) rows, all senses."""
+    rng = np.random.default_rng(seed)
+    n = n_hub + n_other
+    vt = np.concatenate([np.full(n_hub, inst.VAR_INT), rng.integers(0, 3, size=n_other)]).astype(np.uint8)
+    ub = np.where(vt == inst.VAR_BIN, 1.0, np.where(vt == inst.VAR_INT, 25.0, 8.0))
+    ub[:n_hub] = dom
+    lb = np.zeros(n)
+    lb[n_hub + 1::7] = np.where(vt[n_hub + 1::7] == inst.VAR_BIN, 0.0, -3.0)
+    free = n - 1
+    vt[free], lb[free], ub[free] = inst.VAR_INT, -np.inf, np.inf
+    m = n_hub * rows_per
+    rows, cols, vals, rhs = [], [], [], []
+    sense = rng.choice([0, 1, 2], size=m, p=[0.4, 0.4, 0.2]).astype(np.uint8)
+    for i in range(m):
+        js = np.unique(np.concatenate([[i % n_hub], rng.integers(n_hub, n, size=4)]))
+        a = rng.integers(1, 9, size=len(js)) * np.where(rng.random(len(js)) < 0.5, -1, 1).astype(float)
+        if i % 3 == 0:
+            a = rng.standard_normal(len(js))
+        x = np.array([rng.integers(0, dom) if j < n_hub else rng.integers(0, 2) for j in js], dtype=float)
+        rows.append(np.full(len(js), i)); cols.append(js); vals.append(a)
+        rhs.append(float(a @ x) if i % 3 == 0 else float(np.round(a @ x)))
+    return inst.from_triplets("hubs", n, m, np.concatenate(rows), np.concatenate(cols), np.concatenate(vals), lb, ub,
+                              np.ones(n), np.array(rhs), vt, sense, x0=np.clip(np.zeros(n), lb, ub))
+
+
+INSTANCES.update({
+    # non-binary columns: bounds and kept results, short lists and long ones
+    "general": lambda: inst.gen_general(seed=1, n=6_000, m=3_000, len_cap=300),
+    "general_long": lambda: inst.gen_general(seed=2, n=3_001, m=5_003, len_cap=200),
+    "tiny_mixed": lambda: inst.gen_tiny_mixed(3, n=9, m=8, cont_frac=0.3),
+    "no_binary": lambda: inst.gen_tiny_mixed(8, n=300, m=200, dom=30, cont_frac=1.0),
+    # counting-sorted columns; their own moves (more rows than one record list)
+    "hubs": lambda: integers_long_columns(4),
+    "hubs_700": lambda: integers_long_columns(5, n_hub=3, rows_per=700),
+    "skewed": lambda: inst.gen_skewed(seed=6, n=40_000, m=20_000, n_dense=6, dense_len=6_000),
+})
+
+
 def _same_state(a, b):
     for k in ("x", "w", "tabu_inc", "tabu_dec"):
         assert np.array_equal(a[k], b[k]), k
@@ -68,7 +109,10 @@ def test_search_equals_steps(chap, which, tenure):
     a = chap.BestShift(prob, tenure=tenure)
     b = chap.BestShift(prob, tenure=tenure)
     rng = np.random.default_rng(11)
-    starts = [None, rng.integers(0, 2, size=prob.n).astype(float)]
+    lo, hi = np.maximum(prob.lb, -5.0), np.minimum(prob.ub, 40.0)
+    x = np.where(prob.vtype == inst.VAR_CONT, lo + rng.random(prob.n) * (hi - lo),
+                 np.floor(lo + rng.random(prob.n) * (hi - lo + 1)))
+    starts = [None, np.minimum(x, prob.ub)]
     for x in starts:
         w = None if x is None else rng.integers(1, 6, size=a.m_norm).astype(np.int32)
         a.set_state(x, w)
@@ -99,10 +143,12 @@ def test_search_follows_the_oracle_to_feasibility(chap):
     bs.close()
 
 
-def test_checkpointed_tabu_and_aspiration(chap):
-    """Loaded stamps that make the best flips tabu (the admissible scan), and a
-    best count that lets aspiration through."""
-    prob = binary_rows(12, 700, 400, 6, fp=True)
+@pytest.mark.parametrize("mixed", [False, True])
+def test_checkpointed_tabu_and_aspiration(chap, mixed):
+    """Loaded stamps that make the best flips tabu (the admissible scan; kept
+    results of columns with a tabu direction not used), and a best count that
+    lets aspiration through."""
+    prob = integers_long_columns(12) if mixed else binary_rows(12, 700, 400, 6, fp=True)
     a = chap.BestShift(prob, tenure=5)
     b = chap.BestShift(prob, tenure=5)
     rng = np.random.default_rng(3)
