@@ -415,7 +415,13 @@ CHAP_API chap_status chap_bs_get_cutoff(struct chap_bs *h, chap_cutoff_info *inf
  *   launches per iteration.  barrier_limit_ns > 0 bounds each barrier wait
  *   (default 2 s; 0 keeps the current bound): a wait that runs out ends the
  *   launch, chap_batch_run returns CHAP_E_TIMEOUT and the chains' state is
- *   invalid until chap_batch_reset.  Default: persistent.
+ *   invalid until chap_batch_reset.
+ * Where every column has at most 512 entries and a move changes few row
+ *   entries (set-cover shapes), the default is a third schedule: each chain a
+ *   search of its own on scores kept from iteration to iteration (as
+ *   chap_tabu_run), one CTA per chain, graph_iters unused; else the persistent
+ *   one.  chap_batch_autotune (mode -1) times it with the others and keeps the
+ *   fastest; the calls that set a schedule choose between the first two.
  * The incumbents x of every chain are bitsets (one bit per variable); every
  *   launch carries an L2 access-policy window that keeps them persisting in L2
  *   (Sec. 3.1, "Memory Considerations", fourth point); the batch raises the

@@ -21,13 +21,19 @@
 //          (counters, best, feasibility, done flag);
 //   bump   chains flagged for a bump add 1 to the weight of every violated
 //          normalised row.
-// Two schedules run them: three launches per iteration captured K times into
+// Where every column is short and a move changes few entries (ChainSearch;
+// set-cover shapes), each chain instead runs as a search of its own on kept
+// scores, one CTA per chain for thousands of iterations (k_search_chains), no
+// phase shared between chains; the batch's state is converted to the chains'
+// and back around a run.  This schedule is the default where it applies and
+// competes in the autotuner.
+// Two schedules run them otherwise: three launches per iteration captured K times into
 // one CUDA graph, or one persistent cooperative launch per K iterations whose
 // phases are separated by software grid barriers (each wait bounded by a
 // time limit; a wait that runs out stops the launch and the run returns
 // CHAP_E_TIMEOUT).  The autotuner times the (G, CTAs per SM) schedules on the
 // batch itself.
-#include "../../include/chap.h"
+#include "chap_internal.h"
 
 #include <algorithm>
 #include <chrono>
@@ -50,6 +56,7 @@ constexpr int kBThreads = 256;       // threads of the evaluation CTAs
 constexpr int kApplyT = 256;         // threads of one chain's apply CTA
 constexpr int kBumpBlocks = 8;       // bump CTAs per chain
 constexpr int kVarBits = 22;         // variables per instance < 2^22
+constexpr int kChainIters = 8192;    // iterations of one launch of the chains' own searches
 constexpr long long kScoreLimit = 1LL << 41;
 
 struct __align__(16) BRow {
@@ -403,11 +410,117 @@ __global__ void k_batch_begin(BDev d, long long max_iters, int stop_at_feasible)
     if (ctl->done) atomicAdd(d.n_done, 1u);
 }
 
+// Initial row states of every chain from its instance's (blockIdx.y = chain).
+__global__ void k_batch_reset_rows(BDev d, const BRow *rows0, const long long *inst_row0)
+{
+    const int c = blockIdx.y, k = d.ch_inst[c];
+    const int4 *src = reinterpret_cast<const int4 *>(rows0 + inst_row0[k]);
+    int4 *dst = reinterpret_cast<int4 *>(d.rs + d.ch_roff[c]);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.inst_m[k]; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+
+// The search's row store of one instance from its column store: entry of
+// column q in row i to the next free place of the row (any order: only integer
+// sums are formed over a row), the largest coefficient of each row, and the
+// first entries of every column.
+__global__ void k_chain_entries(int n, const int *cptr, const int *crow, const int *cval, chap::SrRow *rows, int *epos,
+                                long long *eval, int2 *head)
+{
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const int e0 = cptr[q], e1 = cptr[q + 1];
+    for (int e = e0; e < e1; ++e) {
+        chap::SrRow *r = rows + crow[e];
+        const long long at = r->p0 + atomicAdd(&r->nbin, 1);
+        epos[at] = q;
+        eval[at] = cval[e];
+        // non-negative floats order as their bits
+        atomicMax(reinterpret_cast<int *>(&r->reach_bin), __float_as_int(fabsf((float)cval[e]) * 1.0001f));
+    }
+    for (int t = 0; t < chap::kSrHead; ++t)
+        head[(size_t)q * chap::kSrHead + t] = e0 + t < e1 ? make_int2(crow[e0 + t], cval[e0 + t]) : make_int2(0, 0);
+}
+
+// Chain states from the batch's: row states, x as doubles and flip bytes, the
+// control block (blockIdx.y = chain).
+__global__ void k_chain_load(BDev d, const chap::ChainSearch *chains)
+{
+    const int c = blockIdx.y;
+    const BCtl &b = d.ctl[c];
+    const chap::Dev &D = chains[c].d;
+    const long long xoff = d.ch_xoff[c];
+    const BRow *rs = d.rs + d.ch_roff[c];
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (tid == 0) {
+        chap::Ctl &k = *D.ctl;
+        k.iter = b.iter;
+        k.nviol = b.nviol;
+        k.best_nviol = b.best_nviol;
+        k.feasible_iter = b.feasible_iter;
+        k.max_iter = b.max_iter;
+        k.moves = b.moves;
+        k.bumps = b.bumps;
+        k.t_start_ns = b.t_start_ns;
+        k.t_feas_ns = b.t_feas_ns;
+        k.stop_at_feasible = b.stop_at_feasible;
+        k.done = b.done;
+    }
+    for (int q = tid; q < D.n; q += stride) {
+        const int j = D.var_list[q];
+        const bool one = x_bit<false>(d, xoff, j);
+        D.x[j] = one ? 1.0 : 0.0;
+        D.bup[q] = one ? 0 : 1;
+    }
+    for (int i = tid; i < D.m; i += stride) {
+        const BRow r = rs[i];
+        D.rs[i] = chap::RowState{r.r, r.w1, r.w2, 0.0, 0.0};
+    }
+}
+
+// And back.
+__global__ void k_chain_store(BDev d, const chap::ChainSearch *chains)
+{
+    const int c = blockIdx.y;
+    BCtl &b = d.ctl[c];
+    const chap::Dev &D = chains[c].d;
+    const long long xoff = d.ch_xoff[c];
+    BRow *rs = d.rs + d.ch_roff[c];
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (tid == 0) {
+        const chap::Ctl &k = *D.ctl;
+        b.iter = k.iter;
+        b.nviol = k.nviol;
+        b.best_nviol = k.best_nviol;
+        b.feasible_iter = k.feasible_iter;
+        b.moves = k.moves;
+        b.bumps = k.bumps;
+        b.t_feas_ns = k.t_feas_ns;
+        b.best_key = 0ull;
+        b.bump = 0;
+        if (k.done && !b.done) atomicAdd(d.n_done, 1u);
+        b.done = k.done;
+    }
+    // a warp per 32 variables: its ballot is a word of the bitset
+    const int n32 = (D.n + 31) & ~31;
+    for (int j = tid; j < n32; j += stride) {
+        const unsigned w = __ballot_sync(FULLMASK, j < D.n && D.x[j < D.n ? j : 0] != 0.0);
+        if ((threadIdx.x & 31) == 0) d.x[xoff + (j >> 5)] = w;
+    }
+    for (int i = tid; i < D.m; i += stride) {
+        const int4 v = *reinterpret_cast<const int4 *>(D.rs + i);
+        *reinterpret_cast<int4 *>(rs + i) = v;
+    }
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------ host
 
 struct chap_batch {
+    // chains as searches of their own (null chains: the batch does not qualify)
+    chap::ChainSearch *chains = nullptr;
+    int chain_smem = 0, max_n = 0;
+    int resident = 0;                         // this schedule is chosen
     cudaStream_t st = nullptr;
     int n_probs = 0, n_chains = 0;
     std::vector<void *> allocs;
@@ -416,7 +529,8 @@ struct chap_batch {
     std::vector<int> ch_inst, ch_tenure;
     std::vector<int> inst_n, inst_m;
     std::vector<long long> ch_xoff, ch_roff, ch_voff;   // bitset words / rows / variables
-    std::vector<BRow> rs0;                 // initial row states of every chain (x = 0, unit weights)
+    BRow *rows0 = nullptr;                 // device: initial row states of every instance (x = 0, unit weights)
+    long long *inst_row0 = nullptr;        // device: first of them per instance
     std::vector<BCtl> ctl0;
     std::vector<std::vector<double>> obj;
     long long total_x = 0, total_rows = 0, total_words = 0;
@@ -571,6 +685,140 @@ cudaError_t launch_iterations(const chap_batch *b, int G, int ctas, int persiste
     return e;
 }
 
+// The batch's chains as searches of their own: columns of at most kSrMaxRows
+// entries and few entries changed by a move, as for one CTA of the single
+// search.  An extra: a batch whose device memory does not hold it, or whose
+// instances do not qualify, keeps the other schedules.
+void make_chains(chap_batch *b, const chap_problem *probs, const std::vector<int> &inst_col0,
+                 const std::vector<int> &pos_of, const int *cptr_d, const int *ceq_d, const int *crow_d,
+                 const int *cval_d, const int *vo_d, const int *po_d)
+{
+    using namespace chap;
+    if (b->max_col > kSrMaxRows) return;
+    const int np = b->n_probs, nc = b->n_chains;
+    // rows of all instances one after another; their entries are filled in from
+    // the column store on the device
+    std::vector<SrRow> rows;
+    std::vector<int> row0(np);
+    long long nnz = 0;
+    int max_m = 0;
+    b->max_n = 0;
+    for (int k = 0; k < np; ++k) {
+        const chap_problem *p = probs + k;
+        row0[k] = (int)rows.size();
+        max_m = std::max(max_m, (int)p->m);
+        b->max_n = std::max(b->max_n, (int)p->n);
+        double touched = 0.0;
+        for (int i = 0; i < p->m; ++i) {
+            const double len = (double)(p->row_ptr[i + 1] - p->row_ptr[i]);
+            touched += len * len;
+            rows.push_back(SrRow{nnz, 0, 0, 0.0f, 0.0f, 0, 0});
+            nnz += p->row_ptr[i + 1] - p->row_ptr[i];
+        }
+        if (touched / std::max(1, (int)p->n) > kSrOneCtaTouched) return;
+    }
+    const size_t kept = b->allocs.size();
+    std::vector<ChainSearch> ch(nc);
+    long long nr = 0, nv = 0, nb = 0, nvb = 0;
+    for (int c = 0; c < nc; ++c) {
+        const int k = b->ch_inst[c];
+        nr += b->inst_m[k];
+        nv += b->inst_n[k];
+        nb += (b->inst_n[k] + kSrBlkPos - 1) / kSrBlkPos;
+        nvb += (b->inst_m[k] + kSrBlkPos - 1) / kSrBlkPos;
+    }
+    SrRow *rows_d = balloc<SrRow>(b, rows.size());
+    int *epos_d = balloc<int>(b, nnz);
+    long long *eval_d = balloc<long long>(b, nnz);
+    int2 *head_d = balloc<int2>(b, pos_of.size() * (size_t)kSrHead);
+    int *zero_d = balloc<int>(b, b->max_n + 1);
+    unsigned char *ones_d = balloc<unsigned char>(b, max_m);
+    RowState *rs_d = balloc<RowState>(b, nr);
+    double *x_d = balloc<double>(b, nv);
+    unsigned char *up_d = balloc<unsigned char>(b, nv);
+    long long *ks_d = balloc<long long>(b, nv);
+    int *kd_d = balloc<int>(b, nv);
+    long long *bs_d = balloc<long long>(b, nb);
+    int2 *bv_d = balloc<int2>(b, nb);
+    int *bd_d = balloc<int>(b, nb), *vc_d = balloc<int>(b, nvb);
+    SrCtl *sc_d = balloc<SrCtl>(b, nc);
+    Ctl *ctl_d = balloc<Ctl>(b, nc);
+    ChainSearch *ch_d = balloc<ChainSearch>(b, nc);
+    bool ok = rows_d && epos_d && eval_d && head_d && zero_d && ones_d && rs_d && x_d && up_d && ks_d && kd_d && bs_d &&
+              bv_d && bd_d && vc_d && sc_d && ctl_d && ch_d;
+    nr = nv = nb = nvb = 0;
+    for (int c = 0; c < nc && ok; ++c) {
+        const int k = b->ch_inst[c], n = b->inst_n[k], m = b->inst_m[k], c0 = inst_col0[k];
+        Dev d{};
+        d.n = n;
+        d.m = m;
+        d.tenure = b->ch_tenure[c];
+        d.ci_ptr = cptr_d + c0; d.ci_row = crow_d; d.ci_val = cval_d; d.ci_eq = ceq_d + c0;
+        d.cf_ptr = zero_d; d.cf_eq = zero_d;
+        d.row_int = ones_d;
+        d.x = x_d + nv; d.rs = rs_d + nr; d.bup = up_d + nv; d.n_bup = n;
+        d.tabu_inc = b->dev.tinc + b->ch_voff[c]; d.tabu_dec = b->dev.tdec + b->ch_voff[c];
+        d.ctl = ctl_d + c;
+        d.var_list = vo_d + c0; d.vpos = po_d + c0;
+        Search S{};
+        S.on = 1;
+        S.bc = n;
+        S.nblk = (n + kSrBlkPos - 1) / kSrBlkPos;
+        S.nvb = (m + kSrBlkPos - 1) / kSrBlkPos;
+        S.kS = ks_d + nv; S.kD = kd_d + nv;
+        S.bS = bs_d + nb; S.bV = bv_d + nb; S.bdirty = bd_d + nb;
+        S.vcnt = vc_d + nvb;
+        S.rowinfo = rows_d + row0[k]; S.epos = epos_d; S.eval = eval_d;
+        S.head = head_d + (size_t)c0 * kSrHead;
+        S.sc = sc_d + c;
+        ok = chain_shape(S);
+        b->chain_smem = std::max(b->chain_smem, S.smem);
+        ch[c] = ChainSearch{d, S};
+        nr += m;
+        nv += n;
+        nb += S.nblk;
+        nvb += S.nvb;
+    }
+    cudaError_t e = cudaSuccess;
+#define CUP(dst, v) if (ok && e == cudaSuccess && !(v).empty()) e = cudaMemcpyAsync(dst, (v).data(), sizeof((v)[0]) * (v).size(), cudaMemcpyHostToDevice, b->st)
+    CUP(rows_d, rows); CUP(ch_d, ch);
+#undef CUP
+    if (ok && e == cudaSuccess) e = cudaMemsetAsync(zero_d, 0, sizeof(int) * (size_t)(b->max_n + 1), b->st);
+    if (ok && e == cudaSuccess && max_m > 0) e = cudaMemsetAsync(ones_d, 1, max_m, b->st);
+    for (int k = 0; k < np && ok && e == cudaSuccess; ++k) {
+        const int n = b->inst_n[k], c0 = inst_col0[k];
+        k_chain_entries<<<(n + 255) / 256, 256, 0, b->st>>>(n, cptr_d + c0, crow_d, cval_d, rows_d + row0[k], epos_d, eval_d,
+                                                            head_d + (size_t)c0 * kSrHead);
+        e = cudaGetLastError();
+    }
+    if (ok && e == cudaSuccess) e = cudaStreamSynchronize(b->st);
+    if (ok && e == cudaSuccess) {
+        b->chains = ch_d;
+        b->resident = 1;
+        return;
+    }
+    cudaGetLastError();
+    while (b->allocs.size() > kept) {
+        cudaFree(b->allocs.back());
+        b->allocs.pop_back();
+    }
+    b->chain_smem = 0;
+}
+
+cudaError_t launch_chains_load(const chap_batch *b)
+{
+    k_chain_load<<<dim3(8, b->n_chains), 256, 0, b->st>>>(b->dev, b->chains);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = chap::launch_chain_keep(b->chains, b->n_chains, b->max_n, b->st);
+    return e;
+}
+
+cudaError_t launch_chains_store(const chap_batch *b)
+{
+    k_chain_store<<<dim3(8, b->n_chains), 256, 0, b->st>>>(b->dev, b->chains);
+    return cudaGetLastError();
+}
+
 chap_status upload_state(chap_batch *b)
 {
     BCK(b, cudaMemsetAsync(b->dev.n_done, 0, sizeof(unsigned int), b->st), "reset done count");
@@ -579,8 +827,8 @@ chap_status upload_state(chap_batch *b)
     BCK(b, cudaMemsetAsync(b->dev.bar, 0, sizeof(GridBar), b->st), "reset barrier");
     BCK(b, cudaMemsetAsync(b->dev.tinc, 0, sizeof(int) * std::max<long long>(b->total_x, 1), b->st), "reset tabu");
     BCK(b, cudaMemsetAsync(b->dev.tdec, 0, sizeof(int) * std::max<long long>(b->total_x, 1), b->st), "reset tabu");
-    BCK(b, cudaMemcpyAsync(b->dev.rs, b->rs0.data(), sizeof(BRow) * b->rs0.size(), cudaMemcpyHostToDevice, b->st),
-        "upload row states");
+    k_batch_reset_rows<<<dim3(8, b->n_chains), 256, 0, b->st>>>(b->dev, b->rows0, b->inst_row0);
+    BCK(b, cudaGetLastError(), "reset row states");
     BCK(b, cudaMemcpyAsync(b->dev.ctl, b->ctl0.data(), sizeof(BCtl) * b->ctl0.size(), cudaMemcpyHostToDevice, b->st),
         "upload control");
     BCK(b, cudaStreamSynchronize(b->st), "synchronise");
@@ -689,7 +937,6 @@ chap_status chap_batch_create(const chap_problem *probs, int32_t n_probs, const 
         wo += (b->inst_n[k] + 31) / 32;
         ro += b->inst_m[k];
         item0.push_back(item0.back() + (b->inst_n[k] + kTile - 1) / kTile);
-        b->rs0.insert(b->rs0.end(), rows0[k].begin(), rows0[k].end());
         long long nv = 0;
         for (const BRow &r : rows0[k]) nv += (r.r > 0) + (r.w2 >= 0 && r.r < 0);
         BCtl cz{};
@@ -706,6 +953,14 @@ chap_status chap_batch_create(const chap_problem *probs, int32_t n_probs, const 
     d.n_chains = n_chains;
     d.total_items = item0.back();
     d.total_rows = ro;
+    std::vector<BRow> rows_all;
+    std::vector<long long> row_first;
+    for (int k = 0; k < n_probs; ++k) {
+        row_first.push_back((long long)rows_all.size());
+        rows_all.insert(rows_all.end(), rows0[k].begin(), rows0[k].end());
+    }
+    b->rows0 = balloc<BRow>(b, rows_all.size());
+    b->inst_row0 = balloc<long long>(b, n_probs);
     int *in_d = balloc<int>(b, n_probs), *im_d = balloc<int>(b, n_probs), *ic_d = balloc<int>(b, n_probs);
     int *cptr_d = balloc<int>(b, cptr.size()), *ceq_d = balloc<int>(b, ceq.size());
     int *crow_d = balloc<int>(b, crow.size()), *cval_d = balloc<int>(b, cval.size());
@@ -721,7 +976,7 @@ chap_status chap_batch_create(const chap_problem *probs, int32_t n_probs, const 
     d.rs = balloc<BRow>(b, ro);
     d.ctl = balloc<BCtl>(b, n_chains);
     d.n_done = balloc<unsigned int>(b, 1);
-    const bool ok = in_d && im_d && ic_d && cptr_d && ceq_d && crow_d && cval_d && vo_d && po_d && chi_d && cht_d &&
+    const bool ok = b->rows0 && b->inst_row0 && in_d && im_d && ic_d && cptr_d && ceq_d && crow_d && cval_d && vo_d && po_d && chi_d && cht_d &&
                     chx_d && chr_d && chv_d && chi0_d && d.x && d.bar && d.tinc && d.tdec && d.rs && d.ctl &&
                     d.n_done &&
                     cudaMallocHost(&b->h_done, 2 * sizeof(unsigned int)) == cudaSuccess;
@@ -736,7 +991,7 @@ chap_status chap_batch_create(const chap_problem *probs, int32_t n_probs, const 
     BUP(in_d, b->inst_n); BUP(im_d, b->inst_m); BUP(ic_d, inst_col0);
     BUP(cptr_d, cptr); BUP(ceq_d, ceq); BUP(crow_d, crow); BUP(cval_d, cval); BUP(vo_d, var_of); BUP(po_d, pos_of);
     BUP(chi_d, b->ch_inst); BUP(cht_d, b->ch_tenure); BUP(chx_d, b->ch_xoff); BUP(chr_d, b->ch_roff); BUP(chi0_d, item0);
-    BUP(chv_d, b->ch_voff);
+    BUP(chv_d, b->ch_voff); BUP(b->rows0, rows_all); BUP(b->inst_row0, row_first);
 #undef BUP
     if (e == cudaSuccess) e = cudaMemsetAsync(d.n_done, 0, sizeof(unsigned int), b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
@@ -778,6 +1033,7 @@ chap_status chap_batch_create(const chap_problem *probs, int32_t n_probs, const 
         delete b;
         return s;
     }
+    make_chains(b, probs, inst_col0, pos_of, cptr_d, ceq_d, crow_d, cval_d, vo_d, po_d);
     *out = b;
     return CHAP_OK;
 }
@@ -813,6 +1069,15 @@ chap_status chap_batch_run(chap_batch *b, int64_t max_iters, int32_t stop_at_fea
     BCK(b, cudaMemsetAsync(b->dev.n_done, 0, sizeof(unsigned int), b->st), "reset done count");
     k_batch_begin<<<(b->n_chains + 255) / 256, 256, 0, b->st>>>(b->dev, max_iters, stop_at_feasible);
     BCK(b, cudaGetLastError(), "begin run");
+    if (b->resident) {
+        // every chain runs to its end on its own: launches of kChainIters
+        // iterations until all are done
+        BCK(b, launch_chains_load(b), "load chains");
+        for (long long left = max_iters; left > 0; left -= kChainIters)
+            BCK(b, chap::launch_chain_search(b->chains, b->n_chains, b->chain_smem, kChainIters, b->st), "chain search");
+        BCK(b, launch_chains_store(b), "store chains");
+        BCK(b, cudaStreamSynchronize(b->st), "synchronise");
+    } else {
     if (!b->gexec || b->g_iters != graph_iters || b->g_G != b->G || b->g_ctas != b->ctas_per_sm ||
         b->g_persistent != b->persistent) {
         if (b->gexec) cudaGraphExecDestroy(b->gexec);
@@ -846,6 +1111,7 @@ chap_status chap_batch_run(chap_batch *b, int64_t max_iters, int32_t stop_at_fea
             return bfail(b, CHAP_E_TIMEOUT, "a grid-barrier wait of the persistent launch ran out");
         }
         if (*b->h_done >= (unsigned)b->n_chains) break;
+    }
     }
     const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (seconds) *seconds = secs;
@@ -903,11 +1169,34 @@ chap_status chap_batch_autotune_mode(chap_batch *b, int32_t iters, int32_t mode,
             }
             if (ms < best_ms) { best_ms = ms; bg = Gs[gi]; bc = Cs[ci]; bp = pm; }
         }
+    bool res = false;
+    if (mode < 0 && b->chains) {
+        // the chains as searches of their own, after the same warm-up (their
+        // kept values are evaluated once per run, not timed here)
+        chap_status s = upload_state(b);
+        if (s != CHAP_OK) { cudaEventDestroy(a); cudaEventDestroy(z); return s; }
+        k_batch_begin<<<(b->n_chains + 255) / 256, 256, 0, b->st>>>(b->dev, iters + 1, 0);
+        cudaError_t e = launch_chains_load(b);
+        if (e == cudaSuccess) e = chap::launch_chain_search(b->chains, b->n_chains, b->chain_smem, 1, b->st);
+        if (e == cudaSuccess) e = cudaEventRecord(a, b->st);
+        if (e == cudaSuccess) e = chap::launch_chain_search(b->chains, b->n_chains, b->chain_smem, iters, b->st);
+        if (e == cudaSuccess) e = cudaEventRecord(z, b->st);
+        if (e == cudaSuccess) e = cudaEventSynchronize(z);
+        float ms = 0.0f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, z);
+        if (e != cudaSuccess) {
+            cudaEventDestroy(a);
+            cudaEventDestroy(z);
+            BCK(b, e, "autotune run");
+        }
+        res = ms < best_ms;
+    }
     cudaEventDestroy(a);
     cudaEventDestroy(z);
     b->G = bg;
     b->ctas_per_sm = bc;
     b->persistent = bp;
+    b->resident = res ? 1 : 0;
     if (chosen) { chosen[0] = bg; chosen[1] = bc; chosen[2] = bp; }
     return upload_state(b);
 }
@@ -925,6 +1214,7 @@ chap_status chap_batch_set_schedule(chap_batch *b, int32_t lanes_per_column, int
         return CHAP_E_INVALID;
     b->G = lanes_per_column;
     b->ctas_per_sm = ctas_per_sm;
+    b->resident = 0;
     return CHAP_OK;
 }
 
@@ -945,6 +1235,7 @@ chap_status chap_batch_set_persistent(chap_batch *b, int32_t on, int64_t barrier
 {
     if (!b || (on != 0 && on != 1) || barrier_limit_ns < 0) return CHAP_E_INVALID;
     b->persistent = on;
+    b->resident = 0;
     if (barrier_limit_ns > 0) b->bar_limit_ns = (unsigned long long)barrier_limit_ns;
     if (b->gexec) { cudaGraphExecDestroy(b->gexec); b->gexec = nullptr; }
     return CHAP_OK;

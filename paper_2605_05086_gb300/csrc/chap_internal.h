@@ -368,6 +368,8 @@ struct Search {
     int nvb;                 // blocks of physical rows with a violation count
     int flip_words;          // words of the flip bits in k_search's shared memory (0: d.bup is read)
     int smem;                // dynamic shared memory of k_search
+    int big_chunks;          // walk chunks, and violated rows of a weight update, above which
+    long long big_viol;      // the whole GPU applies an iteration
     // non-binary columns: place p = position - bc, short ones [0, nnb), then
     // nhist counting-sorted ones
     int mix, nnb, nhist, nnblk;
@@ -394,6 +396,13 @@ struct Search {
     long long *eval;
     int2 *head;              // first kSrHead integral entries (row, coefficient) of every binary position
     SrCtl *sc;
+};
+
+// One chain of a batch as a search of its own (all-binary integral instance):
+// the instance's matrix arrays are shared, the state is the chain's.
+struct ChainSearch {
+    Dev d;
+    Search S;
 };
 
 // Optional per-variable outputs of a best-shift pass (device pointers, may be null).
@@ -475,6 +484,12 @@ cudaError_t launch_apply_records(const Dev &d, const chap_move_record *recs, int
 cudaError_t launch_keep_entries(const Dev &d, const Search &S, cudaStream_t st);
 cudaError_t launch_keep_build(const Dev &d, const LaunchPlan &p, const Search &S, cudaStream_t st);
 cudaError_t launch_search(const Dev &d, const Search &S, int max_launch, cudaStream_t st);
+// Chains of a batch, one CTA each: shape of chain S (false: too large for a
+// CTA), kept values, up to max_launch iterations.  max_n: most variables of a
+// chain; smem: most shared memory.
+bool chain_shape(Search &S);
+cudaError_t launch_chain_keep(const ChainSearch *chains, int n, int max_n, cudaStream_t st);
+cudaError_t launch_chain_search(const ChainSearch *chains, int n, int smem, int max_launch, cudaStream_t st);
 // Chooses S.nct (one CTA, or the largest cluster that fits the current device)
 // and the shared memory of k_search; false when no shape fits.
 bool search_shape(Search &S, bool one_cta);
@@ -509,6 +524,8 @@ constexpr double kBlkMinSeg = 2.0;      // and from this many entries per (block
 constexpr double kSrOneCtaTouched = 4096.0;
 constexpr int kSrHead = 8;              // integral column entries addressed by position
 constexpr int kSrLaunchIters = 2048;    // iterations of one launch of the search
+constexpr int kSrBlkPos = 256;          // positions (and physical rows) of one summary block
+constexpr int kSrMaxRows = 512;         // column entries (and threads) of one CTA's records
 constexpr int kApplyThreads = 256;
 constexpr int kApplyMoveThreads = 1024;
 constexpr int kLazyMaxRows = 2048;      // longer moved columns re-evaluate every kept binary score

@@ -3222,7 +3222,7 @@ cudaError_t static_hist_scratch(HBin **bins, HistAcc **acc)
 // largest size any handle launches with), under a mutex.
 static cudaError_t raise_smem_limit(const void *fn, int slot, int bytes)
 {
-    constexpr int kMaxDevices = 64, kSlots = 11;
+    constexpr int kMaxDevices = 64, kSlots = 12;
     static std::mutex s_mu;
     static int s_set[kMaxDevices][kSlots] = {};
     int dev = 0;
@@ -3535,6 +3535,8 @@ bool search_shape(Search &S, bool one_cta)
     for (S.nct = one_cta && S.nblk <= kSrMaxTops ? 1 : kSrMaxCluster; S.nct >= 1; S.nct >>= 1) {
         SrLocal L;
         S.smem = sr_layout(S, S.nct, nullptr, L);
+        S.big_chunks = kSrBigWalk * kSrWarps * S.nct;
+        S.big_viol = 4LL * kSrRows * S.nct;
         if (L.nl > kSrMaxTops || L.nnl > 0xffff / kSrBlk) return false;   // 16-bit places inside a CTA
         if (raise_smem_limit(fn, S.mix ? 10 : 8, S.smem) == cudaSuccess) {
             cudaLaunchConfig_t cfg;
@@ -3549,6 +3551,32 @@ bool search_shape(Search &S, bool one_cta)
         cudaGetLastError();
     }
     return false;
+}
+
+bool chain_shape(Search &S)
+{
+    const int words = (S.bc + 31) / 32;
+    S.flip_words = words <= kSrFlipWords ? words : 0;
+    S.nct = 1;
+    SrLocal L;
+    S.smem = sr_layout(S, 1, nullptr, L);
+    S.big_chunks = INT_MAX;
+    S.big_viol = LLONG_MAX;
+    return L.nl <= kSrMaxTops && raise_smem_limit((const void *)k_search_chains, 11, S.smem) == cudaSuccess;
+}
+
+cudaError_t launch_chain_keep(const ChainSearch *chains, int n, int max_n, cudaStream_t st)
+{
+    // 4 lanes a column, a few CTAs per chain
+    const int gx = std::max(1, std::min(16, (max_n + 2047) / 2048));
+    k_keep_chains<4><<<dim3(gx, n), kEvalThreads, 0, st>>>(chains);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_chain_search(const ChainSearch *chains, int n, int smem, int max_launch, cudaStream_t st)
+{
+    k_search_chains<<<n, kSrThreads, smem, st>>>(chains, max_launch);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_search(const Dev &d, const Search &S, int max_launch, cudaStream_t st)

@@ -169,3 +169,32 @@ def test_checkpointed_tabu_and_aspiration(chap, mixed):
             _same_state(sa, sb)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("stop", [False, True])
+def test_chains_default_schedule(chap, stop):
+    """A batch on its default schedule (each chain a search of its own where the
+    instances allow it) follows the single handle over split runs and a reset;
+    one instance of long columns keeps the whole batch on the other schedules."""
+    probs = [inst.gen_setcover(seed=5, n=257, m=256, k=6), binary_rows(21, 900, 513, 7),
+             inst.gen_setcover(seed=6, n=3000, m=1500, k=8)]
+    for extra in ([], [binary_rows(22, 40, 700, 30)]):
+        ps = probs + extra
+        chain_prob = [k for k in range(len(ps)) for _ in range(2)]
+        tenures = [0, 12] * len(ps)
+        b = chap.BatchChains(ps, chain_prob, tenures)
+        for again in range(2):
+            if again:
+                b.reset()
+            for iters in (1, 60, 150):
+                res, _ = b.run(max_iters=iters, stop_at_feasible=stop)
+            for c, (k, t) in enumerate(zip(chain_prob, tenures)):
+                bs = chap.BestShift(ps[k], tenure=t)
+                for iters in (1, 60, 150):
+                    bs.run(max_iters=iters, stop_at_feasible=1 if stop else 0)
+                st = bs.state()
+                bs.close()
+                assert (res[c].iters, res[c].moves, res[c].final_nviol, res[c].best_nviol) == \
+                    (st["iter"], st["moves"], st["nviol"], st["best_nviol"]), c
+                assert np.array_equal(b.x(c), st["x"]), c
+        b.close()
