@@ -163,7 +163,7 @@ typedef struct chap_info {
     int64_t bytes_cta;        /* ... of the CTA-sort kernel (long non-integer columns) */
     int64_t bytes_hist;       /* ... of the counting-sort kernel (long integer columns) */
     int32_t bin_lanes;        /* lanes that score one binary column (2, 4, 8 or 16) */
-    int32_t nb_lanes;         /* lanes that score one short non-binary column (4 or 8) */
+    int32_t nb_lanes;         /* lanes that score one short non-binary column (4, 8, 16 or 32) */
     int32_t n_long_cols;      /* columns on the multi-CTA merge-sort path (lists over 8192 entries) */
     int32_t n_cta_cols;       /* columns on the one-CTA shared-memory sort path (129..8192 entries) */
     int32_t bin_rows;         /* 1: binary flips scored row-wise (clusters over column blocks) */

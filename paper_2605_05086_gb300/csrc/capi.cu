@@ -612,7 +612,11 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     }
     // long lists: runs of kLongRun sorted entries per chunk of kLongChunk
     // nonzeros, padded to a power of two runs per column
+    // (columns of at most kRkMaxRuns runs of kRkChunk nonzeros are ranked)
     std::vector<LongCol> lcols;
+    std::vector<RankCol> rcols;
+    std::vector<Tile> tiles_rgen;
+    int rank_runs = 0;
     std::vector<Tile> tiles_lgen, tiles_lscan;
     long long long_entries = 0;
     int long_rounds = 0, long_tiles = 0;
@@ -621,6 +625,20 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         lc.pos = q;
         lc.e_mid = ci_ptr[q + 1] - ci_ptr[q];
         lc.e_end = lc.e_mid + (cf_ptr[q + 1] - cf_ptr[q]);
+        const int rk = (lc.e_end + kRkChunk - 1) / kRkChunk;
+        if (rk <= kRkMaxRuns) {
+            RankCol rc{};
+            rc.pos = q;
+            rc.len = lc.e_end;
+            rc.runs = rk;
+            rc.run0 = rank_runs;
+            rc.base = (long long)rank_runs * kRkRun;
+            rank_runs += rk;
+            const int ri = (int)rcols.size();
+            for (int r = 0; r < rk; ++r) tiles_rgen.push_back(Tile{T_NB_LONG, ri, ri + 1, r});
+            rcols.push_back(rc);
+            continue;
+        }
         lc.nchunks = std::max(1, (lc.e_end + kLongChunk - 1) / kLongChunk);
         int runs = 1, rounds = 0;
         while (runs < lc.nchunks) { runs <<= 1; ++rounds; }
@@ -642,7 +660,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     if (nb_cols > 0) {
         const double mean = (double)((ci_ptr[kind_base[T_NB + 1]] - ci_ptr[kind_base[T_NB]]) +
                                      (cf_ptr[kind_base[T_NB + 1]] - cf_ptr[kind_base[T_NB]])) / nb_cols;
-        nb_G = mean <= kNbG4MaxLen ? 4 : 8;
+        nb_G = nb_lanes(nb_cols, mean <= kNbG4MaxLen ? 4 : 8);
     }
     const int n_tn = nb_cols > 0 ? nb_grid_size(nb_cols, nb_G) : 0;
     const int bin_cols = kind_base[T_BIN + 1] - kind_base[T_BIN];
@@ -860,7 +878,9 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     for (size_t q = 0; q < hcols.size(); ++q) hcols[q].slot = slot_hist + (int)q;
     const int slot_long = slot_hist + (int)hcols.size();
     for (size_t q = 0; q < lcols.size(); ++q) lcols[q].slot = slot_long + (int)q;
-    const int n_bb = slot_long + (int)lcols.size();
+    const int slot_rank = slot_long + (int)lcols.size();
+    for (size_t q = 0; q < rcols.size(); ++q) rcols[q].slot = slot_rank + (int)q;
+    const int n_bb = slot_rank + (int)rcols.size();
 
     // ---- device allocation
     Dev &d = h->dev;
@@ -953,6 +973,19 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     }
     const bool blk_ok = (d.bup || !(bin_blk || keep)) && (!bin_blk || ( bbd.items && bbd.metaI && bbd.metaF && bbd.valI && bbd.valF &&
                                      bbd.acc_s && bbd.acc_dc));
+    RankCol *rc_d = dalloc<RankCol>(h, rcols.size());
+    Tile *trg_d = dalloc<Tile>(h, tiles_rgen.size());
+    const size_t rank_entries = (size_t)rank_runs * kRkRun;
+    d.rkey = dalloc<unsigned long long>(h, rank_entries);
+    d.raux = dalloc<unsigned>(h, rank_entries);
+    d.rsum = dalloc<long long>(h, rank_entries);
+    d.rsumc = dalloc<int>(h, rank_entries);
+    d.rcnt = dalloc<int>(h, rank_runs);
+    d.rccnt = dalloc<int>(h, rank_runs);
+    d.rcand_at = dalloc<unsigned short>(h, rank_entries);
+    d.racc = dalloc<HistAcc>(h, rcols.size());
+    d.rcand = dalloc<LCand>(h, rank_runs);
+    const bool rank_ok = rc_d && trg_d && d.rkey && d.raux && d.rsum && d.rsumc && d.rcnt && d.rccnt && d.rcand_at && d.racc && d.rcand;
     LongCol *lc_d = dalloc<LongCol>(h, lcols.size());
     Tile *tlg_d = dalloc<Tile>(h, tiles_lgen.size()), *tls_d = dalloc<Tile>(h, tiles_lscan.size());
     d.n_long = (int)lcols.size();
@@ -972,11 +1005,15 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
               (!has_long || (d.lbuf0 && d.lbuf1 && d.lacc && d.ltsum && d.ltsumc && d.lcand)) &&
               (!bin_rows || (rbr_d[0] && rbr_d[1] && rbe_d[0] && rbe_d[1] && rbs_d[0] && rbs_d[1] && rbc_d[0] &&
                              rbc_d[1] && rbo_d[0] && rbo_d[1] && rbvi_d && rbvf_d));
-    ok = ok && blk_ok;
+    ok = ok && blk_ok && rank_ok;
     if (ok && cudaMallocHost(&h->h_ctl, sizeof(Ctl)) != cudaSuccess) { cudaGetLastError(); h->h_ctl = nullptr; ok = false; }
     if (ok && cudaStreamCreateWithFlags(&h->cap_st, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); ok = false; }
+    // the long and counting-sorted columns' kernels are the pass's longest
+    // chains where an instance has them: their CTAs go first
+    int prio_low = 0, prio = 0;
+    if (cudaDeviceGetStreamPriorityRange(&prio_low, &prio) != cudaSuccess) { cudaGetLastError(); prio = 0; }
     for (int k = 0; k < 3 && ok; ++k)
-        if (cudaStreamCreateWithFlags(&h->plan.side[k], cudaStreamNonBlocking) != cudaSuccess ||
+        if (cudaStreamCreateWithPriority(&h->plan.side[k], cudaStreamNonBlocking, k == 0 ? 0 : prio) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->plan.ev_join[k], cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); ok = false; }
     if (ok && cudaEventCreateWithFlags(&h->plan.ev_fork, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); ok = false; }
     for (int k = 0; k < 10 && ok; ++k)
@@ -997,6 +1034,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     d.vpos = vpos_d;
     d.hcols = hc_d;
     d.lcols = lc_d;
+    d.rcols = rc_d;
     cudaStream_t st = h->st;
     std::vector<long long> rp(p->row_ptr, p->row_ptr + m + 1);
     cudaError_t e = cudaSuccess;
@@ -1010,6 +1048,8 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     UP(vl_d, var_list.data(), var_list.size()); UP(vpos_d, vpos.data(), n);
     UP(tc_d, tiles_cta.data(), tiles_cta.size());
     UP(th_d, tiles_hist.data(), tiles_hist.size()); UP(hc_d, hcols.data(), hcols.size());
+    UP(rc_d, rcols.data(), rcols.size());
+    UP(trg_d, tiles_rgen.data(), tiles_rgen.size());
     UP(lc_d, lcols.data(), lcols.size());
     for (int t = 0; t < 2 && bin_rows; ++t) {
         UP(rbr_d[t], rb_rows[t].data(), rb_rows[t].size()); UP(rbe_d[t], rb_eptr[t].data(), rb_eptr[t].size());
@@ -1028,6 +1068,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         if (e == cudaSuccess) e = cudaMemsetAsync(bbd.acc_dc, 0, sizeof(int) * (size_t)bin_cols, st);
     }
 #undef UP
+    if (e == cudaSuccess && !rcols.empty()) e = cudaMemsetAsync(d.racc, 0, sizeof(HistAcc) * rcols.size(), st);
     if (e == cudaSuccess && has_long) e = cudaMemsetAsync(d.lacc, 0, sizeof(HistAcc) * lcols.size(), st);
     if (e == cudaSuccess && hist_bins > 0 && !h->no_hist_scratch)
         e = cudaMemsetAsync(d.hbins, 0, sizeof(HBin) * hist_bins, st);
@@ -1049,6 +1090,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     pl.tiles_cta = tc_d; pl.n_cta = n_tc; pl.cta_smem = max_cta_n * 20;
     pl.tiles_hist = th_d; pl.n_hist_tiles = (int)tiles_hist.size(); pl.hist_smem = max_hist_d * (int)sizeof(HBin);
     pl.slot_nb = n_tb; pl.slot_cta = n_tb + n_tn;
+    pl.tiles_rgen = trg_d; pl.n_rgen = (int)tiles_rgen.size();
     pl.tiles_lgen = tlg_d; pl.n_lgen = (int)tiles_lgen.size();
     pl.tiles_lscan = tls_d; pl.n_lscan = (int)tiles_lscan.size();
     pl.long_rounds = long_rounds; pl.long_entries = long_entries;
@@ -1077,15 +1119,16 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     in.n = n; in.m = m; in.m_norm = mn;
     in.n_bin = n_bin; in.n_int = n_int; in.n_cont = n_cont; in.n_fixed = n_fixed;
     in.nnz = p->nnz; in.nnz_int_rows = nnz_int; in.nnz_fp_rows = p->nnz - nnz_int;
-    in.eval_blocks = (bin_blk ? (int)blk_items.size() : n_tb) + n_tn + n_tc + (int)tiles_hist.size() + (int)tiles_lscan.size();
+    in.eval_blocks = (bin_blk ? (int)blk_items.size() : n_tb) + n_tn + n_tc + (int)tiles_hist.size() + (int)tiles_lscan.size() +
+                     (int)tiles_rgen.size();
     in.n_hist_cols = (int)hcols.size();
-    in.n_long_cols = (int)lcols.size();
+    in.n_long_cols = (int)(lcols.size() + rcols.size());
     in.n_cta_cols = n_tc;
     // evaluation kernels (they also select the move), a selection kernel only
     // when none runs, the move apply and the weight bump
     in.launches_per_step = (n_tb > 0) + (bin_blk ? 1 : 0) + (n_tn > 0) + (n_tc > 0) + (!tiles_hist.empty()) + (n_bb == 0) + 2 +
                            (lazy ? 2 : 0) +   // kept binary scores: the scan and the marking kernel
-                           (has_long ? 3 + long_rounds : 0);   // long lists: generation, merges, tile sums, scan
+                           (has_long ? 3 + long_rounds : 0) + (rcols.empty() ? 0 : 2);   // long lists: generation, merges, tile sums, scan
     // algorithmic bytes of one pass: every nonzero once (row + coefficient),
     // every row state and tolerance once, every active variable's state once.
     int64_t n_act = kind_base[T_NUM_KINDS];   // evaluated columns
@@ -1154,7 +1197,7 @@ chap_status chap_bs_kernel_ms(chap_bs *h, float *ms)
     if (h->broken) return fail(h, CHAP_E_STATE, "handle unusable after a CUDA fault");
     if (!h->prof_valid) return fail(h, CHAP_E_STATE, "no profiled pass since chap_bs_profile(h, 1)");
     CK(h, cudaStreamSynchronize(h->st), "synchronise");
-    const bool launched[5] = {h->plan.n_bin > 0, h->plan.nb_grid > 0, h->plan.n_cta > 0 || h->plan.n_lgen > 0,
+    const bool launched[5] = {h->plan.n_bin > 0, h->plan.nb_grid > 0, h->plan.n_cta > 0 || h->plan.n_lgen > 0 || h->plan.n_rgen > 0,
                               h->plan.n_hist_tiles > 0, true};
     for (int k = 0; k < 5; ++k) {
         ms[k] = 0.0f;

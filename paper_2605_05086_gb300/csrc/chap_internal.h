@@ -187,6 +187,17 @@ struct LongCol {
     long long base;       // first entry of the column in the entry buffers
 };
 
+// A long column whose list is ranked instead of merged (k_rank_gen,
+// k_rank_eval): at most kRkMaxRuns sorted runs of kRkChunk nonzeros each.
+struct RankCol {
+    int pos;              // position of the column in var_list
+    int len;              // nonzeros
+    int runs;
+    int run0;             // first run of the column in rcnt and rcand
+    int slot;             // block_best slot of the column
+    long long base;       // first entry of the column in the run buffers
+};
+
 // Row-wise binary flips (Sec. 3.1, "Memory Considerations", third point: the
 // binary columns scored row by row).  The binary positions are dealt round
 // robin into blocks of at most kRbCols columns (position q = c * blocks + b
@@ -300,6 +311,16 @@ struct Dev {
     LCand *lcand;            // per tile: best candidate
     const LongCol *lcols;
     int n_long;
+    // ranked long lists: per entry key, class word, prefix sums of its run; the
+    // places of the run's candidates; entries, candidates and best candidate per run, per-column accumulators, columns
+    unsigned long long *rkey;
+    unsigned *raux;
+    long long *rsum;
+    int *rsumc, *rcnt, *rccnt;
+    unsigned short *rcand_at;
+    HistAcc *racc;
+    LCand *rcand;
+    const RankCol *rcols;
     // rows of the residual computation (set-state only): the integral rows,
     // then the others by decreasing length
     int n_res_int;
@@ -425,6 +446,8 @@ struct LaunchPlan {
     const Tile *tiles_hist;
     int n_hist_tiles;
     int hist_smem;
+    const Tile *tiles_rgen;    // ranked long lists: (column, run)
+    int n_rgen;
     const Tile *tiles_lgen;    // long lists: (column, chunk) of the generation kernel
     int n_lgen;
     const Tile *tiles_lscan;   // (column, tile) of the scan kernels
@@ -459,6 +482,7 @@ cudaError_t static_hist_scratch(HBin **bins, HistAcc **acc);
 int bin_grid_size(int ncols, int G);  // persistent grids of the binary (G lanes per column) and
                                       // short-column kernels on the current device
 int nb_grid_size(int ncols, int G);
+int nb_lanes(int ncols, int G);       // lanes per short non-binary column, from G on
 cudaError_t launch_eval_gated(const Dev &d, const LaunchPlan &p, const VarOut &o, int gate, cudaStream_t st);
 cudaError_t launch_select_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st);
 cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st);
@@ -504,6 +528,10 @@ constexpr int kHistThreads = 512;
 constexpr int kRbCols = 8192;          // binary columns of one row-wise block
 constexpr int kRbCluster = 8;          // CTAs per block (one thread-block cluster)
 constexpr int kRbThreads = 1024;
+constexpr int kRkChunk = 508;          // nonzeros of a ranked run: <= 4 entries each, + 2 bounds
+constexpr int kRkRun = 2048;           // entries of a ranked run at most (power of two)
+constexpr int kRkThreads = 512;
+constexpr int kRkMaxRuns = 64;         // runs of a ranked column at most (longer columns are merged)
 constexpr int kLongChunk = 1020;       // nonzeros per generating CTA: <= 4 entries each, + 2 bounds
 constexpr int kLongRun = 4096;         // entries of one sorted run (power of two)
 constexpr int kLongThreads = 512;
@@ -514,7 +542,7 @@ constexpr int kBlkRows = 8192;          // rows of one row block of the row-bloc
 constexpr int kBlkRowBits = 13;        // bits of the row inside a block in an entry word (kBlkRows = 2^13)
 constexpr int kBlkMaxPos = 1 << (32 - kBlkRowBits);  // binary positions an entry word can name
 constexpr int kBlkThreads = 1024;
-constexpr int kBlkFin = 1024;           // binary positions of one finalize range (one CTA)
+constexpr int kBlkFin = 256;            // binary positions of one finalize range (one CTA, a position per thread)
 constexpr int kBlkFinThreads = 256;
 constexpr int kBlkMaxBlocks = 32;       // the library picks the row-blocked flips up to this many row blocks,
 constexpr int kBlkMinCols = 16384;      // from this many binary columns,
@@ -535,6 +563,7 @@ constexpr double kBinG2MaxLen = 6.0;    // mean binary column length up to which
 constexpr int kBinG2MinCols = 32768;    // (and only with this many binary columns: small instances are latency-bound)
 constexpr double kBinG4MaxLen = 16.0;   // ... up to which 4 lanes do
 constexpr double kBinG8MaxLen = 1.0e30; // ... up to which 8 lanes do (16 above)
+constexpr int kNbWideMin = 1024;        // short non-binary columns from which more than 8 lanes may score one
 constexpr double kNbG4MaxLen = 16.0;    // mean short non-binary column length up to which 4 lanes score a column (8 above)
 
 }  // namespace chap

@@ -14,8 +14,8 @@
 //    two entries of Algorithm 1 merged); entries left of l fold into beta,
 //    entries right of u are dropped.  Short columns (k_eval_nb, at most 128
 //    entries) place every half by products first and compute exact breakpoints
-//    only for the undecided ones, 32 at a time; their lists are sorted by
-//    group bitonic networks in registers.  Longer columns are bitonic-sorted in
+//    only for the undecided ones, 32 at a time; a candidate's score is summed
+//    over its column's list by counting, without a sort.  Longer columns are bitonic-sorted in
 //    shared memory by one CTA (k_eval_cta, up to 8192 entries) or
 //    counting-sorted across many CTAs (k_eval_hist, long integer columns).
 //  * Every CTA reduces its columns to one candidate; the CTA that writes the
@@ -1227,6 +1227,23 @@ __device__ __forceinline__ int int_fp_side(double m, double a, bool apos, const 
     return 0;
 }
 
+// floor(m / a) (a > 0) or ceil(m / a) (a < 0) of the rounded double quotient,
+// clamped: decided by a single-precision quotient when that lies farther from
+// every integer than its error (relative 2^-19), which is nearly always; the
+// double division runs otherwise (GB300's FP64 pipe is narrow: 2 lanes a cycle
+// and SM).
+__device__ __forceinline__ long long int_breakpoint(double m, double a, bool apos)
+{
+    bool ok = true;
+    const float mf = approx_f(m, ok), af = approx_f(a, ok);
+    const float q = __fdividef(mf, af);
+    const float fr = q - rintf(q);
+    if (ok && fabsf(af) < 8.0e37f && fabsf(q) < 65536.0f && fabsf(fr) > fabsf(q) * 2.0e-6f)
+        return (long long)(apos ? __float2int_rd(q) : __float2int_ru(q));
+    const double d = __ddiv_rn(m, a);
+    return clamp_dd(apos ? __double2ll_rd(d) : __double2ll_ru(d));
+}
+
 // Continuous variable: side of xbar - q / a (left of l <=> q/a > xbar - l,
 // right of u <=> q/a < xbar - u) for q = r (the tight point) or q = -m (the
 // boundary), decided from single-precision products with a margin that also
@@ -1300,8 +1317,7 @@ __device__ __forceinline__ void fp_half(double r, double a, double m, double mo,
             half_case(viol, false, apos, side, 0ull, w, c.kl, c.ku, acc, h);
             return;
         }
-        const double q = __ddiv_rn(m, a);
-        const long long dd = clamp_dd(apos ? __double2ll_rd(q) : __double2ll_ru(q));
+        const long long dd = int_breakpoint(m, a, apos);
         half_case(viol, !viol && dd == 0, apos, 0, ikey(c.xbi + dd), w, c.kl, c.ku, acc, h);
     } else {
         const bool near0 = !viol && !dneg(mo);  // |r| <= eps
@@ -1425,10 +1441,9 @@ __device__ __forceinline__ bool is_candidate(unsigned long long k, unsigned a, u
 //     at once (FP64 divisions are slow on this part, so they are never issued
 //     for a single lane), and the entries inside [l, u] are appended to the
 //     column's list in shared memory.
-//  3. Each group sorts its list (bitonic over G lanes, 1, 2 or 4 entries per
-//     lane), prefix-scans it with shuffles and reduces it to the column's best
-//     admissible candidate.  A column whose list outgrows 4 G entries is
-//     evaluated again by the whole warp with a list of kWarpSortMax entries.
+//  3. Each group takes the column's best admissible candidate from its list
+//     (group_count).  A column whose list outgrows 4 G entries is evaluated
+//     again by the whole warp with a list of kWarpListMax entries.
 
 constexpr int kNbWarps = kEvalWarps;
 constexpr int kQCap = 160;                  // queued halves per warp (more: the whole-warp path)
@@ -1517,8 +1532,7 @@ __device__ __forceinline__ void exact_item(const QItem &it, const ColCtx &ci, Ac
         const double a = __longlong_as_double(it.a);
         apos = !dneg(a);
         if (ci.isint) {
-            const double q = __ddiv_rn(__longlong_as_double(it.x), a);
-            const long long dd = clamp_dd(apos ? __double2ll_rd(q) : __double2ll_ru(q));
+            const long long dd = int_breakpoint(__longlong_as_double(it.x), a, apos);
             tight = !viol && dd == 0;
             key = ikey(ci.xbi + dd);
         } else {
@@ -1560,20 +1574,6 @@ __device__ __noinline__ void flush_queue(NbWarp<G> &W, int head, int n, int lane
     __syncwarp();
 }
 
-// Candidate evaluation of one sorted entry (prefix sums P / Pc inclusive).
-__device__ __forceinline__ void eval_entry(VCand &vb, const ColCtx &c, const Acc &a, unsigned long long kk,
-                                           long long del, unsigned aux, long long P, int Pc, unsigned long long kprev,
-                                           unsigned aprev, bool has_prev, unsigned long long knext, unsigned anext,
-                                           long long nviol, long long bestnv)
-{
-    if (!is_candidate(kk, aux, kprev, aprev, has_prev, knext, anext)) return;
-    const bool post = aux_post(aux) != 0;
-    const long long Pi = P - (post ? del : 0);
-    const int Pci = Pc - (post ? aux_dc(aux) : 0);
-    const bool right = kk > c.kxb;
-    consider(vb, c, kk, a.beta + Pi + (right ? a.alpha : 0), a.beta_c + Pci + (right ? a.alpha_c : 0), nviol, bestnv);
-}
-
 __device__ __forceinline__ void load_entry(const SEnt *p, unsigned long long &key, long long &del, unsigned &aux)
 {
     const int4 raw = *reinterpret_cast<const int4 *>(p);
@@ -1582,97 +1582,48 @@ __device__ __forceinline__ void load_entry(const SEnt *p, unsigned long long &ke
     aux = (unsigned)raw.w;
 }
 
-// Bitonic sort of G * K entries held K per lane by aligned groups of G lanes
-// (entry index sub * K + k, sub = lane % G).
-template <int K, int G>
-__device__ __forceinline__ void group_bitonic(unsigned long long (&key)[K], long long (&del)[K], unsigned (&aux)[K],
-                                              int sub)
+// Argmax of each group's list (cnt entries at list, at most cmax in any group
+// of the warp) without sorting: a lane takes every G-th entry and, when it is
+// a candidate, sums the deltas that count at its value (pre entries at or left
+// of it, post entries left of it).  Every lane returns the best candidate of
+// its group.  cnt^2 / G steps of a short loop against a bitonic network of
+// 64-bit keys with their deltas (5 words exchanged a stage): lists average 8
+// entries and hold 256 at most; all short columns of a general 200k-variable
+// MIP with outputs 256 -> 234 us a pass, 224 with the long lists counted too
+// (their network, 36 stages unrolled, waited for its code).
+template <int G>
+__device__ __forceinline__ VCand group_count(const ColCtx &c, const Acc &a, const SEnt *list, int cnt, int cmax,
+                                             long long nviol, long long bestnv)
 {
-    constexpr int N = G * K;
-#pragma unroll
-    for (int size = 2; size <= N; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride < K) {
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    if ((k & stride) == 0) {
-                        const int k2 = k | stride;
-                        const int i = sub * K + k;
-                        const bool asc = (i & size) == 0;
-                        if (entry_less(key[k2], aux[k2], key[k], aux[k]) == asc) {
-                            unsigned long long tk = key[k]; key[k] = key[k2]; key[k2] = tk;
-                            long long td = del[k]; del[k] = del[k2]; del[k2] = td;
-                            unsigned ta = aux[k]; aux[k] = aux[k2]; aux[k2] = ta;
-                        }
-                    }
-                }
-            } else {
-                const int ls = stride / K;
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const unsigned long long pk = __shfl_xor_sync(FULLMASK, key[k], ls);
-                    const long long pd = __shfl_xor_sync(FULLMASK, del[k], ls);
-                    const unsigned pa = __shfl_xor_sync(FULLMASK, aux[k], ls);
-                    const int i = sub * K + k;
-                    const bool lower = (i & stride) == 0;
-                    const bool asc = (i & size) == 0;
-                    const bool take = (lower == asc) ? entry_less(pk, pa, key[k], aux[k])
-                                                     : entry_less(key[k], aux[k], pk, pa);
-                    if (take) { key[k] = pk; del[k] = pd; aux[k] = pa; }
-                }
-            }
-        }
-    }
-}
-
-// Sort, scan and argmax of each group's list (cnt <= G * K entries at list),
-// K entries per lane; every lane returns the best candidate of its group.
-template <int K, int G>
-__device__ __forceinline__ VCand group_sort_scan(const ColCtx &c, const Acc &a, const SEnt *list, int cnt,
-                                                 long long nviol, long long bestnv)
-{
-    const int sub = (threadIdx.x & 31) & (G - 1);
-    unsigned long long key[K];
-    long long del[K];
-    unsigned aux[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int idx = sub * K + k;
-        if (idx < cnt) load_entry(list + idx, key[k], del[k], aux[k]);
-        else { key[k] = kPadKey; del[k] = 0; aux[k] = make_aux(kClsPost, 0); }
-    }
-    group_bitonic<K, G>(key, del, aux, sub);
-    long long P[K];
-    int Pc[K];
-    long long run = 0;
-    int runc = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) { run += del[k]; runc += aux_dc(aux[k]); P[k] = run; Pc[k] = runc; }
-    long long tot = run;
-    int totc = runc;
-#pragma unroll
-    for (int off = 1; off < G; off <<= 1) {
-        const long long x = __shfl_up_sync(FULLMASK, tot, off, G);
-        const int y = __shfl_up_sync(FULLMASK, totc, off, G);
-        if (sub >= off) { tot += x; totc += y; }
-    }
-    const long long ex = tot - run;
-    const int exc = totc - runc;
-    unsigned long long nk = __shfl_down_sync(FULLMASK, key[0], 1, G);
-    unsigned na = __shfl_down_sync(FULLMASK, aux[0], 1, G);
-    const unsigned long long pk = __shfl_up_sync(FULLMASK, key[K - 1], 1, G);
-    const unsigned pa = __shfl_up_sync(FULLMASK, aux[K - 1], 1, G);
-    if (sub == G - 1) { nk = kPadKey; na = make_aux(kClsPost, 0); }
+    const int lane = threadIdx.x & 31, sub = lane & (G - 1);
+    const int rot = min(lane / G, cmax - 1);
     VCand vb{0, 0ull, 0, 0};
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const unsigned long long knext = (k + 1 < K) ? key[(k + 1) % K] : nk;
-        const unsigned anext = (k + 1 < K) ? aux[(k + 1) % K] : na;
-        const unsigned long long kprev = (k > 0) ? key[(k + K - 1) % K] : pk;
-        const unsigned aprev = (k > 0) ? aux[(k + K - 1) % K] : pa;
-        eval_entry(vb, c, a, key[k], del[k], aux[k], ex + P[k], exc + Pc[k], kprev, aprev, k > 0 || sub > 0, knext,
-                   anext, nviol, bestnv);
+#pragma unroll 1
+    for (int k = sub; k - sub < cmax; k += G) {
+        unsigned long long key = kPadKey;
+        long long del;
+        unsigned aux = make_aux(kClsPostDelta, 0);
+        if (k < cnt) load_entry(list + k, key, del, aux);
+        const bool right = key > c.kxb;
+        long long s = a.beta + (right ? a.alpha : 0);
+        int dc = a.beta_c + (right ? a.alpha_c : 0);
+#pragma unroll 2
+        for (int e = 0; e < cmax; ++e) {
+            // the groups' lists lie 4 G entries apart: each starts at another
+            // entry, so that their loads fall into different banks
+            int i = e + rot;
+            i = i >= cmax ? i - cmax : i;
+            if (i >= cnt) continue;
+            unsigned long long ek;
+            long long ed;
+            unsigned ea;
+            load_entry(list + i, ek, ed, ea);
+            const bool in = ek < key || (ek == key && aux_post(ea) == 0);
+            s += in ? ed : 0;
+            dc += in ? aux_dc(ea) : 0;
+        }
+        const unsigned cls = aux_cls(aux);
+        if (k < cnt && (cls == kClsPre || cls == kClsPost)) consider(vb, c, key, s, dc, nviol, bestnv);
     }
 #pragma unroll
     for (int o = G >> 1; o > 0; o >>= 1) {
@@ -1735,21 +1686,13 @@ __device__ __noinline__ void column_warp(const Dev &d, const VarOut &o, int q, S
     const ColCtx c = make_col(d, q, iter);
     Acc acc;
     const int cnt = column_list<false>(d, c, stage, acc);
-    VCand vb;
-    if (cnt <= 32) vb = group_sort_scan<1, 32>(c, acc, stage, cnt, nviol, bestnv);
-    else if (cnt <= 64) vb = group_sort_scan<2, 32>(c, acc, stage, cnt, nviol, bestnv);
-    else if (cnt <= 128) vb = group_sort_scan<4, 32>(c, acc, stage, cnt, nviol, bestnv);
-    else vb = group_sort_scan<8, 32>(c, acc, stage, cnt, nviol, bestnv);
+    const VCand vb = group_count<32>(c, acc, stage, cnt, cnt, nviol, bestnv);
     if (lane == 0) finish_column(d, o, c, vb, best);
     __syncwarp();
 }
 
-// The best candidate of the column at position q in every lane, and its value,
-// without sorting: each lane takes candidates of the list and sums the deltas
-// that count at its value (pre entries at or left of it, post entries left of
-// it).  n^2 / 32 steps of a short loop instead of a sorting network: for the
-// few columns a search evaluates at a time, whose warps wait for the network's
-// code (15 to 115 KB unrolled) longer than for its arithmetic.
+// The best candidate of the column at position q in every lane, and its value;
+// row states may change inside the calling kernel.
 __device__ __noinline__ VCand column_best(const Dev &d, int q, SEnt *stage, long long iter, long long nviol,
                                           long long bestnv, double &xh)
 {
@@ -1757,25 +1700,7 @@ __device__ __noinline__ VCand column_best(const Dev &d, int q, SEnt *stage, long
     const ColCtx c = make_col(d, q, iter);
     Acc acc;
     const int cnt = column_list<true>(d, c, stage, acc);
-    VCand vb{0, 0ull, 0, 0};
-#pragma unroll 1
-    for (int k = lane; k - lane < cnt; k += 32) {
-        const SEnt me = k < cnt ? stage[k] : SEnt{c.kxb, 0, make_aux(kClsPostDelta, 0)};
-        const unsigned cls = aux_cls(me.aux);
-        const bool right = me.key > c.kxb;
-        long long s = acc.beta + (right ? acc.alpha : 0);
-        int dc = acc.beta_c + (right ? acc.alpha_c : 0);
-#pragma unroll 4
-        for (int e = 0; e < cnt; ++e) {
-            const SEnt t = stage[e];
-            if (t.key < me.key || (t.key == me.key && aux_post(t.aux) == 0)) {
-                s += t.del;
-                dc += aux_dc(t.aux);
-            }
-        }
-        if (cls == kClsPre || cls == kClsPost) consider(vb, c, me.key, s, dc, nviol, bestnv);
-    }
-    warp_reduce_vc(vb, c);
+    const VCand vb = group_count<32>(c, acc, stage, cnt, cnt, nviol, bestnv);
     __syncwarp();
     xh = vb.valid ? key_value(c, vb.key) : c.xb;
     return vb;
@@ -2016,12 +1941,8 @@ __global__ void __launch_bounds__(kEvalThreads, 3) k_eval_nb(Dev d, int q0, int 
             const int cn = (over || prune) ? 0 : cnt;
             if (cmax == 0) {
                 // every column of the warp pruned, overflowing or without entries
-            } else if (cmax <= G) {
-                vb = group_sort_scan<1, G>(c, acc, list, cn, nviol, bestnv);
-            } else if (cmax <= 2 * G) {
-                vb = group_sort_scan<2, G>(c, acc, list, cn, nviol, bestnv);
             } else {
-                vb = group_sort_scan<4, G>(c, acc, list, cn, nviol, bestnv);
+                vb = group_count<G>(c, acc, list, cn, cmax, nviol, bestnv);
             }
             if (sub == 0 && live && !over) {
                 finish_column(d, o, c, vb, best);
@@ -2081,12 +2002,13 @@ __device__ __forceinline__ void block_scan2(long long &v, int &vc, long long *ws
 // all threads of the CTA; ends with a barrier.
 __device__ void cta_bitonic(unsigned long long *skey, long long *sdel, unsigned *saux, int N)
 {
-    for (int size = 2; size <= N; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+    for (int ls = 1; (1 << ls) <= N; ++ls) {
+        for (int lt = ls - 1; lt >= 0; --lt) {
+            const int stride = 1 << lt;
             for (int p = threadIdx.x; p < (N >> 1); p += blockDim.x) {
-                const int i = 2 * stride * (p / stride) + (p % stride);
+                const int i = ((p >> lt) << (lt + 1)) | (p & (stride - 1));
                 const int k2 = i + stride;
-                const bool asc = (i & size) == 0;
+                const bool asc = (i & (1 << ls)) == 0;
                 unsigned long long ka = skey[i], kb = skey[k2];
                 unsigned aa = saux[i], ab = saux[k2];
                 if (entry_less(kb, ab, ka, aa) == asc) {
@@ -2523,6 +2445,305 @@ __global__ void __launch_bounds__(kLongThreads) k_long_eval(Dev d, const SEntry 
         finish_column(d, o, c, b, best);
         d.block_best[lc.slot] = best;
         *law = HistAcc{0, 0, 0, 0, 0u, 0};
+    }
+    finish_pass(d);
+}
+
+// -------------------------------------- ranked long lists (up to kRkMaxRuns runs)
+//
+// The same lists without a merge: k_rank_gen (one CTA per kRkChunk nonzeros)
+// sorts its entries in registers and writes the run with the prefix sums of
+// its deltas; k_rank_eval gives every candidate its score as the sum, over the
+// column's runs, of the prefix up to its place in the run (binary searches in
+// shared memory).  Two launches, 34 and 57 us, instead of a generation, log2
+// of the runs merge rounds, tile sums and a scan: 7 columns of 9,000 rows, 221
+// -> 131 us a pass.  The searches grow with entries x runs and the merge rounds
+// with entries x log(runs): at 64 runs (32,512 nonzeros) a thread's searches
+// are 700 steps in shared memory against 8 launches of 13 dependent loads from
+// L2; longer columns are merged.
+
+// Strict order of two entries of a ranked run: (t, class, entry), one
+// comparison for both partners of an exchange.
+__device__ __forceinline__ bool rank_less(unsigned long long k1, unsigned a1, unsigned long long k2, unsigned a2)
+{
+    return k1 < k2 || (k1 == k2 && a1 < a2);
+}
+
+// Sort of kRkRun entries, kRkRun / kRkThreads neighbouring ones per thread, by
+// (t, class): bitonic, the exchanges inside a thread in registers, inside a
+// warp by shuffles and only the widest (10 of 66) through shared memory.
+constexpr int kRkPer = kRkRun / kRkThreads;
+
+__device__ __forceinline__ void rank_sort(unsigned long long (&key)[kRkPer], unsigned (&aux)[kRkPer],
+                                          unsigned long long *skey, unsigned *saux)
+{
+    const int t = threadIdx.x;
+#pragma unroll 1
+    for (int size = 2; size <= kRkRun; size <<= 1) {
+#pragma unroll 1
+        for (int stride = size >> 1; stride >= kRkPer; stride >>= 1) {
+            const int ts = stride / kRkPer;   // distance in threads
+            const bool lower = (t & ts) == 0;
+            const bool wide = ts >= 32;
+            if (wide) {
+#pragma unroll
+                for (int u = 0; u < kRkPer; ++u) { skey[u * kRkThreads + t] = key[u]; saux[u * kRkThreads + t] = aux[u]; }
+                __syncthreads();
+            }
+#pragma unroll
+            for (int u = 0; u < kRkPer; ++u) {
+                unsigned long long pk;
+                unsigned pa;
+                if (wide) {
+                    pk = skey[u * kRkThreads + (t ^ ts)];
+                    pa = saux[u * kRkThreads + (t ^ ts)];
+                } else {
+                    pk = __shfl_xor_sync(FULLMASK, key[u], ts);
+                    pa = __shfl_xor_sync(FULLMASK, aux[u], ts);
+                }
+                const bool asc = ((t * kRkPer + u) & size) == 0;
+                if (rank_less(pk, pa, key[u], aux[u]) == (lower == asc)) { key[u] = pk; aux[u] = pa; }
+            }
+            if (wide) __syncthreads();
+        }
+#pragma unroll
+        for (int st = kRkPer / 2; st > 0; st >>= 1) {
+            if (st >= size) continue;
+#pragma unroll
+            for (int u = 0; u < kRkPer; ++u) {
+                if (u & st) continue;
+                const bool asc = ((t * kRkPer + u) & size) == 0;
+                if (rank_less(key[u | st], aux[u | st], key[u], aux[u]) == asc) {
+                    const unsigned long long tk = key[u]; key[u] = key[u | st]; key[u | st] = tk;
+                    const unsigned ta = aux[u]; aux[u] = aux[u | st]; aux[u | st] = ta;
+                }
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kRkThreads) k_rank_gen(Dev d, const Tile *tiles, int gate)
+{
+    if (gated_done(d, gate)) return;
+    __shared__ unsigned long long skey[kRkRun];
+    __shared__ unsigned saux[kRkRun];   // class (2 bits), entry (12 bits), count change + 1 (2 bits)
+    __shared__ int sdel[kRkRun];
+    __shared__ long long wsum[32];
+    __shared__ int wsumc[32];
+    __shared__ int s_cnt;
+    const Tile tl = tiles[blockIdx.x];
+    const RankCol rc = d.rcols[tl.begin];
+    const int run = tl.aux;
+    const ColCtx c = make_col(d, rc.pos, d.ctl->iter);
+    auto put = [&](int pos, unsigned long long key, long long del, unsigned aux) {
+        skey[pos] = key;
+        sdel[pos] = (int)del;
+        saux[pos] = aux | ((unsigned)pos << 2);
+    };
+    if (threadIdx.x == 0) {
+        int n0 = 0;
+        if (run == 0) {
+            if (dfinite(__ldg(d.lb + c.j))) put(n0++, c.kl, 0, make_aux(kClsPre, 0));
+            if (dfinite(__ldg(d.ub + c.j))) put(n0++, c.ku, 0, make_aux(kClsPre, 0));
+        }
+        s_cnt = n0;
+    }
+    __syncthreads();
+    Acc acc{0, 0, 0, 0};
+    const int v0 = run * kRkChunk, v1 = min(rc.len, v0 + kRkChunk);
+    for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+        Half h[2];
+        gen_entry(d, c, v, acc, h[0], h[1]);
+        const int n = half_entries(h[0]) + half_entries(h[1]);
+        // one atomic per converged group of the warp
+        const unsigned act = __activemask();
+        const int lane = threadIdx.x & 31;
+        int incl = 0, tot = 0;
+        for (unsigned m = act; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const int x = __shfl_sync(act, n, l);
+            tot += x;
+            if (l <= lane) incl += x;
+        }
+        int pos = 0;
+        const int lead = __ffs(act) - 1;
+        if (lane == lead) pos = atomicAdd(&s_cnt, tot);
+        pos = __shfl_sync(act, pos, lead) + incl - n;
+        if (!n) continue;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (h[k].type != 0) put(pos++, h[k].key, h[k].D, half_aux(h[k]));
+            if (h[k].mark) put(pos++, h[k].mkey, 0, marker_aux());
+        }
+    }
+    warp_allreduce_acc(acc);
+    HistAcc *la = d.racc + tl.begin;
+    if ((threadIdx.x & 31) == 0 && (acc.beta | acc.alpha | acc.beta_c | acc.alpha_c)) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(&la->beta), (unsigned long long)acc.beta);
+        atomicAdd(reinterpret_cast<unsigned long long *>(&la->alpha), (unsigned long long)acc.alpha);
+        atomicAdd(&la->beta_c, acc.beta_c);
+        atomicAdd(&la->alpha_c, acc.alpha_c);
+    }
+    __syncthreads();
+    const int cnt = s_cnt;
+    unsigned long long key[kRkPer];
+    unsigned aux[kRkPer];
+    const int i0 = threadIdx.x * kRkPer;
+#pragma unroll
+    for (int u = 0; u < kRkPer; ++u) {
+        key[u] = i0 + u < cnt ? skey[i0 + u] : kPadKey;
+        aux[u] = i0 + u < cnt ? saux[i0 + u] : make_aux(kClsPostDelta, 0) | ((unsigned)(i0 + u) << 2);
+    }
+    __syncthreads();
+    rank_sort(key, aux, skey, saux);
+    // prefix sums
+    long long P = 0;
+    int Pc = 0;
+#pragma unroll
+    for (int u = 0; u < kRkPer; ++u) {
+        if (i0 + u < cnt) {
+            P += sdel[(aux[u] >> 2) & (kRkRun - 1)];
+            Pc += aux_dc(aux[u]);
+        }
+    }
+    block_scan2(P, Pc, wsum, wsumc);
+    const long long base = rc.base + (long long)run * kRkRun;
+#pragma unroll
+    for (int u = 0; u < kRkPer; ++u) {
+        if (i0 + u < cnt) {
+            P += sdel[(aux[u] >> 2) & (kRkRun - 1)];
+            Pc += aux_dc(aux[u]);
+            d.rkey[base + i0 + u] = key[u];
+            d.raux[base + i0 + u] = aux[u];
+            d.rsum[base + i0 + u] = P;
+            d.rsumc[base + i0 + u] = Pc;
+        }
+    }
+    // the places of the run's candidates
+    auto is_cand = [&](int u) {
+        const unsigned cls = aux_cls(aux[u]);
+        return i0 + u < cnt && (cls == kClsPre || cls == kClsPost);
+    };
+    long long none = 0;
+    int nc = 0;
+#pragma unroll
+    for (int u = 0; u < kRkPer; ++u) nc += is_cand(u);
+    const int mine = nc;
+    block_scan2(none, nc, wsum, wsumc);
+    if (threadIdx.x == kRkThreads - 1) d.rccnt[rc.run0 + run] = nc + mine;
+#pragma unroll
+    for (int u = 0; u < kRkPer; ++u)
+        if (is_cand(u)) d.rcand_at[base + nc++] = (unsigned short)(i0 + u);
+    if (threadIdx.x == 0) d.rcnt[rc.run0 + run] = cnt;
+}
+
+// One CTA per run: its candidates (at most 2 per nonzero and the bounds, two a
+// thread, neighbouring ones in neighbouring threads) against every run of the column, the runs' keys staged in shared memory one
+// after the other, the next one loaded while one is searched.
+__global__ void __launch_bounds__(kRkThreads) k_rank_eval(Dev d, const Tile *tiles, VarOut o, int gate)
+{
+    if (gated_done(d, gate)) return;
+    __shared__ unsigned long long skey[kRkRun];
+    __shared__ unsigned char spost[kRkRun];
+    __shared__ int s_last;
+    const Tile tl = tiles[blockIdx.x];
+    const RankCol rc = d.rcols[tl.begin];
+    const long long iter = d.ctl->iter, nviol = d.ctl->nviol, bestnv = d.ctl->best_nviol;
+    const ColCtx c = make_col(d, rc.pos, iter);
+    HistAcc *la = d.racc + tl.begin;
+    const long long beta = __ldcg(&la->beta), alpha = __ldcg(&la->alpha);
+    const int bc = __ldcg(&la->beta_c), ac = __ldcg(&la->alpha_c);
+    const int run = tl.aux;
+    constexpr int PER = 2;
+    static_assert(PER * kRkThreads >= 2 * kRkChunk + 2, "a thread takes PER candidates of its run");
+    const int cnt = __ldg(d.rccnt + rc.run0 + run);
+    VCand vb{0, 0ull, 0, 0};
+    unsigned long long key[PER], nkey[kRkPer];
+    unsigned naux[kRkPer];
+    long long s[PER];
+    int dc[PER];
+    bool cand[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int i = u * kRkThreads + (int)threadIdx.x;
+        const long long at = rc.base + (long long)run * kRkRun;
+        cand[u] = i < cnt;
+        key[u] = cand[u] ? __ldg(d.rkey + at + __ldg(d.rcand_at + at + i)) : 0ull;
+        const bool right = key[u] > c.kxb;
+        s[u] = beta + (right ? alpha : 0);
+        dc[u] = bc + (right ? ac : 0);
+    }
+    auto fetch = [&](int r, int n) {
+        const long long b = rc.base + (long long)r * kRkRun;
+#pragma unroll
+        for (int u = 0; u < kRkPer; ++u) {
+            const int i = u * kRkThreads + (int)threadIdx.x;
+            nkey[u] = i < n ? __ldg(d.rkey + b + i) : kPadKey;
+            naux[u] = i < n ? __ldg(d.raux + b + i) : make_aux(kClsPost, 0);
+        }
+    };
+    int n = __ldg(d.rcnt + rc.run0);
+    fetch(0, n);
+    for (int r = 0; r < rc.runs; ++r) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kRkPer; ++u) {
+            skey[u * kRkThreads + threadIdx.x] = nkey[u];
+            spost[u * kRkThreads + threadIdx.x] = (unsigned char)aux_post(naux[u]);
+        }
+        __syncthreads();
+        const long long b = rc.base + (long long)r * kRkRun;
+        const int nn = r + 1 < rc.runs ? __ldg(d.rcnt + rc.run0 + r + 1) : 0;
+        fetch(min(r + 1, rc.runs - 1), nn);
+        // entries that count at key: those below it, and at it the pre entries
+        // (pads past the end are post entries of the largest key)
+        int lo[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) lo[u] = 0;
+#pragma unroll
+        for (int st = kRkRun >> 1; st > 0; st >>= 1) {
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int i = lo[u] + st - 1;
+                const unsigned long long km = skey[i];
+                if (km < key[u] || (km == key[u] && spost[i] == 0)) lo[u] += st;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            // the last entry of a full run
+            if (lo[u] == kRkRun - 1 && n == kRkRun &&
+                (skey[kRkRun - 1] < key[u] || (skey[kRkRun - 1] == key[u] && spost[kRkRun - 1] == 0))) lo[u] = kRkRun;
+            if (lo[u] == 0 || !cand[u]) continue;
+            s[u] += __ldg(d.rsum + b + lo[u] - 1);
+            dc[u] += __ldg(d.rsumc + b + lo[u] - 1);
+        }
+        n = nn;
+    }
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (cand[u]) consider(vb, c, key[u], s[u], dc[u], nviol, bestnv);
+    vb = block_reduce_vc(vb, c);
+    if (threadIdx.x == 0) {
+        d.rcand[rc.run0 + tl.aux] = LCand{vb.s, vb.key, vb.dc, vb.valid};
+        __threadfence();
+        s_last = atomicAdd(&la->ticket, 1u) == (unsigned)(rc.runs - 1);
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    VCand b{0, 0ull, 0, 0};
+    for (int t = threadIdx.x; t < rc.runs; t += blockDim.x) {
+        const LCand *p = d.rcand + rc.run0 + t;
+        const VCand v{__ldcg(&p->s), __ldcg(&p->key), __ldcg(&p->dc), __ldcg(&p->valid)};
+        if (vc_better(v, b, c)) b = v;
+    }
+    b = block_reduce_vc(b, c);
+    if (threadIdx.x == 0) {
+        Cand best{0, kNoVar, 0, 0.0};
+        finish_column(d, o, c, b, best);
+        d.block_best[rc.slot] = best;
+        *la = HistAcc{0, 0, 0, 0, 0u, 0};
     }
     finish_pass(d);
 }
@@ -3158,14 +3379,34 @@ int bin_grid_size(int ncols, int G)
     return (int)(need < cap ? need : cap);
 }
 
+static const void *nb_kernel(int G)
+{
+    return G == 4 ? (const void *)k_eval_nb<4> : G == 8 ? (const void *)k_eval_nb<8>
+           : G == 16 ? (const void *)k_eval_nb<16> : (const void *)k_eval_nb<32>;
+}
+static int nb_kernel_smem(int G) { return G == 4 ? nb_smem<4>() : G == 8 ? nb_smem<8>() : G == 16 ? nb_smem<16>() : nb_smem<32>(); }
+static int nb_slot(int G) { return G == 4 ? 0 : G == 8 ? 1 : G == 16 ? 12 : 13; }
+
+int nb_lanes(int ncols, int G)
+{
+    // more lanes per column while the columns leave warps of one resident wave
+    // without work (6.3k columns near a feasible point, most on the whole-warp
+    // path: 8 in turn on each of 790 warps with 4 lanes, 140 us; 2 on 3,150
+    // with 16); a handful of columns is latency either way
+    if (ncols < kNbWideMin) return G;
+    const long long warps = (long long)nb_grid_size(INT_MAX, G) * kNbWarps;
+    while (G < 32 && (long long)ncols * (2 * G) / 32 <= warps) G *= 2;
+    return G;
+}
+
 int nb_grid_size(int ncols, int G)
 {
     // one resident wave: every SM holds as many CTAs as fit, and no CTA is
     // launched without a column for each of its warps to start with
     int per_sm = 0;
-    const void *fn = G == 4 ? (const void *)k_eval_nb<4> : (const void *)k_eval_nb<8>;
-    const int smem = G == 4 ? nb_smem<4>() : nb_smem<8>();
-    if (raise_smem_limit(fn, G == 4 ? 0 : 1, smem) != cudaSuccess ||
+    const void *fn = nb_kernel(G);
+    const int smem = nb_kernel_smem(G);
+    if (raise_smem_limit(fn, nb_slot(G), smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kEvalThreads, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
@@ -3222,7 +3463,7 @@ cudaError_t static_hist_scratch(HBin **bins, HistAcc **acc)
 // largest size any handle launches with), under a mutex.
 static cudaError_t raise_smem_limit(const void *fn, int slot, int bytes)
 {
-    constexpr int kMaxDevices = 64, kSlots = 12;
+    constexpr int kMaxDevices = 64, kSlots = 14;
     static std::mutex s_mu;
     static int s_set[kMaxDevices][kSlots] = {};
     int dev = 0;
@@ -3240,8 +3481,7 @@ cudaError_t setup_kernel_attributes(const LaunchPlan &p)
 {
     cudaError_t e = cudaSuccess;
     if (p.nb_grid > 0)
-        e = p.nb_G == 4 ? raise_smem_limit((const void *)k_eval_nb<4>, 0, nb_smem<4>())
-                        : raise_smem_limit((const void *)k_eval_nb<8>, 1, nb_smem<8>());
+        e = raise_smem_limit(nb_kernel(p.nb_G), nb_slot(p.nb_G), nb_kernel_smem(p.nb_G));
     if (e == cudaSuccess && p.cta_smem > 0) e = raise_smem_limit((const void *)k_eval_cta, 2, p.cta_smem);
     if (e == cudaSuccess && p.hist_smem > 0) e = raise_smem_limit((const void *)k_eval_hist, 3, p.hist_smem);
     if (e == cudaSuccess && p.hist_smem > 0) e = raise_smem_limit((const void *)k_keep_hist, 9, p.hist_smem);
@@ -3297,7 +3537,7 @@ cudaError_t launch_eval_gated(const Dev &d, const LaunchPlan &p, const VarOut &o
     // selection.  The same fork/join shape is recorded by graph capture.
     if (o.xhat || o.s || o.dc) k_fill_outputs<<<grid_for(d.n, 256), 256, 0, st>>>(d, o);
     cudaError_t e = cudaEventRecord(p.ev_fork, st);
-    const bool side[3] = {p.nb_grid > 0, p.n_cta > 0 || p.n_lgen > 0, p.n_hist_tiles > 0};
+    const bool side[3] = {p.nb_grid > 0, p.n_cta > 0 || p.n_lgen > 0 || p.n_rgen > 0, p.n_hist_tiles > 0};
     for (int k = 0; k < 3 && e == cudaSuccess; ++k)
         if (side[k]) e = cudaStreamWaitEvent(p.side[k], p.ev_fork, 0);
     if (e != cudaSuccess) return e;
@@ -3333,16 +3573,12 @@ cudaError_t launch_eval_gated(const Dev &d, const LaunchPlan &p, const VarOut &o
         }
         PROF(0, 1);
     }
-    if (p.nb_grid) {
-        PROF(1, 0);
-        if (p.nb_G == 4)
-            k_eval_nb<4><<<p.nb_grid, kEvalThreads, nb_smem<4>(), p.side[0]>>>(d, p.nb_q0, p.nb_cols, o, p.slot_nb, gate);
-        else
-            k_eval_nb<8><<<p.nb_grid, kEvalThreads, nb_smem<8>(), p.side[0]>>>(d, p.nb_q0, p.nb_cols, o, p.slot_nb, gate);
-        PROF(1, 1);
-    }
-    if (p.n_cta || p.n_lgen) {
+    if (p.n_cta || p.n_lgen || p.n_rgen) {
         PROF(2, 0);
+        if (p.n_rgen) {
+            k_rank_gen<<<p.n_rgen, kRkThreads, 0, p.side[1]>>>(d, p.tiles_rgen, gate);
+            k_rank_eval<<<p.n_rgen, kRkThreads, 0, p.side[1]>>>(d, p.tiles_rgen, o, gate);
+        }
         if (p.n_cta) k_eval_cta<<<p.n_cta, kCtaThreads, p.cta_smem, p.side[1]>>>(d, p.tiles_cta, o, p.slot_cta, gate);
         if (p.n_lgen && e == cudaSuccess) e = launch_long(d, p, o, gate, p.side[1]);
         PROF(2, 1);
@@ -3351,6 +3587,16 @@ cudaError_t launch_eval_gated(const Dev &d, const LaunchPlan &p, const VarOut &o
         PROF(3, 0);
         k_eval_hist<<<p.n_hist_tiles, kHistThreads, p.hist_smem, p.side[2]>>>(d, p.tiles_hist, o, gate);
         PROF(3, 1);
+    }
+    if (p.nb_grid) {
+        PROF(1, 0);
+        switch (p.nb_G) {
+        case 4: k_eval_nb<4><<<p.nb_grid, kEvalThreads, nb_smem<4>(), p.side[0]>>>(d, p.nb_q0, p.nb_cols, o, p.slot_nb, gate); break;
+        case 8: k_eval_nb<8><<<p.nb_grid, kEvalThreads, nb_smem<8>(), p.side[0]>>>(d, p.nb_q0, p.nb_cols, o, p.slot_nb, gate); break;
+        case 16: k_eval_nb<16><<<p.nb_grid, kEvalThreads, nb_smem<16>(), p.side[0]>>>(d, p.nb_q0, p.nb_cols, o, p.slot_nb, gate); break;
+        default: k_eval_nb<32><<<p.nb_grid, kEvalThreads, nb_smem<32>(), p.side[0]>>>(d, p.nb_q0, p.nb_cols, o, p.slot_nb, gate); break;
+        }
+        PROF(1, 1);
     }
 #undef PROF
     if (e == cudaSuccess) e = cudaGetLastError();

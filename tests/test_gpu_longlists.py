@@ -118,3 +118,52 @@ def test_long_list_scratch_returns_to_zero(chap):
             bs.step()
     ha.close()
     hb.close()
+
+
+
+def _integer_column_best(prob, x, j):
+    """(value, score in half weights, violation change) of integer column j at x
+    with unit weights and no tabu, rows all <= or >= and integral: every half's
+    penalty change summed over a sorted list (the oracle's definition, whose
+    recomputation of every row at every candidate is quadratic here)."""
+    rows = np.repeat(np.arange(prob.m), np.diff(prob.row_ptr))
+    sgn = np.where(prob.sense == inst.ROW_GE, -1.0, 1.0)
+    res = sgn * (np.bincount(rows, weights=prob.row_val * x[prob.col_idx], minlength=prob.m) - prob.rhs)
+    e = slice(prob.col_ptr[j], prob.col_ptr[j + 1])
+    a, r, xb = sgn[prob.row_idx[e]] * prob.col_val[e], res[prob.row_idx[e]], x[j]
+    v, up = r > 0, a > 0
+    t = xb + np.where(up, np.floor(-r / a), np.ceil(-r / a))     # last satisfied integer
+    cand = np.unique(np.concatenate([t, [prob.lb[j], prob.ub[j]]]))
+    cand = cand[(cand >= prob.lb[j]) & (cand <= prob.ub[j]) & (cand != xb)]
+    # left of everything, the change at t (a > 0: right after it), the change at xb
+    base = np.where(up, np.where(v, 2, 0), np.where(v, -1, -2)).sum()
+    d = np.where(up, np.where(v, -1, -2), np.where(v, 1, 2))
+    cross = np.where(v, np.where(up, -2, 2), 0).sum()
+    cb, c = np.where(up, -v.astype(int), (~v).astype(int)).sum(), np.where(up, 1, -1)
+    order = np.argsort(t, kind="stable")
+
+    def upto(mask, delta, side):
+        k = order[mask[order]]
+        return np.concatenate([[0], np.cumsum(delta[k])])[np.searchsorted(t[k], cand, side)]
+
+    s = base + upto(~up, d, "right") + upto(up, d, "left") + np.where(cand > xb, cross, 0)
+    n = cb + upto(~up, c, "right") + upto(up, c, "left")
+    k = min(range(len(cand)), key=lambda i: (-s[i], abs(cand[i] - xb), cand[i]))
+    return (cand[k], int(s[k]), int(n[k])) if s[k] > 0 else (xb, 0, 0)
+
+
+@pytest.mark.parametrize("rows", [9_000, 32_512, 32_513])
+def test_ranked_and_merged_lists(chap, rows):
+    """The longest list that is ranked (64 runs of 508 nonzeros), the shortest
+    that is merged, and an ordinary one."""
+    prob = long_instance(9, [I], rows_per_long=rows, n_other=40, eq_frac=0.0)
+    bs = chap.BestShift(prob, tenure=3, feas_tol=0.0)
+    assert bs.info.n_long_cols == 1
+    rng = np.random.default_rng(2)
+    for _ in range(3):
+        x = np.floor(rng.random(prob.n) * (prob.ub + 1))
+        x = np.minimum(x, prob.ub)
+        bs.set_state(x)
+        g = bs.best_shift()
+        assert (g[0][0], int(g[1][0]), int(g[2][0])) == _integer_column_best(prob, x, 0)
+    bs.close()

@@ -198,3 +198,28 @@ def test_chains_default_schedule(chap, stop):
                     (st["iter"], st["moves"], st["nviol"], st["best_nviol"]), c
                 assert np.array_equal(b.x(c), st["x"]), c
         b.close()
+
+
+@pytest.mark.parametrize("n,lanes", [(8_000, 32), (20_000, 16), (60_000, 8)])
+def test_short_column_lanes_fill_the_gpu(chap, n, lanes):
+    """Short non-binary columns at every lane count the library picks, far from
+    and near a feasible point (short lists, and lists longer than a group's):
+    scores and violation changes equal the oracle's, values within the rounding
+    of a breakpoint (two roundings of 1e-16, asserted at 1e-9)."""
+    prob = inst.gen_general(seed=17, n=n, m=n // 2, len_cap=n // 100)
+    bs = chap.BestShift(prob, tenure=5)
+    assert bs.info.nb_lanes == lanes
+    orc = Oracle(prob)
+    rng = np.random.default_rng(1)
+    pick = np.sort(rng.choice(np.flatnonzero(prob.vtype != inst.VAR_BIN), size=1500, replace=False)).astype(np.int32)
+    for run in (0, 400):
+        if run:
+            bs.run(max_iters=run, stop_at_feasible=0)
+        bs.set_checkpoint(bs.state())
+        st = bs.state()
+        g = bs.best_shift()
+        o = orc.best_shift(st["x"], st["w"], st["tabu_inc"], st["tabu_dec"], st["iter"], st["nviol"], st["best_nviol"],
+                           vars=pick)
+        assert np.array_equal(g[1][pick], o[1]) and np.array_equal(g[2][pick], o[2])
+        assert np.allclose(g[0][pick], o[0], rtol=1e-9, atol=1e-9)
+    bs.close()
