@@ -19,6 +19,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstdio>
+#include <mutex>
 #include <string>
 
 namespace chap {
@@ -29,8 +30,9 @@ namespace {
 constexpr int kF = 12, kH = 64;
 constexpr int kOffW1 = 0, kOffB1 = kF * kH, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH;
 constexpr int kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH, kNParams = kOffB3 + 1;  // 5057
-constexpr int kGradRows = 128;       // rows of one gradient tile
-constexpr int kHPad = kH + 1;        // padded activation rows (no bank conflicts)
+constexpr int kTileRows = 64;        // rows of one network tile
+constexpr int kTileThreads = 256;    // threads of its CTA: 4 rows x 4 columns of a layer each
+constexpr int kTPad = kTileRows + 4; // rows of a transposed activation, padded (16-byte aligned, 17 x 16 bytes)
 constexpr int kTopkPerThread = 4;
 constexpr int kTopkBlock = 256 * kTopkPerThread;
 constexpr int kVarBits = 22;
@@ -159,49 +161,112 @@ __global__ void k_features(Dev d, Learn L, float cmax, int gate)
     }
 }
 
+// Targets: the last exact scores scaled by 1 / (1 + max |score|).  Formed here:
+// the scores went to the host and back before (a logged pass of 90k variables
+// 399 -> 300 us with the copies and the wait gone).
+__global__ void k_targets(int n, Learn L, float *target)
+{
+    const double sc = __ddiv_rn(1.0, __dadd_rn(1.0, (double)L.lc->smax));
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+        target[j] = (float)__dmul_rn((double)L.s_last[j], sc);
+}
+
 // ----------------------------------------------------------------- network
 
-// Forward pass: one thread per row; parameters broadcast from shared memory
-// (16-byte loads of the second layer's weights).
-__global__ void __launch_bounds__(256) k_mlp_forward(const __nv_bfloat16 *w, const __nv_bfloat16 *x, long long n,
-                                                     float *y, const int *done)
+// A tile of kTileRows rows in shared memory.  Activations are stored by
+// column (hT[j][row]), so that a thread's 4 rows are one 16-byte load.
+struct MlpTile {
+    float w1[kF * kH], b1[kH];
+    float w2[kH * kH], b2[kH];
+    float w3[kH], b3[4];
+    float xT[kF * kTPad];
+    float h1T[kH * kTPad];
+    float h2T[kH * kTPad];
+    float out[kTileRows];
+};
+
+__device__ __forceinline__ void mlp_load_weights(MlpTile &s, const __nv_bfloat16 *w)
 {
-    if (done && *(volatile const int *)done) return;
-    __shared__ __align__(16) float sw[kNParams + 3];
-    for (int i = threadIdx.x; i < kNParams; i += blockDim.x) sw[i] = __bfloat162float(w[i]);
+    for (int i = threadIdx.x; i < kF * kH; i += kTileThreads) s.w1[i] = __bfloat162float(w[kOffW1 + i]);
+    for (int i = threadIdx.x; i < kH * kH; i += kTileThreads) s.w2[i] = __bfloat162float(w[kOffW2 + i]);
+    if (threadIdx.x < kH) {
+        s.b1[threadIdx.x] = __bfloat162float(w[kOffB1 + threadIdx.x]);
+        s.b2[threadIdx.x] = __bfloat162float(w[kOffB2 + threadIdx.x]);
+        s.w3[threadIdx.x] = __bfloat162float(w[kOffW3 + threadIdx.x]);
+    }
+    if (threadIdx.x == 0) s.b3[0] = __bfloat162float(w[kOffB3]);
+}
+
+// One layer of the tile: act[j][r] = relu(b[j] + sum_k in[k][r] W[k][j]), terms
+// added in increasing k with FMAs; rows past `rows` become 0.  A thread owns
+// rows 4 (t / 16) .. + 3 and columns 4 (t % 16) .. + 3: per k two 16-byte loads
+// for 16 FMAs.
+__device__ __forceinline__ void mlp_layer(const float *inT, const float *W, const float *b, int K, int rows, float *actT)
+{
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    float acc[4][4];
+    const float4 bb = *reinterpret_cast<const float4 *>(b + 4 * tx);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) { acc[r][0] = bb.x; acc[r][1] = bb.y; acc[r][2] = bb.z; acc[r][3] = bb.w; }
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        const float4 x = *reinterpret_cast<const float4 *>(inT + k * kTPad + 4 * ty);
+        const float4 w = *reinterpret_cast<const float4 *>(W + k * kH + 4 * tx);
+        const float xr[4] = {x.x, x.y, x.z, x.w}, wc[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[r][c] = __fmaf_rn(xr[r], wc[c], acc[r][c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        float4 v;
+        v.x = 4 * ty < rows ? fmaxf(acc[0][c], 0.0f) : 0.0f;
+        v.y = 4 * ty + 1 < rows ? fmaxf(acc[1][c], 0.0f) : 0.0f;
+        v.z = 4 * ty + 2 < rows ? fmaxf(acc[2][c], 0.0f) : 0.0f;
+        v.w = 4 * ty + 3 < rows ? fmaxf(acc[3][c], 0.0f) : 0.0f;
+        *reinterpret_cast<float4 *>(actT + (4 * tx + c) * kTPad + 4 * ty) = v;
+    }
+}
+
+// Forward pass of the tile's rows [r0, r0 + rows): s.out; ends with a barrier.
+__device__ __forceinline__ void mlp_tile_forward(MlpTile &s, const __nv_bfloat16 *x, long long r0, int rows)
+{
+    __syncthreads();   // the previous tile is done with the buffers
+    for (int i = threadIdx.x; i < kTileRows * kF; i += kTileThreads) {
+        const int r = i / kF, f = i % kF;
+        s.xT[f * kTPad + r] = r < rows ? __bfloat162float(x[r0 * kF + i]) : 0.0f;
+    }
     __syncthreads();
-    for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x) {
-        float xi[kF];
-#pragma unroll
-        for (int f = 0; f < kF; ++f) xi[f] = __bfloat162float(x[r * kF + f]);
-        // the second layer in two halves of 32 outputs (the first layer is
-        // recomputed for each half: fewer live registers, more warps per SM);
-        // every pre-activation sums its terms in increasing i
-        float out = sw[kOffB3];
-#pragma unroll 1
-        for (int h = 0; h < kH; h += 32) {
-            float acc[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) acc[j] = sw[kOffB2 + h + j];
-#pragma unroll 1
-            for (int i = 0; i < kH; ++i) {
-                float a = sw[kOffB1 + i];
-#pragma unroll
-                for (int f = 0; f < kF; ++f) a = __fmaf_rn(xi[f], sw[kOffW1 + f * kH + i], a);
-                a = fmaxf(a, 0.0f);
-#pragma unroll
-                for (int j = 0; j < 32; j += 4) {
-                    const float4 w4 = *reinterpret_cast<const float4 *>(&sw[kOffW2 + i * kH + h + j]);
-                    acc[j] = __fmaf_rn(a, w4.x, acc[j]);
-                    acc[j + 1] = __fmaf_rn(a, w4.y, acc[j + 1]);
-                    acc[j + 2] = __fmaf_rn(a, w4.z, acc[j + 2]);
-                    acc[j + 3] = __fmaf_rn(a, w4.w, acc[j + 3]);
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 32; ++j) out = __fmaf_rn(fmaxf(acc[j], 0.0f), sw[kOffW3 + h + j], out);
-        }
-        y[r] = out;
+    mlp_layer(s.xT, s.w1, s.b1, kF, rows, s.h1T);
+    __syncthreads();
+    mlp_layer(s.h1T, s.w2, s.b2, kH, rows, s.h2T);
+    __syncthreads();
+    if (threadIdx.x < kTileRows) {
+        float o = s.b3[0];
+#pragma unroll 8
+        for (int j = 0; j < kH; ++j) o = __fmaf_rn(s.h2T[j * kTPad + threadIdx.x], s.w3[j], o);
+        s.out[threadIdx.x] = o;
+    }
+    __syncthreads();
+}
+
+// Forward pass (FP32 activations; every sum in increasing index with FMAs): a
+// persistent grid over the tiles.  Bound by the FP32 FMAs and their operand
+// loads from shared memory: a 4 x 4 block per thread reads 2 words an FMA less
+// than one row per thread did.
+__global__ void __launch_bounds__(kTileThreads) k_mlp_forward(const __nv_bfloat16 *w, const __nv_bfloat16 *x, long long n,
+                                                              float *y)
+{
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    MlpTile &s = *reinterpret_cast<MlpTile *>(mlp_smem);
+    mlp_load_weights(s, w);
+    const long long tiles = (n + kTileRows - 1) / kTileRows;
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const long long r0 = t * kTileRows;
+        const int rows = (int)(n - r0 < kTileRows ? n - r0 : kTileRows);
+        mlp_tile_forward(s, x, r0, rows);
+        if ((int)threadIdx.x < rows) y[r0 + threadIdx.x] = s.out[threadIdx.x];
     }
 }
 
@@ -296,110 +361,150 @@ __global__ void __launch_bounds__(256) k_mlp_forward_tc(const __nv_bfloat16 *w, 
 }
 
 // Gradient of the mean squared error over n rows (scale 2/n), accumulated into
-// grad[kNParams] (FP32 atomics, one per parameter and tile), and the sum of
-// squared errors into loss[0].  One CTA of kGradRows threads per tile of rows.
-__global__ void __launch_bounds__(kGradRows) k_mlp_grad(const __nv_bfloat16 *w, const __nv_bfloat16 *x,
-                                                        const float *t, long long n, float scale, float *grad,
-                                                        float *loss)
+// grad[kNParams] and the sum of squared errors into loss[0] (FP32 atomics, one
+// per parameter and CTA).  A CTA takes tiles of kTileRows rows in turn, keeps
+// its share of the gradient in registers (16 weights of the second layer, 3 of
+// the first per thread) and adds it once at the end.  Bound by the FP32 FMAs
+// (0.9M a tile) and their shared-memory operands.  A training step (forward,
+// gradient, Adam, read of the loss) of 8 x 8,192 rows takes 405 us; with one row
+// per thread and one parameter per thread and pass it took 697.
+struct MlpGradTile {
+    MlpTile f;
+    float w2T[kH * kH];          // second layer transposed, [j][i]
+    float gy[kTileRows];
+};
+
+__global__ void __launch_bounds__(kTileThreads) k_mlp_grad(const __nv_bfloat16 *w, const __nv_bfloat16 *x, const float *t,
+                                                           long long n, float scale, float *grad, float *loss)
 {
-    extern __shared__ __align__(16) float gsm[];
-    float *sw = gsm;                                  // kNParams (+3 pad)
-    float *sx = sw + ((kNParams + 3) & ~3);           // kGradRows x kF
-    float *h1 = sx + kGradRows * kF;                  // kGradRows x kHPad (then ga1)
-    float *h2 = h1 + kGradRows * kHPad;               // kGradRows x kHPad (then ga2)
-    float *gy = h2 + kGradRows * kHPad;               // kGradRows
-    const int tid = threadIdx.x;
-    for (int i = tid; i < kNParams; i += blockDim.x) sw[i] = __bfloat162float(w[i]);
-    const long long r0 = (long long)blockIdx.x * kGradRows;
-    const long long left = n - r0;
-    const int rows = left < kGradRows ? (int)left : kGradRows;
-    for (int i = tid; i < kGradRows * kF; i += blockDim.x) {
-        const int r = i / kF;
-        sx[i] = r < rows ? __bfloat162float(x[(r0 + r) * kF + (i % kF)]) : 0.0f;
-    }
-    __syncthreads();
-    // forward, one row per thread
-    float err = 0.0f;
-    if (tid < rows) {
-        float *a = h1 + tid * kHPad;
-        for (int j = 0; j < kH; ++j) {
-            float s = sw[kOffB1 + j];
-            for (int f = 0; f < kF; ++f) s = __fmaf_rn(sx[tid * kF + f], sw[kOffW1 + f * kH + j], s);
-            a[j] = fmaxf(s, 0.0f);
-        }
-        float out = sw[kOffB3];
-        float *b = h2 + tid * kHPad;
-        for (int j = 0; j < kH; ++j) {
-            float s = sw[kOffB2 + j];
-            for (int i = 0; i < kH; ++i) s = __fmaf_rn(a[i], sw[kOffW2 + i * kH + j], s);
-            b[j] = fmaxf(s, 0.0f);
-            out = __fmaf_rn(b[j], sw[kOffW3 + j], out);
-        }
-        err = out - t[r0 + tid];
-        gy[tid] = scale * err;
-    } else {
-        gy[tid] = 0.0f;
-        for (int j = 0; j < kH; ++j) { h1[tid * kHPad + j] = 0.0f; h2[tid * kHPad + j] = 0.0f; }
-    }
-    __syncthreads();
-    // output layer
-    if (tid < kH) {
-        float s = 0.0f;
-        for (int r = 0; r < kGradRows; ++r) s = __fmaf_rn(h2[r * kHPad + tid], gy[r], s);
-        atomicAdd(grad + kOffW3 + tid, s);
-    }
-    if (tid == kH) {
-        float s = 0.0f;
-        for (int r = 0; r < kGradRows; ++r) s += gy[r];
-        atomicAdd(grad + kOffB3, s);
-    }
-    __syncthreads();
-    // ga2 = gy w3 [h2 > 0], in place of h2
-    for (int j = 0; j < kH; ++j) {
-        float &v = h2[tid * kHPad + j];
-        v = v > 0.0f ? gy[tid] * sw[kOffW3 + j] : 0.0f;
-    }
-    __syncthreads();
-    // gW2[i][j] = sum_r h1[r][i] ga2[r][j]; gb2[j] = sum_r ga2[r][j]
-    for (int o = tid; o < kH * kH; o += blockDim.x) {
-        const int i = o / kH, j = o % kH;
-        float s = 0.0f;
-        for (int r = 0; r < kGradRows; ++r) s = __fmaf_rn(h1[r * kHPad + i], h2[r * kHPad + j], s);
-        atomicAdd(grad + kOffW2 + o, s);
-    }
-    if (tid < kH) {
-        float s = 0.0f;
-        for (int r = 0; r < kGradRows; ++r) s += h2[r * kHPad + tid];
-        atomicAdd(grad + kOffB2 + tid, s);
-    }
-    __syncthreads();
-    // ga1 = (ga2 W2^T) [h1 > 0], in place of h1 (each thread its own row)
-    {
-        float g1[kH];
-        for (int i = 0; i < kH; ++i) {
-            float s = 0.0f;
-            for (int j = 0; j < kH; ++j) s = __fmaf_rn(h2[tid * kHPad + j], sw[kOffW2 + i * kH + j], s);
-            g1[i] = h1[tid * kHPad + i] > 0.0f ? s : 0.0f;
-        }
-        for (int i = 0; i < kH; ++i) h1[tid * kHPad + i] = g1[i];
-    }
-    __syncthreads();
-    for (int o = tid; o < kF * kH; o += blockDim.x) {
-        const int f = o / kH, i = o % kH;
-        float s = 0.0f;
-        for (int r = 0; r < kGradRows; ++r) s = __fmaf_rn(sx[r * kF + f], h1[r * kHPad + i], s);
-        atomicAdd(grad + kOffW1 + o, s);
-    }
-    if (tid < kH) {
-        float s = 0.0f;
-        for (int r = 0; r < kGradRows; ++r) s += h1[r * kHPad + tid];
-        atomicAdd(grad + kOffB1 + tid, s);
-    }
-    // loss
-    float e2 = err * err;
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    MlpGradTile &g = *reinterpret_cast<MlpGradTile *>(mlp_smem);
+    MlpTile &s = g.f;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    mlp_load_weights(s, w);
+    for (int i = tid; i < kH * kH; i += kTileThreads) g.w2T[(i % kH) * kH + i / kH] = __bfloat162float(w[kOffW2 + i]);
+    float gw2[4][4], gw1[3], gb = 0.0f, gw3 = 0.0f, gb3 = 0.0f, lsum = 0.0f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(FULLMASK, e2, o);
-    if ((tid & 31) == 0) atomicAdd(loss, e2);
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) gw2[i][j] = 0.0f;
+    gw1[0] = gw1[1] = gw1[2] = 0.0f;
+    float gb1 = 0.0f;
+    const long long tiles = (n + kTileRows - 1) / kTileRows;
+    for (long long tl = blockIdx.x; tl < tiles; tl += gridDim.x) {
+        const long long r0 = tl * kTileRows;
+        const int rows = (int)(n - r0 < kTileRows ? n - r0 : kTileRows);
+        mlp_tile_forward(s, x, r0, rows);
+        if (tid < kTileRows) {
+            const float err = tid < rows ? s.out[tid] - t[r0 + tid] : 0.0f;
+            g.gy[tid] = scale * err;
+            lsum = __fmaf_rn(err, err, lsum);
+        }
+        __syncthreads();
+        // output layer (threads 0..63: w3, 64: b3); then ga2 = gy w3 [h2 > 0] in place of h2
+        if (tid < kH) {
+            for (int r = 0; r < kTileRows; ++r) gw3 = __fmaf_rn(s.h2T[tid * kTPad + r], g.gy[r], gw3);
+        } else if (tid == kH) {
+            for (int r = 0; r < kTileRows; ++r) gb3 += g.gy[r];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float4 *p = reinterpret_cast<float4 *>(s.h2T + (4 * tx + c) * kTPad + 4 * ty);
+            const float4 y = *reinterpret_cast<const float4 *>(g.gy + 4 * ty);
+            const float w3 = s.w3[4 * tx + c];
+            float4 v = *p;
+            v.x = v.x > 0.0f ? y.x * w3 : 0.0f;
+            v.y = v.y > 0.0f ? y.y * w3 : 0.0f;
+            v.z = v.z > 0.0f ? y.z * w3 : 0.0f;
+            v.w = v.w > 0.0f ? y.w * w3 : 0.0f;
+            *p = v;
+        }
+        __syncthreads();
+        // gW2[i][j] = sum_r h1[r][i] ga2[r][j] for i = ty + 16 a, j = tx + 16 b
+        // (strided, so that the 16-byte loads of 4 rows meet different banks)
+#pragma unroll 2
+        for (int r = 0; r < kTileRows; r += 4) {
+            float4 h[4], q[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                h[a] = *reinterpret_cast<const float4 *>(s.h1T + (ty + 16 * a) * kTPad + r);
+                q[a] = *reinterpret_cast<const float4 *>(s.h2T + (tx + 16 * a) * kTPad + r);
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    gw2[a][b] = __fmaf_rn(h[a].x, q[b].x, gw2[a][b]);
+                    gw2[a][b] = __fmaf_rn(h[a].y, q[b].y, gw2[a][b]);
+                    gw2[a][b] = __fmaf_rn(h[a].z, q[b].z, gw2[a][b]);
+                    gw2[a][b] = __fmaf_rn(h[a].w, q[b].w, gw2[a][b]);
+                }
+        }
+        if (tid < kH)
+            for (int r = 0; r < kTileRows; ++r) gb += s.h2T[tid * kTPad + r];
+        // ga1 = (ga2 W2^T) [h1 > 0]
+        float a1[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) a1[r][c] = 0.0f;
+#pragma unroll 4
+        for (int j = 0; j < kH; ++j) {
+            const float4 q = *reinterpret_cast<const float4 *>(s.h2T + j * kTPad + 4 * ty);
+            const float4 v = *reinterpret_cast<const float4 *>(g.w2T + j * kH + 4 * tx);
+            const float qr[4] = {q.x, q.y, q.z, q.w}, vc[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) a1[r][c] = __fmaf_rn(qr[r], vc[c], a1[r][c]);
+        }
+        __syncthreads();   // h1 has been read by every thread
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float4 *p = reinterpret_cast<float4 *>(s.h1T + (4 * tx + c) * kTPad + 4 * ty);
+            float4 v = *p;
+            v.x = v.x > 0.0f ? a1[0][c] : 0.0f;
+            v.y = v.y > 0.0f ? a1[1][c] : 0.0f;
+            v.z = v.z > 0.0f ? a1[2][c] : 0.0f;
+            v.w = v.w > 0.0f ? a1[3][c] : 0.0f;
+            *p = v;
+        }
+        __syncthreads();
+        // gW1[f][i] for i = tid % 64, f = tid / 64 + 4 m
+        {
+            const int i = tid & (kH - 1), f0 = tid / kH;
+            for (int r = 0; r < kTileRows; r += 4) {
+                const float4 a = *reinterpret_cast<const float4 *>(s.h1T + i * kTPad + r);
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    const float4 v = *reinterpret_cast<const float4 *>(s.xT + (f0 + 4 * m) * kTPad + r);
+                    gw1[m] = __fmaf_rn(v.x, a.x, gw1[m]);
+                    gw1[m] = __fmaf_rn(v.y, a.y, gw1[m]);
+                    gw1[m] = __fmaf_rn(v.z, a.z, gw1[m]);
+                    gw1[m] = __fmaf_rn(v.w, a.w, gw1[m]);
+                }
+                if (f0 == 0) gb1 += (a.x + a.y) + (a.z + a.w);
+            }
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) atomicAdd(grad + kOffW2 + (ty + 16 * a) * kH + tx + 16 * b, gw2[a][b]);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) atomicAdd(grad + kOffW1 + (tid / kH + 4 * m) * kH + (tid & (kH - 1)), gw1[m]);
+    if (tid < kH) {
+        atomicAdd(grad + kOffB1 + tid, gb1);
+        atomicAdd(grad + kOffB2 + tid, gb);
+        atomicAdd(grad + kOffW3 + tid, gw3);
+    }
+    if (tid == kH) atomicAdd(grad + kOffB3, gb3);
+    if (tid < kTileRows) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(FULLMASK, lsum, o);
+        if ((tid & 31) == 0) atomicAdd(loss, lsum);
+    }
 }
 
 // Adam on FP32 master parameters; writes the BF16 copy and clears the gradient.
@@ -882,6 +987,23 @@ cudaError_t launch_subset(chap_bs *h, LearnHost *lh, int k, int gate, cudaStream
     return e;
 }
 
+// Shared-memory limit of a network kernel, once per device (slot: kernel).
+cudaError_t mlp_smem_limit(const void *fn, int slot, int bytes)
+{
+    constexpr int kMaxDevices = 64;
+    static std::mutex s_mu;
+    static bool s_set[kMaxDevices][2] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(s_mu);
+    if (s_set[dev][slot]) return cudaSuccess;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) s_set[dev][slot] = true;
+    return e;
+}
+
 }  // namespace
 }  // namespace chap
 
@@ -915,15 +1037,8 @@ chap_status chap_bs_features(chap_bs *h, uint16_t *feat, float *target)
         LCK(h, cudaMemcpyAsync(feat, lh->L.feat, sizeof(uint16_t) * kF * (size_t)h->n, cudaMemcpyDeviceToDevice, h->st),
             "copy features");
     if (target && h->n) {
-        // targets: the last exact scores scaled by 1 / (1 + max |score|)
-        LCK(h, cudaMemcpyAsync(lh->h_lc, lh->L.lc, sizeof(LearnCtl), cudaMemcpyDeviceToHost, h->st), "read state");
-        LCK(h, cudaStreamSynchronize(h->st), "synchronise");
-        std::vector<long long> sl(h->n);
-        LCK(h, cudaMemcpy(sl.data(), lh->L.s_last, sizeof(long long) * h->n, cudaMemcpyDeviceToHost), "copy scores");
-        std::vector<float> t(h->n);
-        const double sc = 1.0 / (1.0 + (double)lh->h_lc->smax);
-        for (int j = 0; j < h->n; ++j) t[j] = (float)((double)sl[j] * sc);
-        LCK(h, cudaMemcpy(target, t.data(), sizeof(float) * h->n, cudaMemcpyHostToDevice), "copy targets");
+        k_targets<<<grid_n(h->n, 256), 256, 0, h->st>>>(h->n, lh->L, target);
+        LCK(h, cudaGetLastError(), "targets");
     }
     LCK(h, cudaStreamSynchronize(h->st), "synchronise");
     return CHAP_OK;
@@ -1023,8 +1138,13 @@ chap_status chap_mlp_forward(const uint16_t *weights, const uint16_t *x, int64_t
     if (!weights || !x || !y || n < 0) return CHAP_E_INVALID;
     if (n == 0) return CHAP_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    k_mlp_forward<<<grid_n(n, 256, 152 * 4), 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16 *>(weights),
-                                                           reinterpret_cast<const __nv_bfloat16 *>(x), n, y, nullptr);
+    if (mlp_smem_limit((const void *)k_mlp_forward, 0, (int)sizeof(MlpTile)) != cudaSuccess) {
+        cudaGetLastError();
+        return CHAP_E_CUDA;
+    }
+    const long long tiles = (n + kTileRows - 1) / kTileRows;
+    k_mlp_forward<<<(unsigned)std::min<long long>(tiles, 152 * 4), kTileThreads, sizeof(MlpTile), st>>>(
+        reinterpret_cast<const __nv_bfloat16 *>(weights), reinterpret_cast<const __nv_bfloat16 *>(x), n, y);
     return cudaGetLastError() == cudaSuccess ? CHAP_OK : CHAP_E_CUDA;
 }
 
@@ -1033,19 +1153,14 @@ chap_status chap_mlp_loss_grad(const uint16_t *weights, const uint16_t *x, const
 {
     if (!weights || !x || !target || !grad || !loss || n < 1) return CHAP_E_INVALID;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int smem = (int)sizeof(float) * (((kNParams + 3) & ~3) + kGradRows * kF + 2 * kGradRows * kHPad + kGradRows);
-    static bool attr = false;
-    if (!attr) {
-        if (cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
-            cudaGetLastError();
-            return CHAP_E_CUDA;
-        }
-        attr = true;
+    if (mlp_smem_limit((const void *)k_mlp_grad, 1, (int)sizeof(MlpGradTile)) != cudaSuccess) {
+        cudaGetLastError();
+        return CHAP_E_CUDA;
     }
-    const long long tiles = (n + kGradRows - 1) / kGradRows;
-    k_mlp_grad<<<(unsigned)tiles, kGradRows, smem, st>>>(reinterpret_cast<const __nv_bfloat16 *>(weights),
-                                                         reinterpret_cast<const __nv_bfloat16 *>(x), target, n,
-                                                         2.0f / (float)n, grad, loss);
+    const long long tiles = (n + kTileRows - 1) / kTileRows;
+    k_mlp_grad<<<(unsigned)std::min<long long>(tiles, 152 * 2), kTileThreads, sizeof(MlpGradTile), st>>>(
+        reinterpret_cast<const __nv_bfloat16 *>(weights), reinterpret_cast<const __nv_bfloat16 *>(x), target, n,
+        2.0f / (float)n, grad, loss);
     return cudaGetLastError() == cudaSuccess ? CHAP_OK : CHAP_E_CUDA;
 }
 
