@@ -485,7 +485,20 @@ int nb_grid_size(int ncols, int G);
 int nb_lanes(int ncols, int G);       // lanes per short non-binary column, from G on
 cudaError_t launch_eval_gated(const Dev &d, const LaunchPlan &p, const VarOut &o, int gate, cudaStream_t st);
 cudaError_t launch_select_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st);
-cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st);
+#ifdef __CUDACC__
+// Chained kernels of one stream: chain_next lets the next kernel be placed while
+// this one runs, chain_wait (the first thing the next one does, before it reads
+// or writes anything an earlier kernel touches) holds it until the one before
+// has finished and its writes are visible.  Both do nothing in a kernel that is
+// launched without the attribute.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+
+// chained: the two kernels are launched as dependents of the kernel before them
+// (chain_wait below), which then has to be one that every earlier kernel they
+// read from precedes in the stream.
+cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st, bool chained = false);
 cudaError_t launch_set_move(const Dev &d, int var, double new_value, cudaStream_t st);
 cudaError_t launch_residuals(const Dev &d, const int *w, cudaStream_t st);
 cudaError_t launch_finish_set_state(const Dev &d, long long iter, long long best_nviol, int use_best, cudaStream_t st);

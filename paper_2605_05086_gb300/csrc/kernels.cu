@@ -2970,6 +2970,8 @@ __device__ __forceinline__ void snapshot_x(const Dev &d)
 // columns); the last of them finishes the iteration.
 __global__ void __launch_bounds__(kApplyMoveThreads) k_apply_move(Dev d, int gate)
 {
+    chain_next();
+    chain_wait();
     if (gated_done(d, gate)) return;
     Ctl *c = d.ctl;
     const int var = c->mv_var;
@@ -3039,6 +3041,8 @@ __global__ void __launch_bounds__(kApplyMoveThreads) k_apply_move(Dev d, int gat
 // iteration.
 __global__ void __launch_bounds__(kApplyThreads) k_apply_bump(Dev d, int gate)
 {
+    chain_next();
+    chain_wait();
     if (gated_done(d, gate)) return;
     Ctl *c = d.ctl;
     if (c->mv_var >= 0) return;
@@ -3623,10 +3627,23 @@ cudaError_t launch_select_gated(const Dev &d, const LaunchPlan &p, int gate, cud
     return e;
 }
 
-cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st)
+cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st, bool chained)
 {
-    k_apply_move<<<p.apply_move_blocks, kApplyMoveThreads, 0, st>>>(d, gate);
-    k_apply_bump<<<p.apply_blocks, kApplyThreads, 0, st>>>(d, gate);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)p.apply_move_blocks);
+    cfg.blockDim = dim3(kApplyMoveThreads);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = chained ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_apply_move, d, gate);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3((unsigned)p.apply_blocks);
+    cfg.blockDim = dim3(kApplyThreads);
+    e = cudaLaunchKernelEx(&cfg, k_apply_bump, d, gate);
+    if (e != cudaSuccess) return e;
     if (p.lazy) k_lazy_mark<<<p.lazy_mark_blocks, kEvalThreads, 0, st>>>(d, p.bin_cols);
     return cudaGetLastError();
 }

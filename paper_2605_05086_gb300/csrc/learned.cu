@@ -13,6 +13,7 @@
 // that hands the chosen move to the apply kernel of the exact path.
 #include "chap_handle.h"
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -25,6 +26,8 @@
 namespace chap {
 namespace {
 
+namespace cg = cooperative_groups;
+
 #define FULLMASK 0xffffffffu
 
 constexpr int kF = 12, kH = 64;
@@ -33,8 +36,11 @@ constexpr int kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH, kNParams = kOffB3 + 1;
 constexpr int kTileRows = 64;        // rows of one network tile
 constexpr int kTileThreads = 256;    // threads of its CTA: 4 rows x 4 columns of a layer each
 constexpr int kTPad = kTileRows + 4; // rows of a transposed activation, padded (16-byte aligned, 17 x 16 bytes)
-constexpr int kTopkPerThread = 4;
-constexpr int kTopkBlock = 256 * kTopkPerThread;
+constexpr int kPropThreads = 128;    // proposal scores: 4 warps of 32 variables
+constexpr int kTkThreads = 1024;     // top-k: threads of a CTA of the cluster
+constexpr int kTkCtas = 16;          // its largest cluster
+constexpr int kTkKeys = 1024;        // keys of a warp kept in shared memory
+constexpr int kTkSmem = (kTkThreads / 32) * kTkKeys * (int)sizeof(unsigned);
 constexpr int kVarBits = 22;
 
 // Device state of the learned driver of one handle.
@@ -43,10 +49,7 @@ struct __align__(16) LearnCtl {
     long long smax;             // max |score| at the last exact pass
     long long passes, misses;   // exact passes and top-1 misses
     long long pass_iter;        // iteration of the last exact pass
-    unsigned prefix;            // radix select: digits fixed so far
-    int need;                   // elements still to take at the current digit
-    unsigned thr;               // k-th largest key
-    int total_gt;
+    unsigned ticket;            // CTAs of the subset kernel that are done
 };
 
 struct Learn {
@@ -55,11 +58,11 @@ struct Learn {
     long long *s_last;            // exact scores of the last pass [n]
     __nv_bfloat16 *feat;          // [n x 12]
     float *y;                     // predictions [n]
-    unsigned *hist;               // 2048 bins
-    int *bcnt, *bpre;             // per-block counts / prefixes (2 x nblocks each)
+    uint2 *fixed;                 // features 8..11 of each variable [n]: they never change
+    unsigned *hist;               // 3 x 2048 bins, zero between selections
+    int *bcnt;                    // per-CTA counts of the selection [2 x kTkCtas]
     int *list;                    // selected variables [k]
     LearnCtl *lc;
-    int nblocks;
 };
 
 __device__ __forceinline__ unsigned long long lglobal_ns()
@@ -81,9 +84,12 @@ __device__ __forceinline__ bool dbl_neg_bits(long long b) { return b < 0; }
 // ---------------------------------------------------------------- features
 
 // Column features recorded at an exact pass: share of violated halves and the
-// weighted (w |a|) share, one thread per variable.
+// weighted (w |a|) share, one thread per variable, and the largest |score|
+// (one atomic per CTA: one per variable on the same word was most of the
+// kernel, 132 us for 200k variables 13 without it).
 __global__ void k_refresh(Dev d, Learn L)
 {
+    unsigned long long top = 0;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x) {
         const int q = d.vpos[j];
         int halves = 0, viol = 0;
@@ -111,7 +117,16 @@ __global__ void k_refresh(Dev d, Learn L)
         L.colviol[j] = halves ? (float)viol / (float)halves : 0.0f;
         L.colwv[j] = wall > 0.0f ? wviol / wall : 0.0f;
         const long long sa = L.s_last[j] < 0 ? -L.s_last[j] : L.s_last[j];
-        if (sa > 0) atomicMax(reinterpret_cast<unsigned long long *>(&L.lc->smax), (unsigned long long)sa);
+        top = max(top, (unsigned long long)sa);
+    }
+    __shared__ unsigned long long s_top[8];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(FULLMASK, top, o));
+    if ((threadIdx.x & 31) == 0) s_top[threadIdx.x >> 5] = top;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < (int)blockDim.x / 32; ++i) top = max(top, s_top[i]);
+        if (top) atomicMax(reinterpret_cast<unsigned long long *>(&L.lc->smax), top);
     }
 }
 
@@ -122,42 +137,83 @@ __global__ void k_refresh_begin(Dev d, Learn L, int gate)
     L.lc->pass_iter = d.ctl->iter;
 }
 
-// The 12 features of every variable (BF16): x/(u-l), (x-l)/(u-l), (u-x)/(u-l),
-// min(tabu age, 64)/64, violated share, violated weighted share, last exact
-// score / (1 + max |score|), iterations since the exact pass / 50,
+// The 12 features of variable j, rounded to BF16: x/(u-l), (x-l)/(u-l),
+// (u-x)/(u-l), min(tabu age, 64)/64, violated share, violated weighted share,
+// last exact score / (1 + max |score|), iterations since the exact pass / 50,
 // log2(1 + column length)/16, is_binary, is_integer, c_j / max |c|.
-__global__ void k_features(Dev d, Learn L, float cmax, int gate)
+//
+// The last four do not change: they are laid out once with the driver's state
+// (column length through two gathers per variable, 19 us of each proposal over
+// 200k variables, with the others, when each formed them).
+__global__ void k_fixed_features(Dev d, Learn L, float cmax)
 {
-    if (gate && done_gate(d)) return;
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x) {
+        const int q = d.vpos[j];
+        const int len = (d.ci_ptr[q + 1] - d.ci_ptr[q]) + (d.cf_ptr[q + 1] - d.cf_ptr[q]);
+        const int vt = d.vtype[j];
+        const float f8 = log2f(1.0f + (float)len) / 16.0f;
+        const float f9 = vt == kVarBin ? 1.0f : 0.0f, f10 = vt == kVarInt ? 1.0f : 0.0f;
+        const float f11 = cmax > 0.0f ? (float)d.obj[j] / cmax : 0.0f;
+        const __nv_bfloat162 a = __floats2bfloat162_rn(f8, f9), b = __floats2bfloat162_rn(f10, f11);
+        L.fixed[j] = make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
+    }
+}
+
+struct VarRaw {
+    double x, l, u;
+    long long s;
+    int ti, td;
+    float cv, cw;
+    uint2 fx;
+};
+
+__device__ __forceinline__ VarRaw var_load(const Dev &d, const Learn &L, int j)
+{
+    VarRaw v;
+    v.x = d.x[j]; v.l = d.lb[j]; v.u = d.ub[j];
+    v.s = L.s_last[j];
+    v.ti = d.tabu_inc[j]; v.td = d.tabu_dec[j];
+    v.cv = L.colviol[j]; v.cw = L.colwv[j];
+    v.fx = L.fixed[j];
+    return v;
+}
+
+__device__ __forceinline__ void var_features(const VarRaw &v, int tenure, long long iter, float smax, float since,
+                                             __nv_bfloat162 (&out)[kF / 2])
+{
+    const bool fin = isfinite(v.u - v.l) && v.u > v.l;
+    const float w = fin ? (float)(v.u - v.l) : 1.0f;
+    float f[8];
+    f[0] = fin ? (float)v.x / w : 0.0f;
+    f[1] = fin ? (float)(v.x - v.l) / w : 0.0f;
+    f[2] = fin ? (float)(v.u - v.x) / w : 0.0f;
+    const int st = v.ti > v.td ? v.ti : v.td;
+    long long age = st > 0 ? iter - (long long)(st - 1 - tenure) : 64;
+    if (age > 64) age = 64;
+    f[3] = (float)age / 64.0f;
+    f[4] = v.cv;
+    f[5] = v.cw;
+    f[6] = (float)v.s / (1.0f + smax);
+    f[7] = since / 50.0f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) out[i] = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+    out[4] = *reinterpret_cast<const __nv_bfloat162 *>(&v.fx.x);
+    out[5] = *reinterpret_cast<const __nv_bfloat162 *>(&v.fx.y);
+}
+
+__global__ void k_features(Dev d, Learn L)
+{
     const long long iter = d.ctl->iter;
     const float smax = (float)L.lc->smax;
     const float since = (float)(iter - L.lc->pass_iter);
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x) {
-        const double x = d.x[j], l = d.lb[j], u = d.ub[j];
-        const bool fin = isfinite(u - l) && u > l;
-        const float w = fin ? (float)(u - l) : 1.0f;
-        float f[kF];
-        f[0] = fin ? (float)x / w : 0.0f;
-        f[1] = fin ? (float)(x - l) / w : 0.0f;
-        f[2] = fin ? (float)(u - x) / w : 0.0f;
-        const int ti = d.tabu_inc[j], td = d.tabu_dec[j];
-        const int st = ti > td ? ti : td;
-        long long age = st > 0 ? iter - (long long)(st - 1 - d.tenure) : 64;
-        if (age > 64) age = 64;
-        f[3] = (float)age / 64.0f;
-        f[4] = L.colviol[j];
-        f[5] = L.colwv[j];
-        f[6] = (float)L.s_last[j] / (1.0f + smax);
-        f[7] = since / 50.0f;
-        const int q = d.vpos[j];
-        const int len = (d.ci_ptr[q + 1] - d.ci_ptr[q]) + (d.cf_ptr[q + 1] - d.cf_ptr[q]);
-        f[8] = log2f(1.0f + (float)len) / 16.0f;
-        const int vt = d.vtype[j];
-        f[9] = vt == kVarBin ? 1.0f : 0.0f;
-        f[10] = vt == kVarInt ? 1.0f : 0.0f;
-        f[11] = cmax > 0.0f ? (float)d.obj[j] / cmax : 0.0f;
+        __nv_bfloat162 f[kF / 2];
+        var_features(var_load(d, L, j), d.tenure, iter, smax, since, f);
+        // a row is 24 bytes, 8-byte aligned
+        uint2 *out = reinterpret_cast<uint2 *>(L.feat + (long long)j * kF);
+        const uint2 *in = reinterpret_cast<const uint2 *>(f);
 #pragma unroll
-        for (int k = 0; k < kF; ++k) L.feat[(long long)j * kF + k] = __float2bfloat16_rn(f[k]);
+        for (int k = 0; k < kF / 4; ++k) out[k] = in[k];
     }
 }
 
@@ -270,61 +326,164 @@ __global__ void __launch_bounds__(kTileThreads) k_mlp_forward(const __nv_bfloat1
     }
 }
 
-// Forward pass with the second layer on the tensor cores: one warp per tile of
-// 16 rows; every lane computes, in FP32 on the CUDA cores, exactly the
-// first-layer activations its A fragments of mma.m16n8k16 need (rows g and
-// g + 8 of the tile, 16 hidden units per 16-wide K chunk), rounds them to BF16,
-// and the warp multiplies the 16 x 64 tile by W2 (64 x 64, BF16 from shared
-// memory) into FP32 accumulators; the output layer is reduced across the four
-// lanes that share a row.  Activations of the first layer are BF16 here
-// (FP32 in k_mlp_forward and in training).
-__global__ void __launch_bounds__(256) k_mlp_forward_tc(const __nv_bfloat16 *w, const __nv_bfloat16 *x, long long n,
-                                                        float *y, const int *done)
+// Order-preserving bits of a float.
+__device__ __forceinline__ unsigned fkey(float v)
 {
-    if (done && *(volatile const int *)done) return;
-    __shared__ float s1[kF * kH + kH];                          // W1, b1
-    __shared__ float s2[kH + kH + 1];                           // b2, w3, b3
-    __shared__ __align__(16) unsigned short sW2t[kH * (kH + 8)];  // W2 transposed, [n][k], padded rows
-    for (int i = threadIdx.x; i < kF * kH + kH; i += blockDim.x) s1[i] = __bfloat162float(w[kOffW1 + i]);
-    for (int i = threadIdx.x; i < 2 * kH + 1; i += blockDim.x) s2[i] = __bfloat162float(w[kOffB2 + i]);
-    const unsigned short *wraw = reinterpret_cast<const unsigned short *>(w);
-    for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) {
-        const int k = i / kH, nn = i % kH;                      // W2[k][nn]
-        sW2t[nn * (kH + 8) + k] = wraw[kOffW2 + i];
+    const unsigned b = __float_as_uint(v);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+
+// The digit of the `need`-th largest key, from a histogram of it over the keys
+// that match the digits before (a block-wide suffix scan, two bins a thread);
+// need becomes its rank among the keys of that digit.
+__device__ __forceinline__ int topk_pick(const unsigned *hist, int &need)
+{
+    __shared__ int wsum[kTkThreads / 32];
+    __shared__ int s_dig, s_need;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // thread t owns bins 2047 - 2t and 2046 - 2t: higher bins first
+    const uint2 v = __ldcg(reinterpret_cast<const uint2 *>(hist) + 1023 - threadIdx.x);
+    const int c0 = (int)v.y, tot = c0 + (int)v.x;
+    int incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(FULLMASK, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[wid] = incl;
+    __syncthreads();
+    const int ws = wsum[lane];
+    const int before = incl - tot + __reduce_add_sync(FULLMASK, lane < wid ? ws : 0);
+    if (before < need && before + tot >= need) {
+        const bool first = before + c0 >= need;
+        s_dig = 2047 - 2 * (int)threadIdx.x - (first ? 0 : 1);
+        s_need = need - before - (first ? 0 : c0);
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const long long tiles = (n + 15) / 16;
-    for (long long tile = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); tile < tiles;
-         tile += (long long)gridDim.x * (blockDim.x >> 5)) {
-        const long long r0 = tile * 16 + g, r1 = r0 + 8;
-        float x0[kF], x1[kF];
+    need = s_need;
+    return s_dig;
+}
+
+// True in the CTA that is the last of the grid to get here (all threads call
+// it; what the others wrote before is visible to it).
+__device__ bool last_cta(const Learn &L)
+{
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&L.lc->ticket, 1u) == gridDim.x - 1;
+        if (s_last) L.lc->ticket = 0u;
+    }
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last != 0;
+}
+
+// Features and predictions of every variable, with the first histogram of the
+// top-k: the forward pass with the second layer on the tensor cores.  A warp
+// takes 32 variables: each lane forms one variable's features (BF16, kept in
+// shared memory), then for the two 16-row tiles together every lane computes, in
+// FP32 on the CUDA cores, exactly the first-layer activations its A fragments of
+// mma.m16n8k16 need (rows g and g + 8 of a tile, 16 hidden units per 16-wide K
+// chunk; the 12 weights of a unit are three 16-byte loads for 4 rows), rounds
+// them to BF16, and the warp multiplies the tiles by W2 (64 x 64, BF16 from
+// shared memory, one fragment load for both) into FP32 accumulators; the output
+// layer is reduced across the four lanes that share a row.  Activations of the
+// first layer are BF16 here (FP32 in k_mlp_forward and in training).  Bound by
+// the operand loads from shared memory and the first layer's FMAs; the next
+// group's inputs are loaded under this one's arithmetic.  200k variables: 27 us,
+// against 49 as three kernels (features 19, forward 25 one tile at a time,
+// histogram 5).
+__global__ void __launch_bounds__(kPropThreads, 3) k_propose_scores(Dev d, Learn L, const __nv_bfloat16 *w, int gate)
+{
+    constexpr int kPadF = kF + 4;                               // padded feature rows
+    __shared__ __align__(16) float s1[kH * kF + kH];            // W1 by hidden unit ([c][f]), b1
+    __shared__ float s2[kH + kH + 1];                           // b2, w3, b3
+    __shared__ __align__(16) unsigned short sW2t[kH * (kH + 8)];  // W2 transposed, [n][k], padded rows
+    __shared__ __align__(16) float sx[kPropThreads / 32][32 * kPadF];  // features of each warp's 32 variables
+    __shared__ unsigned h[2048];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int n = d.n, groups = (n + 31) / 32, step = gridDim.x * (kPropThreads / 32);
+    int gr = blockIdx.x * (kPropThreads / 32) + warp;
+    chain_next();
+    // the weights do not depend on the kernel before
+    for (int i = threadIdx.x; i < kF * kH; i += blockDim.x) s1[(i % kH) * kF + i / kH] = __bfloat162float(w[kOffW1 + i]);
+    for (int i = threadIdx.x; i < kH; i += blockDim.x) s1[kF * kH + i] = __bfloat162float(w[kOffB1 + i]);
+    for (int i = threadIdx.x; i < 2 * kH + 1; i += blockDim.x) s2[i] = __bfloat162float(w[kOffB2 + i]);
+    for (int i = threadIdx.x; i < 2048; i += blockDim.x) h[i] = 0u;
+    const unsigned short *wraw = reinterpret_cast<const unsigned short *>(w);
+#pragma unroll 8
+    for (int i = threadIdx.x; i < kH * kH; i += kPropThreads) {
+        const int kk = i / kH, nn = i % kH;                     // W2[kk][nn]
+        sW2t[nn * (kH + 8) + kk] = wraw[kOffW2 + i];
+    }
+    chain_wait();
+    if (gate && done_gate(d)) return;
+    __syncthreads();
+    VarRaw raw = var_load(d, L, min(gr * 32 + lane, n - 1));
+    const long long iter = d.ctl->iter;
+    const float smax = (float)L.lc->smax;
+    const float since = (float)(iter - L.lc->pass_iter);
+    float *xw = sx[warp];
+    for (; gr < groups; gr += step) {
+        {
+            __nv_bfloat162 f[kF / 2];
+            var_features(raw, d.tenure, iter, smax, since, f);
+            __syncwarp();
 #pragma unroll
-        for (int f = 0; f < kF; ++f) {
-            x0[f] = r0 < n ? __bfloat162float(x[r0 * kF + f]) : 0.0f;
-            x1[f] = r1 < n ? __bfloat162float(x[r1 * kF + f]) : 0.0f;
+            for (int i = 0; i < kF / 2; i += 2) {
+                const float2 a = __bfloat1622float2(f[i]), b = __bfloat1622float2(f[i + 1]);
+                *reinterpret_cast<float4 *>(xw + lane * kPadF + 2 * i) = make_float4(a.x, a.y, b.x, b.y);
+            }
+            __syncwarp();
         }
-        float acc[8][4];
+        // the next group's loads run under this one's arithmetic
+        raw = var_load(d, L, min((int)min((long long)gr + step, (long long)groups - 1) * 32 + lane, n - 1));
+        // rows g, g + 8 (first tile), g + 16, g + 24 (second)
+        float x[4][kF];
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
+            for (int i = 0; i < kF; i += 4) {
+                const float4 a = *reinterpret_cast<const float4 *>(xw + (8 * r + g) * kPadF + i);
+                x[r][i] = a.x; x[r][i + 1] = a.y; x[r][i + 2] = a.z; x[r][i + 3] = a.w;
+            }
+        float acc[2][8][4];
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[0][nt][e] = acc[1][nt][e] = 0.0f;
+#pragma unroll 1
         for (int kc = 0; kc < 4; ++kc) {
-            // A fragment: rows g / g+8, hidden units 16 kc + {2t, 2t+1, 2t+8, 2t+9}
-            unsigned a[4];
+            // A fragments: hidden units 16 kc + {2t, 2t+1} and {2t+8, 2t+9}
+            unsigned a[2][4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = 16 * kc + 2 * t + (q >= 2 ? 8 : 0);
-                const float *xr = (q & 1) ? x1 : x0;
-                float v[2];
+            for (int half = 0; half < 2; ++half) {
+                float v[4][2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    float s = s1[kF * kH + c + e];
+                    const int c = 16 * kc + 2 * t + 8 * half + e;
+                    const float b = s1[kF * kH + c];
 #pragma unroll
-                    for (int f = 0; f < kF; ++f) s = __fmaf_rn(xr[f], s1[f * kH + c + e], s);
-                    v[e] = fmaxf(s, 0.0f);
+                    for (int r = 0; r < 4; ++r) v[r][e] = b;
+#pragma unroll
+                    for (int i = 0; i < kF; i += 4) {
+                        const float4 wv = *reinterpret_cast<const float4 *>(s1 + c * kF + i);
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            v[r][e] = __fmaf_rn(x[r][i], wv.x, v[r][e]);
+                            v[r][e] = __fmaf_rn(x[r][i + 1], wv.y, v[r][e]);
+                            v[r][e] = __fmaf_rn(x[r][i + 2], wv.z, v[r][e]);
+                            v[r][e] = __fmaf_rn(x[r][i + 3], wv.w, v[r][e]);
+                        }
+                    }
                 }
-                const __nv_bfloat162 pr = __floats2bfloat162_rn(v[0], v[1]);
-                a[q] = *reinterpret_cast<const unsigned *>(&pr);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const __nv_bfloat162 pr = __floats2bfloat162_rn(fmaxf(v[r][0], 0.0f), fmaxf(v[r][1], 0.0f));
+                    a[r >> 1][(r & 1) + 2 * half] = *reinterpret_cast<const unsigned *>(&pr);
+                }
             }
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
@@ -332,32 +491,49 @@ __global__ void __launch_bounds__(256) k_mlp_forward_tc(const __nv_bfloat16 *w, 
                 const unsigned short *bp = sW2t + (8 * nt + g) * (kH + 8) + 16 * kc + 2 * t;
                 const unsigned b0 = *reinterpret_cast<const unsigned *>(bp);
                 const unsigned b1 = *reinterpret_cast<const unsigned *>(bp + 8);
-                asm volatile(
-                    "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-                    "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                    : "+f"(acc[nt][0]), "+f"(acc[nt][1]), "+f"(acc[nt][2]), "+f"(acc[nt][3])
-                    : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+                    asm volatile(
+                        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+                        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                        : "+f"(acc[m][nt][0]), "+f"(acc[m][nt][1]), "+f"(acc[m][nt][2]), "+f"(acc[m][nt][3])
+                        : "r"(a[m][0]), "r"(a[m][1]), "r"(a[m][2]), "r"(a[m][3]), "r"(b0), "r"(b1));
             }
         }
-        // output layer: rows g (acc[.][0..1]) and g + 8 (acc[.][2..3]), columns 8 nt + 2t (+1)
-        float o0 = 0.0f, o1 = 0.0f;
+        // output layer: rows g (acc[.][.][0..1]) and g + 8 (acc[.][.][2..3]) of a tile, columns 8 nt + 2t (+1)
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int c = 8 * nt + 2 * t;
-            o0 = __fmaf_rn(fmaxf(acc[nt][0] + s2[c], 0.0f), s2[kH + c], o0);
-            o0 = __fmaf_rn(fmaxf(acc[nt][1] + s2[c + 1], 0.0f), s2[kH + c + 1], o0);
-            o1 = __fmaf_rn(fmaxf(acc[nt][2] + s2[c], 0.0f), s2[kH + c], o1);
-            o1 = __fmaf_rn(fmaxf(acc[nt][3] + s2[c + 1], 0.0f), s2[kH + c + 1], o1);
-        }
-        o0 += __shfl_xor_sync(FULLMASK, o0, 1);
-        o0 += __shfl_xor_sync(FULLMASK, o0, 2);
-        o1 += __shfl_xor_sync(FULLMASK, o1, 1);
-        o1 += __shfl_xor_sync(FULLMASK, o1, 2);
-        if (t == 0) {
-            if (r0 < n) y[r0] = o0 + s2[2 * kH];
-            if (r1 < n) y[r1] = o1 + s2[2 * kH];
+        for (int m = 0; m < 2; ++m) {
+            float o0 = 0.0f, o1 = 0.0f;
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt) {
+                const int c = 8 * nt + 2 * t;
+                o0 = __fmaf_rn(fmaxf(acc[m][nt][0] + s2[c], 0.0f), s2[kH + c], o0);
+                o0 = __fmaf_rn(fmaxf(acc[m][nt][1] + s2[c + 1], 0.0f), s2[kH + c + 1], o0);
+                o1 = __fmaf_rn(fmaxf(acc[m][nt][2] + s2[c], 0.0f), s2[kH + c], o1);
+                o1 = __fmaf_rn(fmaxf(acc[m][nt][3] + s2[c + 1], 0.0f), s2[kH + c + 1], o1);
+            }
+            o0 += __shfl_xor_sync(FULLMASK, o0, 1);
+            o0 += __shfl_xor_sync(FULLMASK, o0, 2);
+            o1 += __shfl_xor_sync(FULLMASK, o1, 1);
+            o1 += __shfl_xor_sync(FULLMASK, o1, 2);
+            const int r0 = gr * 32 + 16 * m + g, r1 = r0 + 8;
+            if (t == 0) {
+                if (r0 < n) {
+                    const float y = o0 + s2[2 * kH];
+                    L.y[r0] = y;
+                    atomicAdd(&h[fkey(y) >> 21], 1u);
+                }
+                if (r1 < n) {
+                    const float y = o1 + s2[2 * kH];
+                    L.y[r1] = y;
+                    atomicAdd(&h[fkey(y) >> 21], 1u);
+                }
+            }
         }
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2048; i += blockDim.x)
+        if (h[i]) atomicAdd(&L.hist[i], h[i]);
 }
 
 // Gradient of the mean squared error over n rows (scale 2/n), accumulated into
@@ -365,9 +541,9 @@ __global__ void __launch_bounds__(256) k_mlp_forward_tc(const __nv_bfloat16 *w, 
 // per parameter and CTA).  A CTA takes tiles of kTileRows rows in turn, keeps
 // its share of the gradient in registers (16 weights of the second layer, 3 of
 // the first per thread) and adds it once at the end.  Bound by the FP32 FMAs
-// (0.9M a tile) and their shared-memory operands.  A training step (forward,
-// gradient, Adam, read of the loss) of 8 x 8,192 rows takes 405 us; with one row
-// per thread and one parameter per thread and pass it took 697.
+// (0.9M a tile) and their shared-memory operands.  8 training steps of
+// 8,192 rows and a forward pass of 100,003 take 370 us; with one row per thread
+// and one parameter per thread and pass they took 697.
 struct MlpGradTile {
     MlpTile f;
     float w2T[kH * kH];          // second layer transposed, [j][i]
@@ -526,173 +702,95 @@ __global__ void k_adam(float *w32, __nv_bfloat16 *wbf, float *m, float *v, float
 
 // ------------------------------------------------------------------- top-k
 
-__device__ __forceinline__ unsigned fkey(float v)
+// The variables with the k largest predictions, ties by the lower index, in
+// index order (above the k-th value first, then those equal to it): a radix
+// select over the order-preserving keys in one cluster.  The first digit (bits
+// 31..21) is counted where the predictions are made; a warp owns a run of
+// consecutive keys, keeps the first kTkKeys of it in shared memory and counts
+// the second (bits 20..10) and third digit (bits 9..0) of those that match, then
+// the keys above and equal, then writes.  Bound by its three cluster-wide
+// barriers and the L2 round trip of the counts around each; 18 us for
+// 200k variables (cold cache) against 44 with a launch over the whole GPU for
+// each step.
+__global__ void __launch_bounds__(kTkThreads) k_topk(Dev d, Learn L, int n, int k, int gate)
 {
-    const unsigned b = __float_as_uint(v);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-// Histogram of one digit of the keys that match the digits fixed so far.
-// level 0: bits 31..21, level 1: bits 20..10, level 2: bits 9..0.
-__global__ void k_topk_hist(Dev d, Learn L, const float *y, int n, int level, int gate)
-{
+    chain_next();
+    chain_wait();
     if (gate && done_gate(d)) return;
+    extern __shared__ unsigned tk_keys[];
     __shared__ unsigned h[2048];
-    for (int i = threadIdx.x; i < 2048; i += blockDim.x) h[i] = 0u;
-    __syncthreads();
-    const unsigned prefix = L.lc->prefix;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const unsigned k = fkey(y[j]);
-        bool match;
-        unsigned dig;
-        if (level == 0) { match = true; dig = k >> 21; }
-        else if (level == 1) { match = (k >> 21) == (prefix >> 21); dig = (k >> 10) & 0x7ffu; }
-        else { match = (k >> 10) == (prefix >> 10); dig = k & 0x3ffu; }
-        if (match) atomicAdd(&h[dig], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 2048; i += blockDim.x)
-        if (h[i]) atomicAdd(&L.hist[i], h[i]);
-}
-
-// Fix the digit of this level: the largest digit whose count from the top
-// reaches the elements still needed (a block-wide suffix scan of the 2048
-// bins); clears the histogram for the next level.
-__global__ void __launch_bounds__(256) k_topk_pick(Dev d, Learn L, int level, int k, int n, int gate)
-{
-    if (gate && done_gate(d)) return;
-    constexpr int PER = 2048 / 256;
-    __shared__ int wsum[8];
-    __shared__ int s_dig, s_need;
-    LearnCtl *c = L.lc;
-    const int need0 = level == 0 ? min(k, n) : c->need;
-    const int nb = level == 2 ? 1024 : 2048;
-    // thread t owns bins [2048 - (t+1) PER, 2048 - t PER): higher bins first
-    const int hi = 2048 - threadIdx.x * PER;
-    int cnt[PER];
-    int tot = 0;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int b = hi - 1 - u;
-        cnt[u] = b < nb ? (int)L.hist[b] : 0;
-        tot += cnt[u];
-    }
-    // exclusive prefix of the per-thread totals in thread order (= from the top)
+    __shared__ int sg[kTkThreads / 32], se[kTkThreads / 32];
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)gridDim.x, rank = (int)blockIdx.x;   // the grid is one cluster
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int incl = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(FULLMASK, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) wsum[wid] = incl;
-    if (threadIdx.x == 0) { s_dig = 0; s_need = need0; }
-    __syncthreads();
-    int before = incl - tot;
-    for (int w = 0; w < wid; ++w) before += wsum[w];
-    // the thread whose range contains the need0-th element from the top fixes the digit
-    if (before < need0 && before + tot >= need0) {
-        int acc = before;
-        for (int u = 0; u < PER; ++u) {
-            if (acc + cnt[u] >= need0) { s_dig = hi - 1 - u; s_need = need0 - acc; break; }
-            acc += cnt[u];
-        }
+    const int nw = C * (kTkThreads / 32);
+    const int chunk = ((n + nw - 1) / nw + 31) & ~31;
+    const long long lo = (long long)(rank * (kTkThreads / 32) + wid) * chunk;
+    const int j0 = (int)(lo < n ? lo : n), cnt = min(chunk, n - j0);
+    unsigned *kw = tk_keys + wid * kTkKeys;
+    auto key_at = [&](int i) { return i < kTkKeys ? kw[i] : fkey(__ldcg(L.y + j0 + i)); };
+    for (int i = threadIdx.x; i < 2048; i += kTkThreads) h[i] = 0u;
+#pragma unroll 8
+    for (int i = lane; i < min(cnt, kTkKeys); i += 32) kw[i] = fkey(__ldcg(L.y + j0 + i));
+    int need = k;
+    unsigned prefix = (unsigned)topk_pick(L.hist, need);
+    for (int i = lane; i < cnt; i += 32) {
+        const unsigned key = key_at(i);
+        if (key >> 21 == prefix) atomicAdd(&h[(key >> 10) & 0x7ffu], 1u);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const int dig = s_dig;
-        c->need = s_need;
-        const unsigned p = level == 0 ? ((unsigned)dig << 21) : level == 1 ? (c->prefix | ((unsigned)dig << 10))
-                                                                           : (c->prefix | (unsigned)dig);
-        c->prefix = p;
-        if (level == 2) c->thr = p;
+    for (int i = threadIdx.x; i < 2048; i += kTkThreads) {
+        if (h[i]) atomicAdd(&L.hist[2048 + i], h[i]);
+        h[i] = 0u;
     }
-    for (int i = threadIdx.x; i < 2048; i += blockDim.x) L.hist[i] = 0u;
-}
-
-__global__ void __launch_bounds__(256) k_topk_count(Dev d, Learn L, const float *y, int n, int gate)
-{
-    if (gate && done_gate(d)) return;
-    const unsigned thr = L.lc->thr;
+    cl.sync();
+    // every CTA has read the first histogram: clear it for the next selection
+    if (rank == 0)
+        for (int i = threadIdx.x; i < 2048; i += kTkThreads) L.hist[i] = 0u;
+    prefix = (prefix << 11) | (unsigned)topk_pick(L.hist + 2048, need);
+    for (int i = lane; i < cnt; i += 32) {
+        const unsigned key = key_at(i);
+        if (key >> 10 == prefix) atomicAdd(&h[key & 0x3ffu], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 1024; i += kTkThreads)
+        if (h[i]) atomicAdd(&L.hist[4096 + i], h[i]);
+    cl.sync();
+    if (rank == 0)
+        for (int i = threadIdx.x; i < 2048; i += kTkThreads) L.hist[2048 + i] = 0u;
+    const unsigned thr = (prefix << 10) | (unsigned)topk_pick(L.hist + 4096, need);
     int gt = 0, eq = 0;
-    const int base = blockIdx.x * kTopkBlock + threadIdx.x * kTopkPerThread;
-    for (int u = 0; u < kTopkPerThread; ++u) {
-        const int j = base + u;
-        if (j < n) {
-            const unsigned k = fkey(y[j]);
-            gt += k > thr;
-            eq += k == thr;
-        }
+    for (int i = lane; i < chunk; i += 32) {
+        const unsigned key = i < cnt ? key_at(i) : 0u;
+        gt += __popc(__ballot_sync(FULLMASK, i < cnt && key > thr));
+        eq += __popc(__ballot_sync(FULLMASK, i < cnt && key == thr));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        gt += __shfl_xor_sync(FULLMASK, gt, o);
-        eq += __shfl_xor_sync(FULLMASK, eq, o);
-    }
-    __shared__ int sg[8], se[8];
-    if ((threadIdx.x & 31) == 0) { sg[threadIdx.x >> 5] = gt; se[threadIdx.x >> 5] = eq; }
+    if (lane == 0) { sg[wid] = gt; se[wid] = eq; }
     __syncthreads();
+    const int tg = __reduce_add_sync(FULLMASK, sg[lane]), te = __reduce_add_sync(FULLMASK, se[lane]);
+    int pg = __reduce_add_sync(FULLMASK, lane < wid ? sg[lane] : 0);
+    int pe = __reduce_add_sync(FULLMASK, lane < wid ? se[lane] : 0);
     if (threadIdx.x == 0) {
-        int a = 0, b = 0;
-        for (int w = 0; w < 8; ++w) { a += sg[w]; b += se[w]; }
-        L.bcnt[2 * blockIdx.x] = a;
-        L.bcnt[2 * blockIdx.x + 1] = b;
+        L.bcnt[2 * rank] = tg;
+        L.bcnt[2 * rank + 1] = te;
     }
-}
-
-__global__ void k_topk_scan(Dev d, Learn L, int gate)
-{
-    if (gate && done_gate(d)) return;
-    if (threadIdx.x != 0) return;
-    int a = 0, b = 0;
-    for (int i = 0; i < L.nblocks; ++i) {
-        L.bpre[2 * i] = a;
-        L.bpre[2 * i + 1] = b;
-        a += L.bcnt[2 * i];
-        b += L.bcnt[2 * i + 1];
-    }
-    L.lc->total_gt = a;
-}
-
-// Stable compaction: every key above the threshold, then the first `need`
-// keys equal to it in index order.
-__global__ void __launch_bounds__(256) k_topk_write(Dev d, Learn L, const float *y, int n, int gate)
-{
-    if (gate && done_gate(d)) return;
-    const unsigned thr = L.lc->thr;
-    const int need = L.lc->need, total_gt = L.lc->total_gt;
-    const int base = blockIdx.x * kTopkBlock + threadIdx.x * kTopkPerThread;
-    unsigned kk[kTopkPerThread];
-    int gt = 0, eq = 0;
-    for (int u = 0; u < kTopkPerThread; ++u) {
-        const int j = base + u;
-        kk[u] = j < n ? fkey(y[j]) : 0u;
-        gt += j < n && kk[u] > thr;
-        eq += j < n && kk[u] == thr;
-    }
-    // block exclusive scan of (gt, eq) in thread order
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int sgt = gt, seq = eq;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int a = __shfl_up_sync(FULLMASK, sgt, o), b = __shfl_up_sync(FULLMASK, seq, o);
-        if (lane >= o) { sgt += a; seq += b; }
-    }
-    __shared__ int wg[8], we[8];
-    if (lane == 31) { wg[wid] = sgt; we[wid] = seq; }
-    __syncthreads();
-    int og = 0, oe = 0;
-    for (int w = 0; w < wid; ++w) { og += wg[w]; oe += we[w]; }
-    int pg = L.bpre[2 * blockIdx.x] + og + sgt - gt;
-    int pe = L.bpre[2 * blockIdx.x + 1] + oe + seq - eq;
-    for (int u = 0; u < kTopkPerThread; ++u) {
-        const int j = base + u;
-        if (j >= n) break;
-        if (kk[u] > thr) L.list[pg++] = j;
-        else if (kk[u] == thr) {
-            if (pe < need) L.list[total_gt + pe] = j;
-            ++pe;
-        }
+    cl.sync();
+    if (rank == 0)
+        for (int i = threadIdx.x; i < 1024; i += kTkThreads) L.hist[4096 + i] = 0u;
+    const int cgt = lane < C ? __ldcg(L.bcnt + 2 * lane) : 0, ceq = lane < C ? __ldcg(L.bcnt + 2 * lane + 1) : 0;
+    const int total_gt = __reduce_add_sync(FULLMASK, cgt);
+    pg += __reduce_add_sync(FULLMASK, lane < rank ? cgt : 0);
+    pe += __reduce_add_sync(FULLMASK, lane < rank ? ceq : 0);
+    for (int i = lane; i < chunk; i += 32) {
+        const unsigned key = i < cnt ? key_at(i) : 0u;
+        const unsigned mg = __ballot_sync(FULLMASK, i < cnt && key > thr);
+        const unsigned me = __ballot_sync(FULLMASK, i < cnt && key == thr);
+        const unsigned below = (1u << lane) - 1u;
+        if (mg >> lane & 1u) L.list[pg + __popc(mg & below)] = j0 + i;
+        const int r = pe + __popc(me & below);
+        if ((me >> lane & 1u) && r < need) L.list[total_gt + r] = j0 + i;
+        pg += __popc(mg);
+        pe += __popc(me);
     }
 }
 
@@ -716,11 +814,37 @@ __device__ __forceinline__ long long flip_sign(long long b)
     return r;
 }
 
+// Hand the proposal's move to the apply kernel of the exact path.
+__device__ __forceinline__ void learn_select(const Dev &d, const Learn &L)
+{
+    Ctl *c = d.ctl;
+    const unsigned long long key = __ldcg(&L.lc->key);
+    L.lc->key = 0ull;
+    if (key != 0ull) {
+        const int j = (1 << kVarBits) - 1 - (int)(key & ((1ull << kVarBits) - 1));
+        const double x = d.x[j];
+        c->mv_var = j;
+        c->mv_s = (long long)(key >> kVarBits);
+        c->mv_dc = 0;
+        c->mv_old = x;
+        c->mv_new = d.vtype[j] == kVarBin ? (__double_as_longlong(x) == 0 ? 1.0 : 0.0) : L.xh[j];
+    } else {
+        c->mv_var = -1;
+        c->mv_s = 0;
+        c->mv_dc = 0;
+        c->mv_new = 0.0;
+        c->mv_old = 0.0;
+    }
+}
+
 // Flip score of every listed binary variable (8 lanes per variable, as the
 // exact binary kernel); the best admissible positive flip is folded into
 // lc->key with one 64-bit atomicMax (larger score, then lower variable).
-__global__ void __launch_bounds__(256) k_subset_eval(Dev d, Learn L, int k, int gate)
+// select: the last CTA hands the move to the apply kernel.
+__global__ void __launch_bounds__(256) k_subset_eval(Dev d, Learn L, int k, int select, int gate)
 {
+    chain_next();
+    chain_wait();
     if (gate && done_gate(d)) return;
     const int lane = threadIdx.x & 31, g = lane >> 3, sub = lane & 7;
     const long long iter = d.ctl->iter, nviol = d.ctl->nviol, bestnv = d.ctl->best_nviol;
@@ -797,30 +921,13 @@ __global__ void __launch_bounds__(256) k_subset_eval(Dev d, Learn L, int k, int 
             }
         }
     }
+    if (select && last_cta(L) && threadIdx.x == 0) learn_select(d, L);
 }
 
-// Hand the proposal's move to the apply kernel of the exact path.
 __global__ void k_learn_select(Dev d, Learn L, int gate)
 {
     if (gate && done_gate(d)) return;
-    Ctl *c = d.ctl;
-    const unsigned long long key = L.lc->key;
-    L.lc->key = 0ull;
-    if (key != 0ull) {
-        const int j = (1 << kVarBits) - 1 - (int)(key & ((1ull << kVarBits) - 1));
-        const double x = d.x[j];
-        c->mv_var = j;
-        c->mv_s = (long long)(key >> kVarBits);
-        c->mv_dc = 0;
-        c->mv_old = x;
-        c->mv_new = d.vtype[j] == kVarBin ? (__double_as_longlong(x) == 0 ? 1.0 : 0.0) : L.xh[j];
-    } else {
-        c->mv_var = -1;
-        c->mv_s = 0;
-        c->mv_dc = 0;
-        c->mv_new = 0.0;
-        c->mv_old = 0.0;
-    }
+    learn_select(d, L);
 }
 
 // At an exact pass: the proposal misses when the exact best score exceeds the
@@ -845,6 +952,7 @@ namespace chap {
 
 struct LearnHost {
     Learn L{};
+    int tk_ctas = 8;             // CTAs of the top-k cluster
     std::vector<void *> allocs;
     cudaGraphExec_t gexec = nullptr;
     int g_key[4] = {0, 0, 0, 0};   // topk, exact_every, propose_every, graph weights pointer (low bits)
@@ -893,6 +1001,55 @@ chap_status lfail(chap_bs *h, chap_status s, const std::string &msg)
         }                                                                                    \
     } while (0)
 
+int grid_n(long long n, int threads, int cap = 152 * 8)
+{
+    long long g = (n + threads - 1) / threads;
+    return (int)std::max<long long>(1, std::min<long long>(g, cap));
+}
+
+// Adds the attribute of a chained launch to cfg (whose attrs, if any, are at) for
+// the iterations of a captured run (51 -> 48 us an iteration of 5 kernels over 200k
+// variables); a kernel launched by itself follows work of the
+// caller's, which may still be writing the weights, and takes none.
+void chain_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, int gate)
+{
+    if (!gate) return;
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs += 1;
+}
+
+void topk_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, int ctas, cudaStream_t st)
+{
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(kTkThreads);
+    cfg.dynamicSmemBytes = kTkSmem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+}
+
+// Cluster of the top-k kernel: 16 CTAs where the GPU can hold such a cluster, else 8.
+cudaError_t topk_shape(LearnHost *lh)
+{
+    cudaError_t e = cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, kTkSmem);
+    if (e != cudaSuccess) return e;
+    lh->tk_ctas = 8;
+    if (cudaFuncSetAttribute(k_topk, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at[1];
+        topk_config(cfg, at, kTkCtas, nullptr);
+        int fits = 0;
+        if (cudaOccupancyMaxActiveClusters(&fits, k_topk, &cfg) == cudaSuccess && fits > 0) lh->tk_ctas = kTkCtas;
+    }
+    cudaGetLastError();
+    return cudaSuccess;
+}
+
 // Learned-driver state of the handle, created on first use.
 chap_status ensure_learn(chap_bs *h, LearnHost **out)
 {
@@ -904,27 +1061,32 @@ chap_status ensure_learn(chap_bs *h, LearnHost **out)
     if (!lh) return CHAP_E_OOM;
     const int n = h->n;
     Learn &L = lh->L;
-    L.nblocks = (n + kTopkBlock - 1) / kTopkBlock;
     L.colviol = lalloc<float>(lh, n);
     L.colwv = lalloc<float>(lh, n);
     L.s_last = lalloc<long long>(lh, n);
     L.feat = lalloc<__nv_bfloat16>(lh, (size_t)n * kF);
     L.y = lalloc<float>(lh, n);
-    L.hist = lalloc<unsigned>(lh, 2048);
-    L.bcnt = lalloc<int>(lh, 2 * (size_t)std::max(1, L.nblocks));
-    L.bpre = lalloc<int>(lh, 2 * (size_t)std::max(1, L.nblocks));
+    L.fixed = lalloc<uint2>(lh, n);
+    L.hist = lalloc<unsigned>(lh, 3 * 2048);
+    L.bcnt = lalloc<int>(lh, 2 * kTkCtas);
     L.list = lalloc<int>(lh, n);
     L.xh = lalloc<double>(lh, n);
     L.lc = lalloc<LearnCtl>(lh, 1);
-    bool ok = L.colviol && L.colwv && L.s_last && L.feat && L.y && L.hist && L.bcnt && L.bpre && L.list && L.xh && L.lc &&
+    bool ok = L.colviol && L.colwv && L.s_last && L.feat && L.y && L.fixed && L.hist && L.bcnt && L.list && L.xh && L.lc &&
               cudaMallocHost(&lh->h_lc, sizeof(LearnCtl)) == cudaSuccess;
+    for (int j = 0; j < n; ++j) lh->cmax = std::max(lh->cmax, (float)std::fabs(h->obj[j]));
     cudaError_t e = cudaSuccess;
     if (ok) {
-        e = cudaMemsetAsync(L.colviol, 0, sizeof(float) * std::max(1, n), h->st);
+        e = topk_shape(lh);
+        if (e == cudaSuccess) e = cudaMemsetAsync(L.colviol, 0, sizeof(float) * std::max(1, n), h->st);
         if (e == cudaSuccess) e = cudaMemsetAsync(L.colwv, 0, sizeof(float) * std::max(1, n), h->st);
         if (e == cudaSuccess) e = cudaMemsetAsync(L.s_last, 0, sizeof(long long) * std::max(1, n), h->st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(L.hist, 0, sizeof(unsigned) * 2048, h->st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(L.hist, 0, sizeof(unsigned) * 3 * 2048, h->st);
         if (e == cudaSuccess) e = cudaMemsetAsync(L.lc, 0, sizeof(LearnCtl), h->st);
+        if (e == cudaSuccess) {
+            k_fixed_features<<<grid_n(n, 256), 256, 0, h->st>>>(h->dev, L, lh->cmax);
+            e = cudaGetLastError();
+        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     }
     if (!ok || e != cudaSuccess) {
@@ -933,16 +1095,9 @@ chap_status ensure_learn(chap_bs *h, LearnHost **out)
         learn_free(h);
         return ok ? CHAP_E_CUDA : CHAP_E_OOM;
     }
-    for (int j = 0; j < n; ++j) lh->cmax = std::max(lh->cmax, (float)std::fabs(h->obj[j]));
     h->learn = lh;
     *out = lh;
     return CHAP_OK;
-}
-
-int grid_n(long long n, int threads, int cap = 152 * 8)
-{
-    long long g = (n + threads - 1) / threads;
-    return (int)std::max<long long>(1, std::min<long long>(g, cap));
 }
 
 // exact scores into s_last and the pass-time column features
@@ -955,8 +1110,7 @@ cudaError_t launch_refresh(chap_bs *h, LearnHost *lh, int gate, cudaStream_t st)
     if (e != cudaSuccess) return e;
     k_refresh_begin<<<1, 1, 0, st>>>(d, lh->L, gate);
     // the refresh reads the state before the move; gated like the rest
-    if (!gate) k_refresh<<<grid_n(d.n, 256), 256, 0, st>>>(d, lh->L);
-    else k_refresh<<<grid_n(d.n, 256), 256, 0, st>>>(d, lh->L);
+    k_refresh<<<grid_n(d.n, 256), 256, 0, st>>>(d, lh->L);
     return cudaGetLastError();
 }
 
@@ -965,25 +1119,41 @@ cudaError_t launch_propose(chap_bs *h, LearnHost *lh, const __nv_bfloat16 *w, in
     const Dev &d = h->dev;
     const Learn &L = lh->L;
     const int n = d.n;
-    k_features<<<grid_n(n, 256), 256, 0, st>>>(d, L, lh->cmax, gate);
-    k_mlp_forward_tc<<<grid_n((n + 15) / 16 * 32, 256, 152 * 4), 256, 0, st>>>(w, L.feat, n, L.y,
-                                                                             gate ? &d.ctl->done : nullptr);
-    for (int level = 0; level < 3; ++level) {
-        k_topk_hist<<<grid_n(n, 256, 152 * 2), 256, 0, st>>>(d, L, L.y, n, level, gate);
-        k_topk_pick<<<1, 256, 0, st>>>(d, L, level, k, n, gate);
-    }
-    k_topk_count<<<std::max(1, L.nblocks), 256, 0, st>>>(d, L, L.y, n, gate);
-    k_topk_scan<<<1, 32, 0, st>>>(d, L, gate);
-    k_topk_write<<<std::max(1, L.nblocks), 256, 0, st>>>(d, L, L.y, n, gate);
-    return cudaGetLastError();
+    if (n < 1) return cudaSuccess;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[2];
+    cfg.gridDim = dim3((unsigned)grid_n((n + 31) / 32 * 32LL, kPropThreads, 152 * 3));
+    cfg.blockDim = dim3(kPropThreads);
+    cfg.stream = st;
+    chain_config(cfg, at, gate);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_propose_scores, d, L, w, gate);
+    if (e != cudaSuccess) return e;
+    topk_config(cfg, at, lh->tk_ctas, st);
+    chain_config(cfg, at, gate);
+    return cudaLaunchKernelEx(&cfg, k_topk, d, L, n, k, gate);
 }
 
-cudaError_t launch_subset(chap_bs *h, LearnHost *lh, int k, int gate, cudaStream_t st)
+// Exact scores of the listed variables; select: their best move goes to the
+// apply kernel.
+cudaError_t launch_subset(chap_bs *h, LearnHost *lh, int k, int select, int gate, cudaStream_t st)
 {
-    if (h->info.n_bin > 0) k_subset_eval<<<grid_n((long long)k * 8, 256, 152 * 4), 256, 0, st>>>(h->dev, lh->L, k, gate);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && h->info.n_bin < h->n - h->info.n_fixed)
-        e = launch_subset_nb(h->dev, h->plan, lh->L.list, k, lh->L.xh, &lh->L.lc->key, gate, st);
+    const bool nb = h->info.n_bin < h->n - h->info.n_fixed;
+    const bool fuse = select && !nb && h->info.n_bin > 0;   // the flips' last CTA selects
+    cudaError_t e = cudaSuccess;
+    if (h->info.n_bin > 0) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at[1];
+        cfg.gridDim = dim3((unsigned)grid_n((long long)k * 8, 256, 152 * 4));
+        cfg.blockDim = dim3(256);
+        cfg.stream = st;
+        chain_config(cfg, at, gate);
+        e = cudaLaunchKernelEx(&cfg, k_subset_eval, h->dev, lh->L, k, fuse ? 1 : 0, gate);
+    }
+    if (e == cudaSuccess && nb) e = launch_subset_nb(h->dev, h->plan, lh->L.list, k, lh->L.xh, &lh->L.lc->key, gate, st);
+    if (e == cudaSuccess && select && !fuse) {
+        k_learn_select<<<1, 1, 0, st>>>(h->dev, lh->L, gate);
+        e = cudaGetLastError();
+    }
     return e;
 }
 
@@ -1031,7 +1201,7 @@ chap_status chap_bs_features(chap_bs *h, uint16_t *feat, float *target)
     LearnHost *lh = nullptr;
     chap_status s = ensure_learn(h, &lh);
     if (s != CHAP_OK) return lfail(h, s, "learned-driver state");
-    k_features<<<grid_n(h->n, 256), 256, 0, h->st>>>(h->dev, lh->L, lh->cmax, 0);
+    k_features<<<grid_n(h->n, 256), 256, 0, h->st>>>(h->dev, lh->L);
     LCK(h, cudaGetLastError(), "features");
     if (feat && h->n)
         LCK(h, cudaMemcpyAsync(feat, lh->L.feat, sizeof(uint16_t) * kF * (size_t)h->n, cudaMemcpyDeviceToDevice, h->st),
@@ -1091,15 +1261,14 @@ chap_status chap_learned_run(chap_bs *h, const uint16_t *weights, const chap_lea
         cudaError_t e = cudaSuccess;
         // one block: the exact iteration, then exact_every - 1 proposal iterations
         e = launch_propose(h, lh, w, k, 1, cs);
-        if (e == cudaSuccess) e = launch_subset(h, lh, k, 1, cs);
+        if (e == cudaSuccess) e = launch_subset(h, lh, k, 0, 1, cs);
         if (e == cudaSuccess) e = launch_refresh(h, lh, 1, cs);
         if (e == cudaSuccess) { k_learn_miss<<<1, 1, 0, cs>>>(h->dev, lh->L, 1); e = cudaGetLastError(); }
-        if (e == cudaSuccess) e = launch_apply_gated(h->dev, h->plan, 1, cs);
+        if (e == cudaSuccess) e = launch_apply_gated(h->dev, h->plan, 1, cs, true);
         for (int i = 1; i < lo->exact_every && e == cudaSuccess; ++i) {
             if (i % lo->propose_every == 0) e = launch_propose(h, lh, w, k, 1, cs);
-            if (e == cudaSuccess) e = launch_subset(h, lh, k, 1, cs);
-            if (e == cudaSuccess) { k_learn_select<<<1, 1, 0, cs>>>(h->dev, lh->L, 1); e = cudaGetLastError(); }
-            if (e == cudaSuccess) e = launch_apply_gated(h->dev, h->plan, 1, cs);
+            if (e == cudaSuccess) e = launch_subset(h, lh, k, 1, 1, cs);
+            if (e == cudaSuccess) e = launch_apply_gated(h->dev, h->plan, 1, cs, true);
         }
         cudaError_t e2 = cudaStreamEndCapture(cs, &g);
         if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); LCK(h, e, "capture"); }

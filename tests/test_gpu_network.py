@@ -1,8 +1,10 @@
-"""The network's tile kernels at the edges of their tiles, against the FP64 oracle (oracle/mlp.py)."""
+"""The network's tile kernels and the proposal's selection at the edges of their
+tiles, against the FP64 oracle (oracle/mlp.py)."""
 import numpy as np
 import pytest
 
 from oracle import mlp
+from paper_2605_05086_gb300 import instances as inst
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +51,26 @@ def test_tiles_match_oracle(env, rows):
     # whole vector, as for the 1,000-row case of the general test
     assert np.linalg.norm(gg - g_ref) <= 1e-3 * np.linalg.norm(g_ref)
     assert abs(loss.item() / rows - l_ref) <= 1e-4 * l_ref
+
+
+# a warp's 32 variables less / exactly / plus one, one CTA's worth, several rounds
+@pytest.mark.parametrize("n", [31, 32, 33, 257, 152 * 2 * 256 + 33])
+@pytest.mark.parametrize("weights", ["drawn", "constant"])
+def test_selection_edges(env, n, weights):
+    torch, chap, learn = env
+    prob = inst.gen_setcover(seed=n, n=n, m=max(8, n // 2), k=min(6, n))
+    bs = chap.BestShift(prob, tenure=10)
+    chap.chap_bs_refresh_features(bs.h)
+    p = mlp.init_params(5)
+    if weights == "constant":
+        p[:] = 0.0          # every prediction equal: the first k variables
+    w = learn.to_bf16_bits(torch.tensor(p, device="cuda"))
+    for k in sorted({1, n // 3, n - 1, n}):
+        lst = torch.empty(k, dtype=torch.int32, device="cuda")
+        pred = torch.empty(n, dtype=torch.float32, device="cuda")
+        chap.chap_bs_propose(bs.h, w, k, lst, pred)
+        got = np.sort(lst.cpu().numpy())
+        assert np.array_equal(got, mlp.topk(pred.cpu().numpy(), k)), k
+        if weights == "constant":
+            assert np.array_equal(got, np.arange(k))
+    bs.close()
