@@ -437,13 +437,18 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     }
     h->m_norm = mn;
 
-    // rows of the residual kernel: the integral ones in index order, then the
-    // others by decreasing length (32 rows of like length per CTA)
+    // rows of the residual kernel: the short integral ones in index order (32 to a
+    // warp), the long ones by decreasing length (a warp each), then the others by
+    // decreasing length (32 rows of like length per CTA)
     std::vector<int> res_rows;
     res_rows.reserve(m);
     for (int i = 0; i < m; ++i)
         if (rint[i]) res_rows.push_back(i);
     const int n_res_int = (int)res_rows.size();
+    auto row_len = [&](int i) { return p->row_ptr[i + 1] - p->row_ptr[i]; };
+    const auto res_long = std::stable_partition(res_rows.begin(), res_rows.end(), [&](int i) { return row_len(i) <= kResShort; });
+    const int n_res_short = (int)(res_long - res_rows.begin());
+    std::stable_sort(res_long, res_rows.end(), [&](int a, int b) { return row_len(a) > row_len(b); });
     for (int i = 0; i < m; ++i)
         if (!rint[i]) res_rows.push_back(i);
     std::stable_sort(res_rows.begin() + n_res_int, res_rows.end(), [&](int a, int b) {
@@ -1028,7 +1033,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     d.ci_eq = ci_eq_d; d.cf_eq = cf_eq_d;
     d.row_ptr = row_ptr_d; d.col_idx = col_idx_d; d.row_val = row_val_d;
     d.rhs = rhs_d; d.eps = eps_d; d.row_int = rint_d; d.nrow_base = nrb_d;
-    d.res_rows = resr_d; d.n_res_int = n_res_int; d.m_norm = mn;
+    d.res_rows = resr_d; d.n_res_int = n_res_int; d.n_res_short = n_res_short; d.m_norm = mn;
     d.vtype = vt_d; d.lb = lb_d; d.ub = ub_d; d.obj = obj_d;
     d.var_list = vl_d;
     d.vpos = vpos_d;

@@ -321,9 +321,10 @@ struct Dev {
     HistAcc *racc;
     LCand *rcand;
     const RankCol *rcols;
-    // rows of the residual computation (set-state only): the integral rows,
-    // then the others by decreasing length
-    int n_res_int;
+    // rows of the residual computation (set-state only): n_res_short short
+    // integral rows, the other integral rows and then the rest, both by
+    // decreasing length
+    int n_res_int, n_res_short;
     const int *res_rows;
     // row-blocked binary flips only (else null / 0): per binary position 1 when
     // x of its variable is 0 (the flip raises it), kept by every x update
@@ -563,6 +564,7 @@ constexpr double kBlkMinSeg = 2.0;      // and from this many entries per (block
 // Entries a move changes on average up to which one CTA runs the search (16
 // chunks of 256, one per warp: a cluster would add its barriers and save nothing).
 constexpr double kSrOneCtaTouched = 4096.0;
+constexpr int kResShort = 64;            // entries up to which integral rows share a warp in the residual kernel
 constexpr int kSrHead = 8;              // integral column entries addressed by position
 constexpr int kSrLaunchIters = 2048;    // iterations of one launch of the search
 constexpr int kSrBlkPos = 256;          // positions (and physical rows) of one summary block

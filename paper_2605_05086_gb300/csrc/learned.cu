@@ -7,10 +7,11 @@
 //
 // Kernels: features, refresh of the pass-time features, network forward
 // (BF16 parameters and features, FP32 accumulation with explicit FMAs), loss
-// gradient over a minibatch (tile of 128 rows per CTA, activations in shared
-// memory), Adam, deterministic top-k by three-level radix select + stable
-// compaction, exact flip scores of the selected binary columns, and the glue
-// that hands the chosen move to the apply kernel of the exact path.
+// gradient over a minibatch (tiles of 64 rows, activations in shared memory),
+// Adam, the proposal's scores (features, forward pass and first histogram),
+// deterministic top-k by three-level radix select + stable compaction in one
+// cluster, exact flip scores of the selected binary columns, and the glue that
+// hands the chosen move to the apply kernel of the exact path.
 #include "chap_handle.h"
 
 #include <cooperative_groups.h>

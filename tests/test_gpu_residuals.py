@@ -1,0 +1,49 @@
+"""Row residuals, weights and the violated count after set_state, at the edges of
+the residual kernel's split: rows of 0, 7 to 9 and 63 to 65 entries, partly
+filled groups of 32 short rows, integral and floating-point rows mixed."""
+import numpy as np
+import pytest
+
+from oracle.oracle import Oracle
+from paper_2605_05086_gb300 import instances as inst
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def chap():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2605_05086_gb300 import chap as c
+    c.load()
+    return c
+
+
+@pytest.mark.parametrize("m", [1, 31, 32, 33, 700])
+@pytest.mark.parametrize("lens", [(8,), (0, 1, 7, 8, 9, 63, 64), (64, 65), (3, 200)])
+@pytest.mark.parametrize("fp_rows", [0.0, 0.3])
+def test_residuals(chap, m, lens, fp_rows):
+    rng = np.random.default_rng(1000 * m + len(lens) + int(10 * fp_rows))
+    n = 400
+    vt = rng.choice([inst.VAR_BIN, inst.VAR_INT], n)
+    ub = np.where(vt == inst.VAR_BIN, 1.0, 9.0)
+    rows, cols, vals = [], [], []
+    for i in range(m):
+        k = lens[i % len(lens)]
+        rows += [i] * k
+        cols += list(rng.choice(n, k, replace=False))
+        fp = rng.random() < fp_rows
+        vals += list(rng.standard_normal(k) if fp else rng.integers(1, 9, k) * rng.choice([-1.0, 1.0], k))
+    kind = rng.choice([inst.ROW_LE, inst.ROW_GE, inst.ROW_EQ], m)
+    prob = inst.from_triplets("residuals", n, m, rows, cols, vals, np.zeros(n), ub, np.ones(n),
+                              rng.integers(-4, 5, m).astype(float), vt, kind)
+    orc = Oracle(prob)
+    bs = chap.BestShift(prob, tenure=3)
+    for _ in range(2):
+        x = np.floor(rng.random(n) * (ub + 1))
+        bs.set_state(x)
+        r, _, nv = orc.residuals(x)
+        assert np.array_equal(bs.residuals(), r)
+        assert bs.state()["nviol"] == nv
+    bs.close()
