@@ -1117,8 +1117,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         }
         search_create(h, bin_cols, nb_cols, hist_vars, p->nnz, touched / std::max(1, n));
     }
-    pl.apply_blocks = (int)std::min<int64_t>(304, std::max<int64_t>(1, ((int64_t)m + kApplyThreads - 1) / kApplyThreads));
-    pl.apply_move_blocks = (int)std::min<int64_t>(152, std::max<int64_t>(1, ((int64_t)max_col + kApplyMoveThreads - 1) / kApplyMoveThreads));
+    pl.apply_blocks = (int)std::min<int64_t>(152, std::max<int64_t>(1, ((int64_t)std::max(max_col, m) + kApplyThreads - 1) / kApplyThreads));
 
     chap_info &in = h->info;
     in.n = n; in.m = m; in.m_norm = mn;

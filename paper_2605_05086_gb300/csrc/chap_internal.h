@@ -462,8 +462,7 @@ struct LaunchPlan {
     int bin_blk;               // binary flips row-blocked (k_eval_bin_blk, bb.n_items CTAs; k_bin_blk_final, n_bin = bb.n_fin)
     BinBlk bb;
     int lazy_mark_blocks;      // CTAs of the marking kernel
-    int apply_blocks;          // CTAs of the weight bump
-    int apply_move_blocks;     // CTAs of the move apply (longest column / kApplyMoveThreads)
+    int apply_blocks;          // CTAs of the apply kernel (longest column or all rows / kApplyThreads)
     cudaStream_t side[3];      // side streams of the non-binary evaluation kernels
     cudaEvent_t ev_fork, ev_join[3];
     // optional timing of the kernels of one pass (outside graph capture):
@@ -496,9 +495,9 @@ __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.laun
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 
-// chained: the two kernels are launched as dependents of the kernel before them
-// (chain_wait below), which then has to be one that every earlier kernel they
-// read from precedes in the stream.
+// chained: the kernel is launched as a dependent of the kernel before it
+// (chain_wait above), which then has to be one that every earlier kernel it
+// reads from precedes in the stream.
 cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st, bool chained = false);
 cudaError_t launch_set_move(const Dev &d, int var, double new_value, cudaStream_t st);
 cudaError_t launch_residuals(const Dev &d, const int *w, cudaStream_t st);
@@ -569,8 +568,7 @@ constexpr int kSrHead = 8;              // integral column entries addressed by 
 constexpr int kSrLaunchIters = 2048;    // iterations of one launch of the search
 constexpr int kSrBlkPos = 256;          // positions (and physical rows) of one summary block
 constexpr int kSrMaxRows = 512;         // column entries (and threads) of one CTA's records
-constexpr int kApplyThreads = 256;
-constexpr int kApplyMoveThreads = 1024;
+constexpr int kApplyThreads = 1024;
 constexpr int kLazyMaxRows = 2048;      // longer moved columns re-evaluate every kept binary score
 constexpr int kWarpSortMax = 128;       // longest list of an integer short column (one warp sorts it, K <= 4)
 constexpr int kWarpListMax = 256;       // ... of a continuous short column (a delta and a marker per half, K <= 8)

@@ -21,9 +21,9 @@
 //  * Every CTA reduces its columns to one candidate; the CTA that writes the
 //    last candidate slot reduces them all into the move (finish_pass: largest
 //    score, then lowest variable; k_select only when no evaluation CTA runs).
-//  * k_apply_move walks the chosen column and updates the residuals
+//  * k_apply walks the chosen column and updates the residuals
 //    incrementally (Sec. 3.1, "Memory Considerations", first point); when no
-//    positive move exists k_apply_bump adds 1 to the weight of every violated
+//    positive move exists it adds 1 to the weight of every violated
 //    normalised row.  The CTA that ends the iteration (finish_iteration) also
 //    tightens the objective cutoff row when the iteration ends feasible
 //    (Sec. 3.2) and copies x to the best solution.
@@ -2964,88 +2964,11 @@ __device__ __forceinline__ void snapshot_x(const Dev &d)
     for (int j = threadIdx.x; j < d.n; j += blockDim.x) d.x_best[j] = d.x[j];
 }
 
-// Apply a move: walk the moved column and update its rows' residuals
-// (Sec. 3.1, "Memory Considerations", first point).  The column is split over
-// as many CTAs of kApplyMoveThreads as its length needs (one for the usual
-// columns); the last of them finishes the iteration.
-__global__ void __launch_bounds__(kApplyMoveThreads) k_apply_move(Dev d, int gate)
-{
-    chain_next();
-    chain_wait();
-    if (gated_done(d, gate)) return;
-    Ctl *c = d.ctl;
-    const int var = c->mv_var;
-    if (var < 0) return;
-    const int q = d.vpos[var];
-    const int e0 = d.ci_ptr[q], e1 = d.ci_ptr[q + 1];
-    const int f0 = d.cf_ptr[q], f1 = d.cf_ptr[q + 1];
-    const int len = (e1 - e0) + (f1 - f0);
-    const int nwork = max(1, (len + kApplyMoveThreads - 1) / kApplyMoveThreads);
-    if ((int)blockIdx.x >= nwork) return;
-    const double dl = __dsub_rn(c->mv_new, c->mv_old);
-    const long long di = (long long)dl;
-    const int stride = nwork * kApplyMoveThreads;
-    long long local = 0;
-    for (int v = blockIdx.x * kApplyMoveThreads + threadIdx.x; v < len; v += stride) {
-        if (v < e1 - e0) {
-            const int e = e0 + v;
-            RowState *p = d.rs + d.ci_row[e];
-            const long long r0 = p->r;
-            const long long r1 = r0 + (long long)d.ci_val[e] * di;
-            p->r = r1;
-            local += (long long)(r1 > 0) - (long long)(r0 > 0);
-            if (p->w2 >= 0) local += (long long)(-r1 > 0) - (long long)(-r0 > 0);
-        } else {
-            const int e = f0 + (v - (e1 - e0));
-            const int i = d.cf_row[e];
-            RowState *p = d.rs + i;
-            const double eps = d.eps[i];
-            const double r1 = __dadd_rn(__longlong_as_double(p->r), __dmul_rn(d.cf_val[e], dl));
-            const double m1 = __dsub_rn(eps, r1), m2 = __dadd_rn(eps, r1);
-            local += (long long)dneg(m1) - (long long)dneg(p->m1);
-            if (p->w2 >= 0) local += (long long)dneg(m2) - (long long)dneg(p->m2);
-            p->r = __double_as_longlong(r1);
-            p->m1 = m1;
-            p->m2 = m2;
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) local += __shfl_xor_sync(FULLMASK, local, off);
-    __shared__ long long red[kApplyMoveThreads / 32];
-    __shared__ int s_snap;
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = local;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long t = 0;
-        for (int w = 0; w < kApplyMoveThreads / 32; ++w) t += red[w];
-        bool last = true;
-        if (nwork > 1) {
-            if (t) atomicAdd(reinterpret_cast<unsigned long long *>(&c->nviol_delta), (unsigned long long)t);
-            __threadfence();
-            last = atomicAdd(&c->apply_ticket, 1u) == (unsigned)(nwork - 1);
-            if (last) {
-                __threadfence();
-                t = (long long)__ldcg(reinterpret_cast<const long long *>(&c->nviol_delta));
-                c->nviol_delta = 0;
-                c->apply_ticket = 0;
-            }
-        }
-        s_snap = last && finish_iteration(d, c, var, q, t);
-    }
-    __syncthreads();
-    if (s_snap) snapshot_x(d);
-}
-
 // No admissible positive move: add 1 to the weight of every violated
 // normalised row (the weights of Sec. 3.1's scores); the last CTA finishes the
 // iteration.
-__global__ void __launch_bounds__(kApplyThreads) k_apply_bump(Dev d, int gate)
+__device__ void apply_bump(const Dev &d, Ctl *c)
 {
-    chain_next();
-    chain_wait();
-    if (gated_done(d, gate)) return;
-    Ctl *c = d.ctl;
-    if (c->mv_var >= 0) return;
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const int gstride = gridDim.x * blockDim.x;
     for (int i = gtid; i < d.m; i += gstride) {
@@ -3074,6 +2997,82 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply_bump(Dev d, int gate)
     if (s_snap) snapshot_x(d);
 }
 
+// Apply a move: walk the moved column and update its rows' residuals
+// (Sec. 3.1, "Memory Considerations", first point).  The column is split over
+// as many CTAs of kApplyThreads as its length needs (one for the usual
+// columns); the last of them finishes the iteration.  Without a move all CTAs
+// add to the weights; as a kernel of its own that returned at once when there
+// was a move it cost 3 us of each iteration.
+__global__ void __launch_bounds__(kApplyThreads) k_apply(Dev d, int gate)
+{
+    chain_next();
+    chain_wait();
+    if (gated_done(d, gate)) return;
+    Ctl *c = d.ctl;
+    const int var = c->mv_var;
+    if (var < 0) {
+        apply_bump(d, c);
+        return;
+    }
+    const int q = d.vpos[var];
+    const int e0 = d.ci_ptr[q], e1 = d.ci_ptr[q + 1];
+    const int f0 = d.cf_ptr[q], f1 = d.cf_ptr[q + 1];
+    const int len = (e1 - e0) + (f1 - f0);
+    const int nwork = min((int)gridDim.x, max(1, (len + kApplyThreads - 1) / kApplyThreads));
+    if ((int)blockIdx.x >= nwork) return;
+    const double dl = __dsub_rn(c->mv_new, c->mv_old);
+    const long long di = (long long)dl;
+    const int stride = nwork * kApplyThreads;
+    long long local = 0;
+    for (int v = blockIdx.x * kApplyThreads + threadIdx.x; v < len; v += stride) {
+        if (v < e1 - e0) {
+            const int e = e0 + v;
+            RowState *p = d.rs + d.ci_row[e];
+            const long long r0 = p->r;
+            const long long r1 = r0 + (long long)d.ci_val[e] * di;
+            p->r = r1;
+            local += (long long)(r1 > 0) - (long long)(r0 > 0);
+            if (p->w2 >= 0) local += (long long)(-r1 > 0) - (long long)(-r0 > 0);
+        } else {
+            const int e = f0 + (v - (e1 - e0));
+            const int i = d.cf_row[e];
+            RowState *p = d.rs + i;
+            const double eps = d.eps[i];
+            const double r1 = __dadd_rn(__longlong_as_double(p->r), __dmul_rn(d.cf_val[e], dl));
+            const double m1 = __dsub_rn(eps, r1), m2 = __dadd_rn(eps, r1);
+            local += (long long)dneg(m1) - (long long)dneg(p->m1);
+            if (p->w2 >= 0) local += (long long)dneg(m2) - (long long)dneg(p->m2);
+            p->r = __double_as_longlong(r1);
+            p->m1 = m1;
+            p->m2 = m2;
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) local += __shfl_xor_sync(FULLMASK, local, off);
+    __shared__ long long red[kApplyThreads / 32];
+    __shared__ int s_snap;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = local;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        long long t = 0;
+        for (int w = 0; w < kApplyThreads / 32; ++w) t += red[w];
+        bool last = true;
+        if (nwork > 1) {
+            if (t) atomicAdd(reinterpret_cast<unsigned long long *>(&c->nviol_delta), (unsigned long long)t);
+            __threadfence();
+            last = atomicAdd(&c->apply_ticket, 1u) == (unsigned)(nwork - 1);
+            if (last) {
+                __threadfence();
+                t = (long long)__ldcg(reinterpret_cast<const long long *>(&c->nviol_delta));
+                c->nviol_delta = 0;
+                c->apply_ticket = 0;
+            }
+        }
+        s_snap = last && finish_iteration(d, c, var, q, t);
+    }
+    __syncthreads();
+    if (s_snap) snapshot_x(d);
+}
 // --------------------------------------------------------- state handling
 
 // x_j + 0: a -0 from the caller is stored as +0, like every value the search
@@ -3681,16 +3680,12 @@ cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cuda
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)p.apply_move_blocks);
-    cfg.blockDim = dim3(kApplyMoveThreads);
+    cfg.gridDim = dim3((unsigned)p.apply_blocks);
+    cfg.blockDim = dim3(kApplyThreads);
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = chained ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_apply_move, d, gate);
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3((unsigned)p.apply_blocks);
-    cfg.blockDim = dim3(kApplyThreads);
-    e = cudaLaunchKernelEx(&cfg, k_apply_bump, d, gate);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_apply, d, gate);
     if (e != cudaSuccess) return e;
     if (p.lazy) k_lazy_mark<<<p.lazy_mark_blocks, kEvalThreads, 0, st>>>(d, p.bin_cols);
     return cudaGetLastError();
