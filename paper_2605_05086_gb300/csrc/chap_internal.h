@@ -500,6 +500,7 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // reads from precedes in the stream.
 cudaError_t launch_apply_gated(const Dev &d, const LaunchPlan &p, int gate, cudaStream_t st, bool chained = false);
 cudaError_t launch_set_move(const Dev &d, int var, double new_value, cudaStream_t st);
+cudaError_t launch_check_x(const Dev &d, const double *x, unsigned long long *bad, cudaStream_t st);
 cudaError_t launch_residuals(const Dev &d, const int *w, cudaStream_t st);
 cudaError_t launch_finish_set_state(const Dev &d, long long iter, long long best_nviol, int use_best, cudaStream_t st);
 cudaError_t launch_begin_run(const Dev &d, long long max_iters, int stop_at_feasible, cudaStream_t st);
@@ -563,6 +564,7 @@ constexpr double kBlkMinSeg = 2.0;      // and from this many entries per (block
 // Entries a move changes on average up to which one CTA runs the search (16
 // chunks of 256, one per warp: a cluster would add its barriers and save nothing).
 constexpr double kSrOneCtaTouched = 4096.0;
+constexpr int kCheckDevice = 1 << 14;    // variables from which a host state is checked on the device
 constexpr int kResShort = 64;            // entries up to which integral rows share a warp in the residual kernel
 constexpr int kSrHead = 8;              // integral column entries addressed by position
 constexpr int kSrLaunchIters = 2048;    // iterations of one launch of the search

@@ -3075,6 +3075,19 @@ __global__ void __launch_bounds__(kApplyThreads) k_apply(Dev d, int gate)
 }
 // --------------------------------------------------------- state handling
 
+// First variable whose value is out of its bounds (2 j) or fractional where an
+// integer is wanted (2 j + 1): the least of them to *bad.
+__global__ void k_check_x(Dev d, const double *x, unsigned long long *bad)
+{
+    unsigned long long b = ~0ull;
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n && b == ~0ull; j += gridDim.x * blockDim.x) {
+        const double v = x[j];
+        if (!(v >= d.lb[j] && v <= d.ub[j])) b = 2ull * j;
+        else if (d.vtype[j] != kVarCont && !(isfinite(v) && floor(v) == v)) b = 2ull * j + 1;
+    }
+    if (b != ~0ull) atomicMin(bad, b);
+}
+
 // x_j + 0: a -0 from the caller is stored as +0, like every value the search
 // writes itself.
 __global__ void k_canon_x(Dev d)
@@ -3700,6 +3713,12 @@ cudaError_t launch_lazy_init(const Dev &d, cudaStream_t st)
 cudaError_t launch_set_move(const Dev &d, int var, double nv, cudaStream_t st)
 {
     k_set_move<<<1, 1, 0, st>>>(d, var, nv);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_check_x(const Dev &d, const double *x, unsigned long long *bad, cudaStream_t st)
+{
+    k_check_x<<<grid_for(d.n, 256), 256, 0, st>>>(d, x, bad);
     return cudaGetLastError();
 }
 

@@ -47,3 +47,35 @@ def test_residuals(chap, m, lens, fp_rows):
         assert np.array_equal(bs.residuals(), r)
         assert bs.state()["nviol"] == nv
     bs.close()
+
+
+# the least sizes on either side of the device's check, and a last partial block
+@pytest.mark.parametrize("n", [16383, 16384, 20001])
+def test_refused_states(chap, n):
+    rng = np.random.default_rng(n)
+    vt = np.array([inst.VAR_BIN, inst.VAR_INT, inst.VAR_CONT])[np.arange(n) % 3]
+    lb, ub = np.zeros(n), np.where(vt == inst.VAR_BIN, 1.0, 9.0)
+    ub[4] = np.inf
+    m = 50
+    rows = np.repeat(np.arange(m), 6)
+    prob = inst.from_triplets("states", n, m, rows, rng.integers(0, n, 6 * m), np.ones(6 * m), lb, ub, np.ones(n),
+                              np.full(m, 2.0), vt, np.full(m, inst.ROW_LE))
+    bs = chap.BestShift(prob, tenure=3)
+    good = np.floor(rng.random(n) * (np.minimum(ub, 9.0) + 1))
+    bs.set_state(good)
+    before = bs.state()
+    bounds, frac = "x out of bounds at variable %d", "fractional value of integer variable %d"
+    for changes, msg in [({n - 1: -1.0}, bounds % (n - 1)), ({0: np.nan}, bounds % 0), ({1: 0.5}, frac % 1),
+                         ({2: 9.5, 3: 0.5}, bounds % 2), ({9: 0.5, 10: 100.0}, frac % 9), ({4: np.inf}, frac % 4)]:
+        x = good.copy()
+        for j, v in changes.items():
+            x[j] = v
+        with pytest.raises(chap.ChapError, match=msg):
+            bs.set_state(x)
+        st = bs.state()
+        assert all(np.array_equal(st[k], before[k]) for k in before)
+    x = good.copy()
+    x[2] = 3.25          # a continuous variable takes any value in its bounds
+    bs.set_state(x)
+    assert np.array_equal(bs.state()["x"], x)
+    bs.close()
