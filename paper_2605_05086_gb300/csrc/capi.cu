@@ -246,7 +246,7 @@ void search_create(chap_bs *h, int bin_cols, int nb_cols, const std::vector<int>
         const int j = hist_vars[k];
         S.hist_bins += ((int64_t)(h->ub[j] - h->lb[j]) + 2) & ~1LL;
     }
-    if (!search_shape(S, touched <= kSrOneCtaTouched)) {
+    if (!search_shape(S, !S.mix && touched <= kSrOneCtaTouched)) {
         S = Search{};
         return;
     }
@@ -1135,6 +1135,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         return CHAP_E_CUDA;
     }
     if (keep) {
+        h->srch_dense = kind_base[T_NB_HIST] != kind_base[T_NB_HIST + 1] && p->nnz < kSrHistNnz;
         const std::vector<int> hist_vars(var_list.begin() + kind_base[T_NB_HIST], var_list.begin() + kind_base[T_NB_HIST + 1]);
         // mean entries a move's walk meets: sum of len^2 over the rows, per column
         double touched = 0.0;
@@ -1529,7 +1530,7 @@ chap_status chap_tabu_run(chap_bs *h, const chap_options *opts, chap_tabu_result
         return fail(h, CHAP_E_UNSUPPORTED, "iteration counter would exceed the 32-bit tabu stamps");
     Dev &d = h->dev;
     CK(h, launch_begin_run(d, o.max_iters, o.stop_at_feasible, h->st), "begin run");
-    if (h->srch.on && !h->h_ctl->cut_on) {
+    if (h->srch.on && !h->h_ctl->cut_on && !(h->srch_dense && h->h_ctl->nviol * kSrHistNear > h->m)) {
         s = search_run(h);
         if (s != CHAP_OK) return s;
     } else {

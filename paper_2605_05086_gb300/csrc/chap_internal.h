@@ -561,9 +561,21 @@ constexpr int kBlkFinThreads = 256;
 constexpr int kBlkMaxBlocks = 32;       // the library picks the row-blocked flips up to this many row blocks,
 constexpr int kBlkMinCols = 16384;      // from this many binary columns,
 constexpr double kBlkMinSeg = 2.0;      // and from this many entries per (block, column) on average
-// Entries a move changes on average up to which one CTA runs the search (16
-// chunks of 256, one per warp: a cluster would add its barriers and save nothing).
+// Entries a move changes on average up to which one CTA runs the search of an
+// all-binary instance (16 chunks of 256, one per warp: a cluster would add its
+// barriers and save nothing).  A mixed one takes the cluster: 20k variables
+// 2.9 ms for 100 iterations against 3.5 in one CTA, 60k with 50 counting-sorted
+// columns 4.7 for 48 against 10.0.
 constexpr double kSrOneCtaTouched = 4096.0;
+// With counting-sorted columns a move from a far state changes so much that the
+// kept scores cost about 100 us an iteration at any size, a full pass its
+// nonzeros: 48 iterations of 120k variables (0.9M nonzeros) 5.5 ms against 3.3
+// for the iteration graph, of 300k (2.3M) 3.8 against 4.8, 64 of 2M (20M) 10.3
+// against 26.  Near feasibility (few violated rows) the search wins at 60k too
+// (1.9 against 4.1).  The graph runs below the first with more than a row in
+// kSrHistNear violated at the start of the call.
+constexpr long long kSrHistNnz = 2000000;
+constexpr int kSrHistNear = 16;
 constexpr int kCheckDevice = 1 << 14;    // variables from which a host state is checked on the device
 constexpr int kResShort = 64;            // entries up to which integral rows share a warp in the residual kernel
 constexpr int kSrHead = 8;              // integral column entries addressed by position

@@ -79,3 +79,19 @@ def test_refused_states(chap, n):
     bs.set_state(x)
     assert np.array_equal(bs.state()["x"], x)
     bs.close()
+
+
+def test_column_longer_than_the_apply_grid(chap):
+    # 152 CTAs of 1,024 threads apply a move: this column has more entries
+    m = 152 * 1024 + 77
+    rows = np.concatenate([np.arange(m), [0, 1]])
+    cols = np.concatenate([np.zeros(m, np.int64), [1, 2]])
+    prob = inst.from_triplets("long_column", 3, m, rows, cols, np.ones(m + 2), np.zeros(3), np.ones(3), np.ones(3),
+                              np.ones(m), np.full(3, inst.VAR_BIN), np.full(m, inst.ROW_GE))
+    bs = chap.BestShift(prob, tenure=3)
+    assert bs.state()["nviol"] == m
+    mv = bs.step()
+    assert (mv.var, mv.dnviol) == (0, -m)
+    st = bs.state()
+    assert st["nviol"] == 0 and np.array_equal(bs.residuals(), Oracle(prob).residuals(st["x"])[0])
+    bs.close()

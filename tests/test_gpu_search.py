@@ -82,6 +82,16 @@ def integers_long_columns(seed, n_hub=5, rows_per=200, dom=300, n_other=120):
                               np.ones(n), np.array(rhs), vt, sense, x0=np.clip(np.zeros(n), lb, ub))
 
 
+def nearly_feasible(prob):
+    """The instance with the right-hand sides moved so that the start point
+    violates at most every 20th row."""
+    x0 = np.clip(0.0, prob.lb, prob.ub)
+    rows = np.repeat(np.arange(prob.m), np.diff(prob.row_ptr))
+    act = np.bincount(rows, weights=prob.row_val * x0[prob.col_idx], minlength=prob.m)
+    prob.rhs = np.where(np.arange(prob.m) % 20 == 0, prob.rhs, act)
+    return prob
+
+
 INSTANCES.update({
     # non-binary columns: bounds and kept results, short lists and long ones
     "general": lambda: inst.gen_general(seed=1, n=6_000, m=3_000, len_cap=300),
@@ -92,6 +102,12 @@ INSTANCES.update({
     "hubs": lambda: integers_long_columns(4),
     "hubs_700": lambda: integers_long_columns(5, n_hub=3, rows_per=700),
     "skewed": lambda: inst.gen_skewed(seed=6, n=40_000, m=20_000, n_dense=6, dense_len=6_000),
+    # the two forms in which a search with counting-sorted columns starts: many
+    # nonzeros, or few violated rows (else the iteration graph runs)
+    "skewed_many_nonzeros": lambda: inst.gen_skewed(seed=6, n=320_000, m=160_000, n_dense=6, dense_len=20_000),
+    "skewed_near": lambda: nearly_feasible(inst.gen_skewed(seed=6, n=40_000, m=20_000, n_dense=6, dense_len=6_000)),
+    "hubs_near": lambda: nearly_feasible(integers_long_columns(4)),
+    "hubs_700_near": lambda: nearly_feasible(integers_long_columns(5, n_hub=3, rows_per=700)),
 })
 
 
