@@ -616,7 +616,7 @@ def main():
                     "h2d_bytes_per_step": 8 * prob.n,
                     "d2h_bytes_per_step": 8 * prob.n + 2 * 256 + 8,
                     "iters_per_e2e_step": e2e_iters, "steps": e2e_steps,
-                    "call": "chap_bs_set_state(pinned host x) + chap_tabu_run(64 iterations, one graph replay) "
+                    "call": "chap_bs_set_state(pinned host x) + chap_tabu_run(64 iterations) "
                             "+ x and the run's counters to the host",
                     "variants": {
                         "one_iteration_per_step": {

@@ -339,7 +339,9 @@ CHAP_API chap_status chap_bs_step(struct chap_bs *h, chap_move *out);
  * changes; the same moves), in launches of many iterations.  Instances with
  * CTA- or merge-sorted columns, handles created with lazy_binary, bin_kernel 2
  * or 3 or static_scratch_only, handles whose device memory did not hold the
- * kept state, and runs under an objective cutoff evaluate every iteration from
+ * kept state, runs under an objective cutoff, and runs with counting-sorted
+ * columns on fewer than 2M nonzeros that start with more than a 16th of the
+ * rows violated evaluate every iteration from
  * scratch, recorded into a CUDA graph of opts->graph_iters iterations
  * (Sec. 3.1, "Kernel Specialization", last point) and replayed.
  * opts may be NULL (the create options).  result (host) is filled on success.
