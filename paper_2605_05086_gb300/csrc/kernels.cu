@@ -49,6 +49,8 @@ namespace chap {
 
 #define FULLMASK 0xffffffffu
 
+constexpr long long kNoScore = 1LL << 60;   // beyond every score
+
 constexpr unsigned long long kSign = 0x8000000000000000ull;
 constexpr unsigned long long kPadKey = ~0ull;
 constexpr int kNoVar = INT_MAX;
@@ -1591,21 +1593,28 @@ __device__ __forceinline__ void load_entry(const SEnt *p, unsigned long long &ke
 // entries and hold 256 at most; all short columns of a general 200k-variable
 // MIP with outputs 256 -> 234 us a pass, 224 with the long lists counted too
 // (their network, 36 stages unrolled, waited for its code).
-template <int G>
+// TOP (whole-warp lists of a continuous column): top becomes the largest score
+// of any value of the column, candidate or not.  The score is constant between
+// neighbouring entries and xbar, so it is the largest of the scores at the
+// entries, right after each entry and xbar (one more step of the loop), and
+// left of the first entry where there is no lower bound.
+template <int G, bool TOP = false>
 __device__ __forceinline__ VCand group_count(const ColCtx &c, const Acc &a, const SEnt *list, int cnt, int cmax,
-                                             long long nviol, long long bestnv)
+                                             long long nviol, long long bestnv, long long *top = nullptr)
 {
     const int lane = threadIdx.x & 31, sub = lane & (G - 1);
     const int rot = min(lane / G, cmax - 1);
     VCand vb{0, 0ull, 0, 0};
+    long long t = TOP && c.kl == dkey(-1.7976931348623157e308) ? a.beta : -kNoScore;
 #pragma unroll 1
-    for (int k = sub; k - sub < cmax; k += G) {
+    for (int k = sub; k - sub < cmax + (TOP ? 1 : 0); k += G) {
         unsigned long long key = kPadKey;
         long long del;
         unsigned aux = make_aux(kClsPostDelta, 0);
         if (k < cnt) load_entry(list + k, key, del, aux);
+        else if (TOP && k == cnt) key = c.kxb;
         const bool right = key > c.kxb;
-        long long s = a.beta + (right ? a.alpha : 0);
+        long long s = a.beta + (right ? a.alpha : 0), after = a.beta + (key >= c.kxb ? a.alpha : 0);
         int dc = a.beta_c + (right ? a.alpha_c : 0);
 #pragma unroll 2
         for (int e = 0; e < cmax; ++e) {
@@ -1621,8 +1630,13 @@ __device__ __forceinline__ VCand group_count(const ColCtx &c, const Acc &a, cons
             const bool in = ek < key || (ek == key && aux_post(ea) == 0);
             s += in ? ed : 0;
             dc += in ? aux_dc(ea) : 0;
+            if (TOP) after += ek <= key ? ed : 0;
         }
         const unsigned cls = aux_cls(aux);
+        if (TOP && k <= cnt) {
+            if (key != c.kxb) t = max(t, s);
+            if (key < c.ku) t = max(t, after);
+        }
         if (k < cnt && (cls == kClsPre || cls == kClsPost)) consider(vb, c, key, s, dc, nviol, bestnv);
     }
 #pragma unroll
@@ -1633,7 +1647,9 @@ __device__ __forceinline__ VCand group_count(const ColCtx &c, const Acc &a, cons
         p.dc = __shfl_xor_sync(FULLMASK, vb.dc, o);
         p.valid = __shfl_xor_sync(FULLMASK, vb.valid, o);
         if (vc_better(p, vb, c)) vb = p;
+        if (TOP) t = max(t, __shfl_xor_sync(FULLMASK, t, o));
     }
+    if (TOP) *top = t;
     return vb;
 }
 
@@ -1691,16 +1707,24 @@ __device__ __noinline__ void column_warp(const Dev &d, const VarOut &o, int q, S
     __syncwarp();
 }
 
-// The best candidate of the column at position q in every lane, and its value;
-// row states may change inside the calling kernel.
+// The best candidate of the column at position q in every lane, its value and
+// the largest score of any value of the column (-kNoScore: of none); row states
+// may change inside the calling kernel.
 __device__ __noinline__ VCand column_best(const Dev &d, int q, SEnt *stage, long long iter, long long nviol,
-                                          long long bestnv, double &xh)
+                                          long long bestnv, double &xh, long long &top)
 {
-    const int lane = threadIdx.x & 31;
     const ColCtx c = make_col(d, q, iter);
     Acc acc;
     const int cnt = column_list<true>(d, c, stage, acc);
-    const VCand vb = group_count<32>(c, acc, stage, cnt, cnt, nviol, bestnv);
+    const VCand vb = group_count<32, true>(c, acc, stage, cnt, cnt, nviol, bestnv, &top);
+    // Integer columns: every breakpoint is a candidate and none is better than
+    // the values past it, so only a side without a candidate (no bound, no row
+    // that gets better there) is not covered, and no row gains on such a side.
+    if (c.isint) {
+        const bool open = c.lo == -(1LL << 62) || c.hi == (1LL << 62);
+        top = vb.valid ? vb.s : -kNoScore;
+        if (open) top = max(top, 0LL);
+    }
     __syncwarp();
     xh = vb.valid ? key_value(c, vb.key) : c.xb;
     return vb;

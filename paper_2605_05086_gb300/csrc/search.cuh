@@ -17,8 +17,10 @@
 //    entry is the move when tabu and aspiration admit it; otherwise the blocks
 //    that can hold the best admissible one are scanned.
 //  * A short non-binary column keeps its best shift while none of its halves
-//    change, and else an upper bound of its score; it is evaluated again
-//    (Algorithm 1, one warp) only when that bound reaches the best score found.
+//    change, and else an upper bound of its score (of every value's: a later
+//    change of a row moves candidates to values that were none); it is evaluated
+//    again (Algorithm 1, one warp) only when that bound reaches the best score
+//    found.
 //    A counting-sorted column keeps its bins.
 //  * Apply: one thread per row of the moved column computes the row state
 //    after the move into a shared-memory record (every CTA all of them, so
@@ -269,7 +271,9 @@ __device__ __forceinline__ void sr_nmark(const SrTeam *T, const SrLocal &L, int 
 // A half whose breakpoint is certainly outside the bounds, or certainly at
 // the first step, has the same penalty change at every candidate of a side
 // (decided); a change of its residual that leaves it so leaves the column's
-// scores as they are.
+// scores as they are.  On a continuous column the candidate of a satisfied row,
+// its tight point, lies eps / |a| before its breakpoint: it has to be outside
+// too, or it moves.
 
 struct SrTerm {
     int l, r;       // largest penalty change left and right of xbar, in weights
@@ -277,12 +281,13 @@ struct SrTerm {
 };
 
 // Half with magnitude |m| of its margin (m = eps - r; |r| on an integral row),
-// violated V, coefficient sign P (a > 0) and magnitude |a|; ok: both
-// magnitudes are usable floats.
-__device__ __forceinline__ SrTerm sr_term(bool V, bool P, float mf, float af, bool ok, const NbCtx &c)
+// violated V, coefficient sign P (a > 0) and magnitude |a|; tf: |r| where a
+// satisfied half has a tight point, else |m|; ok: the magnitudes are usable
+// floats.
+__device__ __forceinline__ SrTerm sr_term(bool V, bool P, float mf, float tf, float af, bool ok, const NbCtx &c)
 {
     const float to = V == P ? c.dl : c.dh;        // distance to the bound the breakpoint lies towards
-    const float reach = af * to * 1.00001f + c.tol * af, lo = mf * 0.99999f;
+    const float reach = af * to * 1.00001f + c.tol * af, lo = (V ? mf : tf) * 0.99999f;
     const bool outside = ok && reach < lo;        // the breakpoint is past that bound
     SrTerm t;
     if (V) {
@@ -311,12 +316,12 @@ __device__ __forceinline__ SrTerms sr_terms(long long rb, double eps, int w1, in
 {
     SrTerms o;
     bool ok = true, P;
-    float m1, m2, af;
+    float m1, m2, t1, t2, af;
     if (!FP) {
         o.v1 = rb > 0;
         o.v2 = rb < 0;
         P = a > 0;
-        m1 = m2 = fabsf((float)rb);
+        m1 = m2 = t1 = t2 = fabsf((float)rb);
         af = fabsf((float)(int)a);
     } else {
         const double rr = __longlong_as_double(rb), b1 = __dsub_rn(eps, rr), b2 = __dadd_rn(eps, rr);
@@ -326,13 +331,16 @@ __device__ __forceinline__ SrTerms sr_terms(long long rb, double eps, int w1, in
         m1 = fabsf(approx_f(b1, ok));
         m2 = fabsf(approx_f(b2, ok));
         af = fabsf(approx_f(__longlong_as_double(a), ok));
+        t1 = m1;
+        t2 = m2;
+        if (!c.isint && (o.v1 || o.v2)) t1 = t2 = fabsf(approx_f(rr, ok));
     }
-    const SrTerm t = sr_term(o.v1, P, m1, af, ok, c);
+    const SrTerm t = sr_term(o.v1, P, m1, t1, af, ok, c);
     o.l = (long long)t.l * w1;
     o.r = (long long)t.r * w1;
     o.decided = t.decided;
     if (w2 < 0) return o;
-    const SrTerm u = sr_term(o.v2, !P, m2, af, ok, c);
+    const SrTerm u = sr_term(o.v2, !P, m2, t2, af, ok, c);
     o.l += (long long)u.l * w2;
     o.r += (long long)u.r * w2;
     o.decided = o.decided && u.decided;
@@ -471,7 +479,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_keep_bin(Dev d, Search S)
     keep_bin<G>(d, S);
 }
 
-constexpr long long kSrNoBound = 1LL << 60;   // kU of a column never evaluated
+constexpr long long kSrNoBound = kNoScore;   // kU of a column never evaluated
 
 // Contexts and bounds of the short non-binary columns: 8 lanes per column.
 __global__ void __launch_bounds__(kEvalThreads) k_keep_nb(Dev d, Search S)
@@ -1214,16 +1222,19 @@ __device__ __noinline__ VCand sr_hist_eval(const Search &S, int k, const ColCtx 
 }
 
 // The best shift of the column at place p by the warp: with free = true
-// regardless of tabu (kept), else of the admissible ones.
+// regardless of tabu (kept), else of the admissible ones.  top: of a short
+// column, the largest score of any of its values.
 __device__ __forceinline__ VCand sr_eval_column(const Dev &d, const Search &S, const SrLocal &L, int p, bool free,
-                                                long long iter, long long nviol, long long bestnv, double &xh)
+                                                long long iter, long long nviol, long long bestnv, double &xh,
+                                                long long &top)
 {
     const int warp = threadIdx.x >> 5;
     const int q = S.bc + p;
     const long long it = free ? LLONG_MAX : iter;
     VCand vb;
+    top = 0;
     if (p < S.nnb) {
-        vb = column_best(d, q, L.stage + warp * kWarpListMax, it, nviol, bestnv, xh);
+        vb = column_best(d, q, L.stage + warp * kWarpListMax, it, nviol, bestnv, xh, top);
     } else {
         const ColCtx c = make_col(d, q, it);
         vb = sr_hist_eval(S, p - S.nnb, c, nviol, bestnv);
@@ -1253,9 +1264,11 @@ __device__ __forceinline__ void sr_refresh(const Dev &d, const Search &S, const 
     const int lane = threadIdx.x & 31, q = S.bc + p;
     const int j = __ldg(d.var_list + q);
     double xh;
-    VCand v = sr_eval_column(d, S, L, p, true, iter, nviol, bestnv, xh);
+    long long top;
+    VCand v = sr_eval_column(d, S, L, p, true, iter, nviol, bestnv, xh, top);
     if (lane == 0) {
-        S.kU[p] = v.valid ? v.s : -kSrNoBound;
+        S.cS[p] = v.valid ? v.s : 0;
+        if (p < S.nnb) S.kU[p] = top;
         S.cX[p] = xh;
         S.cD[p] = v.dc;
         S.clean[p] = 1;
@@ -1263,7 +1276,7 @@ __device__ __forceinline__ void sr_refresh(const Dev &d, const Search &S, const 
     bool ok = v.valid && v.s > 0;
     if (!ok) return;
     if (!sr_admissible(d, j, xh, v.dc, iter, nviol, bestnv)) {
-        v = sr_eval_column(d, S, L, p, false, iter, nviol, bestnv, xh);
+        v = sr_eval_column(d, S, L, p, false, iter, nviol, bestnv, xh, top);
         ok = v.valid && v.s > 0;
     }
     if (ok && lane == 0) sr_take(m, v.s, j, q, xh, v.dc);
@@ -1285,18 +1298,19 @@ __device__ __forceinline__ void sr_load_nb(const Search &S, int gb, SrNbBlock &B
 {
     constexpr int PER = kSrBlk / 32;
     const int lane = threadIdx.x & 31;
-    long long kl[PER], kr[PER], ku[PER];
+    long long kl[PER], kr[PER], ku[PER], cs[PER];
     int sd[PER], cl[PER];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int p = gb * kSrBlk + 32 * k + lane;
-        kl[k] = kr[k] = ku[k] = 0;
+        kl[k] = kr[k] = ku[k] = cs[k] = 0;
         sd[k] = 0;
         cl[k] = 1;
         if (p < S.nnb) {
             kl[k] = __ldcg(S.kL + p);
             kr[k] = __ldcg(S.kR + p);
             ku[k] = __ldcg(S.kU + p);
+            cs[k] = __ldcg(S.cS + p);
             sd[k] = __ldcg(S.side + p);
             cl[k] = __ldcg(S.clean + p);
         }
@@ -1304,7 +1318,7 @@ __device__ __forceinline__ void sr_load_nb(const Search &S, int gb, SrNbBlock &B
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const long long a = (sd[k] & 1) ? kl[k] : 0, b = (sd[k] & 2) ? kr[k] : 0;
-        B.s[k] = cl[k] && ku[k] > 0 ? ku[k] : 0;
+        B.s[k] = cl[k] && cs[k] > 0 ? cs[k] : 0;
         B.u[k] = cl[k] ? 0u : sr_sat(min(max(a, b), ku[k]));
     }
 }
@@ -1484,7 +1498,7 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
         for (int h = threadIdx.x; h < S.nhist; h += kSrThreads) L.hc[h] = S.hctx[h];
         for (int kk = threadIdx.x; kk * nct + T.rank < S.nhist; kk += kSrThreads) {
             const int p = S.nnb + kk * nct + T.rank;
-            const long long s = S.clean[p] ? S.kU[p] : 0;
+            const long long s = S.clean[p] ? S.cS[p] : 0;
             L.htops[kk] = s > 0 ? SrBest{s, d.var_list[S.bc + p], S.bc + p} : SrBest{0, kNoVar, 0};
         }
         if (threadIdx.x == 0) sh.ncand = 0;
@@ -1555,9 +1569,10 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
                 const int p = S.nnb + kk * nct + T.rank;
                 if (!__ldcg(S.clean + p)) {
                     double xh;
-                    const VCand v = sr_eval_column(d, S, L, p, true, iter, nviol, bestnv, xh);
+                    long long top;
+                    const VCand v = sr_eval_column(d, S, L, p, true, iter, nviol, bestnv, xh, top);
                     if (lane == 0) {
-                        S.kU[p] = v.valid ? v.s : -kSrNoBound;
+                        S.cS[p] = v.valid ? v.s : 0;
                         S.cX[p] = xh;
                         S.cD[p] = v.dc;
                         S.clean[p] = 1;

@@ -239,3 +239,68 @@ def test_short_column_lanes_fill_the_gpu(chap, n, lanes):
         assert np.array_equal(g[1][pick], o[1]) and np.array_equal(g[2][pick], o[2])
         assert np.allclose(g[0][pick], o[0], rtol=1e-9, atol=1e-9)
     bs.close()
+
+
+def _run_equals_steps(chap, prob, start, tenure=0, feas_tol=1e-9, iters=(1, 2, 9, 30)):
+    """Runs and single steps from `start` (x, w) give the same state."""
+    a = chap.BestShift(prob, tenure=tenure, feas_tol=feas_tol)
+    b = chap.BestShift(prob, tenure=tenure, feas_tol=feas_tol)
+    a.set_state(*start)
+    b.set_state(*start)
+    for k in iters:
+        a.run(max_iters=k, stop_at_feasible=0)
+        for _ in range(k):
+            b.step()
+        sa, sb = a.state(), b.state()
+        sb["feasible_iter"] = sa["feasible_iter"]
+        _same_state(sa, sb)
+    a.close()
+    b.close()
+    return sa
+
+
+@pytest.mark.parametrize("vt", [inst.VAR_CONT, inst.VAR_INT])
+def test_column_without_a_candidate_on_its_unbounded_side(chap, vt):
+    """y in [0, inf) at 5, z binary at 0; y <= 3 (weight 1), y >= 5 (3),
+    y - 10 z >= -4 (1), z >= 1 (2).  At first y's candidates 3 and 0 score -4
+    while every value right of 5 scores -1; z flips, and then y moves to 6
+    with score 1 (two gained on the third row, one lost on the first)."""
+    prob = inst.from_triplets("open_side", 2, 4, [0, 1, 2, 2, 3], [0, 0, 0, 1, 1], [1.0, 1.0, 1.0, -10.0, 1.0],
+                              [0.0, 0.0], [np.inf, 1.0], [1.0, 1.0], [3.0, 5.0, -4.0, 1.0], [vt, inst.VAR_BIN],
+                              [inst.ROW_LE, inst.ROW_GE, inst.ROW_GE, inst.ROW_GE], x0=[5.0, 0.0])
+    st = _run_equals_steps(chap, prob, (np.array([5.0, 0.0]), np.array([1, 3, 1, 2], np.int32)), tenure=3, iters=(2,))
+    assert st["x"].tolist() == [6.0, 1.0] and st["moves"] == 2
+
+
+def open_bounds(seed, finite=0.3):
+    """Short rows over binaries, integers and continuous columns, most of the
+    latter in [0, inf) or free; "=" rows and a third of the others tight at the
+    start point, uneven right-hand sides elsewhere."""
+    rng = np.random.default_rng(seed)
+    n, m = int(rng.integers(6, 60)), int(rng.integers(6, 70))
+    vt = rng.choice(np.array([inst.VAR_BIN, inst.VAR_INT, inst.VAR_CONT], np.uint8), size=n, p=[0.4, 0.2, 0.4])
+    lb, ub = np.zeros(n), np.where(vt == inst.VAR_BIN, 1.0, np.inf)
+    other = vt != inst.VAR_BIN
+    lb[other & (rng.random(n) < 0.3)] = -np.inf
+    fin = other & (rng.random(n) < finite)
+    ub[fin] = rng.integers(3, 12, size=int(fin.sum()))
+    x0 = np.where(vt == inst.VAR_CONT, rng.integers(0, 25, size=n) / 8.0, rng.integers(0, 4, size=n)).astype(float)
+    x0 = np.where(vt == inst.VAR_BIN, rng.integers(0, 2, size=n), x0).astype(float)
+    rows, cols, vals = [], [], []
+    for i in range(m):
+        js = rng.choice(n, size=int(rng.integers(1, min(6, n) + 1)), replace=False)
+        rows += [i] * len(js); cols += sorted(js.tolist())
+        vals += rng.choice([-4, -2, -1, -0.5, 0.5, 1, 2, 4, 8], size=len(js)).tolist()
+    act = np.bincount(rows, weights=np.array(vals) * x0[cols], minlength=m)
+    sense = rng.choice([0, 1, 2], size=m, p=[0.4, 0.4, 0.2]).astype(np.uint8)
+    off = np.where((sense == 2) & (rng.random(m) < 0.7) | (rng.random(m) < 0.33), 0.0, rng.integers(-12, 13, size=m) / 4.0)
+    w = rng.integers(1, 7, size=int(m + (sense == 2).sum())).astype(np.int32)
+    return inst.from_triplets(f"open_{seed}", n, m, rows, cols, vals, lb, ub, np.ones(n), act + off, vt, sense, x0=x0), x0, w
+
+
+@pytest.mark.parametrize("seed", range(240))
+def test_unbounded_columns_equal_steps(chap, seed):
+    """Dyadic data (exact sums), tolerances 0, 1e-9 and a quarter (whose windows
+    between boundary and tight point hold other rows' candidates)."""
+    prob, x, w = open_bounds(seed, finite=(0.3, 1.0)[seed % 2])
+    _run_equals_steps(chap, prob, (x, w), tenure=seed % 5, feas_tol=(0.0, 1e-9, 0.25, 0.25)[seed // 2 % 4])
