@@ -77,6 +77,8 @@ struct SrShared {
     int incl[kSrRows];                  // chunks up to and with each record, inside its warp
     int nrec;
     int nlist[2];                       // stale blocks of the iteration
+    long long rev;                      // the flip back of the moved binary column against the opposite of the
+    int revc;                           // move: score and violation change (0 but for rounding)
     SrRec rec[kSrRows];
 };
 
@@ -741,9 +743,34 @@ __device__ __forceinline__ void sr_own_add(const Search &S, const SrWalk &W, SrO
     }
 }
 
+// What the flip back over a non-integral row gives beside the opposite of the
+// move (up: of the move) over it.  On an integral row, and but for rounding on
+// any, nothing: the flip back changes every half's penalty by the opposite
+// amount.  But the moved residual is rounded, and from it the flip back can
+// meet another side of the tolerance than the one the move started from (a
+// coefficient whose last place exceeds the residual's distance to it).
+__device__ __forceinline__ void sr_reverse(const SrRec &r, double a, bool up, long long &s, int &dc)
+{
+    sr_flip<true>(r.r0, r.eps, r.w1, r.w2, __double_as_longlong(a), up, s, dc);
+    sr_flip<true>(r.r1, r.eps, r.w1, r.w2, __double_as_longlong(a), !up, s, dc);
+}
+
+// The same over the moved column's records in shared memory, into sh.rev and
+// sh.revc (apart from the search's body: its live ranges cost the iterations
+// without such rows 1% otherwise).
+__device__ __noinline__ void sr_reverse_rows(const Dev &d, SrShared &sh, int nI, int len, int f0, bool up)
+{
+    const int v = threadIdx.x;
+    if (v < nI || v >= len) return;
+    long long s = 0;
+    int dc = 0;
+    sr_reverse(sh.rec[v], __ldg(d.cf_val + f0 + (v - nI)), up, s, dc);
+    if (s) atomicAdd(reinterpret_cast<unsigned long long *>(&sh.rev), (unsigned long long)s);
+    if (dc) atomicAdd(&sh.revc, dc);
+}
+
 // One entry of a binary column.  The moved column's own sums are not walked:
-// the flip back changes every half's penalty by exactly the opposite amount,
-// so they change sign.
+// they become the opposite of the move's, with sr_reverse on non-integral rows.
 template <bool FP>
 __device__ __forceinline__ void sr_entry_bin(const Search &S, const SrTeam *T, const SrLocal &L, const SrRec &r, int q,
                                              long long a, bool up, int moved)
@@ -1488,6 +1515,10 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
         L.stale[l] = st;
     }
     if (threadIdx.x < 2) sh.nlist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        sh.rev = 0;
+        sh.revc = 0;
+    }
     if (MIX) {
         // the summaries of the non-binary columns are all taken again
         for (int l = threadIdx.x; l < L.nnl; l += kSrThreads) {
@@ -1677,6 +1708,7 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
             if (!pending) {
                 finish(true, dnv);
                 if (!done) sr_walk_local<MIX>(d, S, T, L, gw, nw, W);
+                if (f1 > f0 && (!MIX || b.q < S.bc)) sr_reverse_rows(d, sh, nI, len, f0, up);
             }
         } else if (!move && !pending) {
             finish(false, 0);
@@ -1708,8 +1740,8 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
             d.x[b.var] = xnew;
             (xnew > xold ? d.tabu_dec : d.tabu_inc)[b.var] = (int)stamp;
             if (!MIX || b.q < S.bc) {
-                S.kS[b.q] = -b.s;
-                S.kD[b.q] = -dc;
+                S.kS[b.q] = sh.rev - b.s;
+                S.kD[b.q] = sh.revc - dc;
                 d.bup[b.q] = up ? 0 : 1;
                 if (pending) L.stale[own >> T.lg] = 1;
             } else {
@@ -1722,6 +1754,10 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
                     S.side[place] = (xnew > __ldg(d.lb + b.var) ? 1 : 0) | (xnew < __ldg(d.ub + b.var) ? 2 : 0);
                 }
             }
+        }
+        if (threadIdx.x == kSrThreads - 1) {
+            sh.rev = 0;
+            sh.revc = 0;
         }
     }
     __syncthreads();
@@ -1798,16 +1834,16 @@ __global__ void __launch_bounds__(kEvalThreads) k_keep_chains(const ChainSearch 
 // Record v of the pending iteration: row v of the moved column, or physical
 // row v of a weight update; false when there is nothing to change.
 __device__ __forceinline__ bool sr_big_record(const Dev &d, const Search &S, int q, int e0, int f0, int nI, int rows,
-                                              double dl, int v, SrRec &r, int &row, int &ch)
+                                              double dl, int v, SrRec &r, int &row, int &ch, double &af)
 {
     if (v >= rows) return false;
     ch = 0;
+    af = 0.0;
     if (q < 0) {
         row = v;
         return sr_bump_row(d, S, v, r);
     }
     int ai = 0;
-    double af = 0.0;
     row = sr_col_entry(d, e0, f0, nI, v, ai, af);
     ch = sr_move_row(d, S, row, ai, af, dl, (long long)dl, r, v < nI);
     return true;
@@ -1853,7 +1889,8 @@ __global__ void __launch_bounds__(kSrBigThreads) k_search_big(Dev d, Search S)
         const int g = (int)(un / sl), s = (int)(un % sl);
         SrRec r;
         int row, ch, t = 0;
-        if (sr_big_record(d, S, q, e0, f0, nI, rows, dl, 32 * g + lane, r, row, ch)) {
+        double af;
+        if (sr_big_record(d, S, q, e0, f0, nI, rows, dl, 32 * g + lane, r, row, ch, af)) {
             t = r.lenB + r.lenN;
             rec[lane] = r;
         }
@@ -1928,7 +1965,8 @@ __global__ void __launch_bounds__(kSrBigThreads) k_search_big(Dev d, Search S)
     }
 }
 
-// Writes the row states of a pending iteration, after its walk.
+// Writes the row states of a pending iteration, after its walk, and what a
+// moved binary column's own sums lack for its flip back.
 __global__ void __launch_bounds__(kSrBigThreads) k_search_put(Dev d, Search S)
 {
     if (!S.sc->pending) return;
@@ -1942,15 +1980,20 @@ __global__ void __launch_bounds__(kSrBigThreads) k_search_put(Dev d, Search S)
         rows = nI + d.cf_ptr[q + 1] - f0;
         dl = __dsub_rn(d.ctl->mv_new, d.ctl->mv_old);
     }
-    int sum = 0;
+    int sum = 0, rd = 0;
+    long long rs = 0;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < rows; v += gridDim.x * blockDim.x) {
         SrRec r;
         int row, ch;
-        if (!sr_big_record(d, S, q, e0, f0, nI, rows, dl, v, r, row, ch)) continue;
+        double af;
+        if (!sr_big_record(d, S, q, e0, f0, nI, rows, dl, v, r, row, ch, af)) continue;
         if (q < 0) sr_put_weights(d, row, r);
         else sr_put_row(d, S, row, r, ch);
+        if (q >= 0 && q < S.bc && !r.integral) sr_reverse(r, af, dl > 0.0, rs, rd);
         sum += ch;
     }
+    if (rs) atomicAdd(reinterpret_cast<unsigned long long *>(S.kS + q), (unsigned long long)rs);
+    if (rd) atomicAdd(S.kD + q, rd);
     sum = __reduce_add_sync(FULLMASK, sum);
     if ((threadIdx.x & 31) == 0 && sum) atomicAdd(reinterpret_cast<unsigned long long *>(&S.sc->dnv), (unsigned long long)(long long)sum);
 }

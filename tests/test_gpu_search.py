@@ -304,3 +304,46 @@ def test_unbounded_columns_equal_steps(chap, seed):
     between boundary and tight point hold other rows' candidates)."""
     prob, x, w = open_bounds(seed, finite=(0.3, 1.0)[seed % 2])
     _run_equals_steps(chap, prob, (x, w), tenure=seed % 5, feas_tol=(0.0, 1e-9, 0.25, 0.25)[seed // 2 % 4])
+
+
+def test_reverse_flip_on_an_absorbed_residual(chap):
+    """feas_tol 0: 0.1 x + 0.2 y + z <= 0.3 (weight 3) with x = y = 1 fixed has
+    residual 5.6e-17 at z = 0, violated; z >= 1 (weight 2).  z rises with score
+    -3 + 4; at z = 1 the first row's residual rounds to 1, and back at 0 it is
+    satisfied: the flip back scores 6 - 4, not -1."""
+    prob = inst.from_triplets("absorbed", 3, 2, [0, 0, 0, 1], [0, 1, 2, 2], [0.1, 0.2, 1.0, 1.0], [1.0, 1.0, 0.0],
+                              [1.0, 1.0, 1.0], [1.0] * 3, [0.3, 1.0], [inst.VAR_BIN] * 3, [inst.ROW_LE, inst.ROW_GE],
+                              x0=[1.0, 1.0, 0.0])
+    st = _run_equals_steps(chap, prob, (np.array([1.0, 1.0, 0.0]), np.array([3, 2], np.int32)), feas_tol=0.0, iters=(2,))
+    assert st["x"].tolist() == [1.0, 1.0, 0.0] and st["moves"] == 2
+
+
+def absorbing_rows(seed, n, m, k):
+    """Binary rows of decimal coefficients, some of them with one coefficient of
+    1e8 whose rounding exceeds the tolerance; many rows tight at a hidden point."""
+    rng = np.random.default_rng(seed)
+    xs = rng.integers(0, 2, size=n).astype(float)
+    rows, cols, vals, rhs = [], [], [], []
+    sense = rng.choice([0, 1, 2], size=m, p=[0.4, 0.4, 0.2]).astype(np.uint8)
+    for i in range(m):
+        js = np.sort(rng.choice(n, size=min(k, n), replace=False))
+        a = rng.integers(1, 30, size=len(js)) * np.where(rng.random(len(js)) < 0.5, -0.1, 0.1)
+        if i % 3 == 0:
+            a[rng.integers(0, len(js))] = rng.choice([-1e8, 1e8])
+        rows.append(np.full(len(js), i)); cols.append(js); vals.append(a)
+        rhs.append(float(a[::-1] @ xs[js[::-1]]) + rng.choice([0.0, 0.0, 5e-9, -5e-9, 0.3]))
+    return inst.from_triplets("absorb", n, m, np.concatenate(rows), np.concatenate(cols), np.concatenate(vals), np.zeros(n),
+                              np.ones(n), np.ones(n), np.array(rhs), np.full(n, inst.VAR_BIN), sense, x0=xs)
+
+
+@pytest.mark.parametrize("feas_tol", [0.0, 1e-9])
+@pytest.mark.parametrize("n,m,k", [(40, 30, 5), (500, 400, 6), (600, 60, 400), (700, 600, 500)])
+def test_reverse_flips_on_rounded_rows(chap, n, m, k, feas_tol):
+    """Every form in which a move is applied: one CTA, a cluster, the whole GPU
+    (more rows than one record list)."""
+    for seed in range(4):
+        prob = absorbing_rows(seed, n, m, k)
+        rng = np.random.default_rng(seed)
+        x = np.where(rng.random(n) < 0.05, 1.0 - prob.x0, prob.x0)
+        w = rng.integers(1, 5, size=int(m + (prob.sense == 2).sum())).astype(np.int32)
+        _run_equals_steps(chap, prob, (x, w), tenure=seed, feas_tol=feas_tol, iters=(1, 2, 37, 60))
