@@ -840,7 +840,9 @@ __device__ __forceinline__ void learn_select(const Dev &d, const Learn &L)
 
 // Flip score of every listed binary variable (8 lanes per variable, as the
 // exact binary kernel); the best admissible positive flip is folded into
-// lc->key with one 64-bit atomicMax (larger score, then lower variable).
+// lc->key with one 64-bit atomicMax (larger score, then lower variable).  Row
+// states are read through L2: the apply kernel before may still be writing them
+// when this one starts.
 // select: the last CTA hands the move to the apply kernel.
 __global__ void __launch_bounds__(256) k_subset_eval(Dev d, Learn L, int k, int select, int gate)
 {
@@ -869,7 +871,7 @@ __global__ void __launch_bounds__(256) k_subset_eval(Dev d, Learn L, int k, int 
                 const int v = v0 + sub;
                 if (v < len) {
                     const int e = e0 + v;
-                    const int4 st = __ldg(reinterpret_cast<const int4 *>(d.rs + d.ci_row[e]));
+                    const int4 st = __ldcg(reinterpret_cast<const int4 *>(d.rs + d.ci_row[e]));
                     const long long r = i4_r(st);
                     const int ad = up ? d.ci_val[e] : -d.ci_val[e];
                     const long long r1 = r + ad;
@@ -892,17 +894,19 @@ __global__ void __launch_bounds__(256) k_subset_eval(Dev d, Learn L, int k, int 
                 const int v = v0 + sub;
                 if (v < len) {
                     const int e = e0 + v;
-                    const RowState st = d.rs[d.cf_row[e]];
+                    const int4 *st = reinterpret_cast<const int4 *>(d.rs + d.cf_row[e]);
+                    const int4 s0 = __ldcg(st), s1 = __ldcg(st + 1);
                     const long long ab = __double_as_longlong(d.cf_val[e]);
                     const long long ad = up ? ab : flip_sign(ab);
-                    const long long m1 = __double_as_longlong(st.m1), m2 = __double_as_longlong(st.m2);
+                    const long long m1 = i4_r(s1);
+                    const long long m2 = (long long)(((unsigned long long)(unsigned)s1.w << 32) | (unsigned)s1.z);
                     const bool neg = ad < 0;
                     const bool v0b = m1 < 0, v1b = dkey_bits(ad) > dkey_bits(m1);
-                    s += (long long)lflip_f(v0b, v1b, neg) * st.w1;
+                    s += (long long)lflip_f(v0b, v1b, neg) * s0.z;
                     dc += (int)v1b - (int)v0b;
-                    if (st.w2 >= 0) {
+                    if (s0.w >= 0) {
                         const bool u0 = m2 < 0, u1 = dkey_bits(flip_sign(ad)) > dkey_bits(m2);
-                        s += (long long)lflip_f(u0, u1, !neg) * st.w2;
+                        s += (long long)lflip_f(u0, u1, !neg) * s0.w;
                         dc += (int)u1 - (int)u0;
                     }
                 }
