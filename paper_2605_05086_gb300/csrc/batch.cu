@@ -477,6 +477,13 @@ __global__ void k_chain_load(BDev d, const chap::ChainSearch *chains)
     }
 }
 
+// Chains whose own search is done.
+__global__ void k_chain_count(int n, const chap::ChainSearch *chains, unsigned *count)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < n && chains[c].d.ctl->done) atomicAdd(count, 1u);
+}
+
 // And back.
 __global__ void k_chain_store(BDev d, const chap::ChainSearch *chains)
 {
@@ -497,7 +504,6 @@ __global__ void k_chain_store(BDev d, const chap::ChainSearch *chains)
         b.t_feas_ns = k.t_feas_ns;
         b.best_key = 0ull;
         b.bump = 0;
-        if (k.done && !b.done) atomicAdd(d.n_done, 1u);
         b.done = k.done;
     }
     // a warp per 32 variables: its ballot is a word of the bitset
@@ -1071,10 +1077,21 @@ chap_status chap_batch_run(chap_batch *b, int64_t max_iters, int32_t stop_at_fea
     BCK(b, cudaGetLastError(), "begin run");
     if (b->resident) {
         // every chain runs to its end on its own: launches of kChainIters
-        // iterations until all are done
+        // iterations until all are done.  The done chains are counted before
+        // another launch is queued, not after the last one (a launch is 30 ms and
+        // more, the count and its wait 20 us).
         BCK(b, launch_chains_load(b), "load chains");
-        for (long long left = max_iters; left > 0; left -= kChainIters)
+        for (long long left = max_iters; left > 0;) {
             BCK(b, chap::launch_chain_search(b->chains, b->n_chains, b->chain_smem, kChainIters, b->st), "chain search");
+            left -= kChainIters;
+            if (left <= 0) break;
+            BCK(b, cudaMemsetAsync(b->dev.n_done, 0, sizeof(unsigned int), b->st), "reset done count");
+            k_chain_count<<<(b->n_chains + 255) / 256, 256, 0, b->st>>>(b->n_chains, b->chains, b->dev.n_done);
+            BCK(b, cudaGetLastError(), "count done chains");
+            BCK(b, cudaMemcpyAsync(b->h_done, b->dev.n_done, sizeof(unsigned int), cudaMemcpyDeviceToHost, b->st), "read done");
+            BCK(b, cudaStreamSynchronize(b->st), "synchronise");
+            if (*b->h_done >= (unsigned)b->n_chains) break;
+        }
         BCK(b, launch_chains_store(b), "store chains");
         BCK(b, cudaStreamSynchronize(b->st), "synchronise");
     } else {

@@ -150,3 +150,32 @@ def test_persistent_barrier_wait_runs_out(chap):
         r, st = single_run(chap, probs[k], t, 100, False)
         assert res[c].moves == st["moves"] and np.array_equal(b.x(c), st["x"]), c
     b.close()
+
+
+def test_a_batch_that_is_done_queues_no_more_launches(chap):
+    """Chains that are feasible after a few hundred iterations end the run under
+    any limit: 2e10 iterations (2.4 million launches) take what 20,000 take (two
+    seconds are the bound; the empty launches alone took more)."""
+    probs = [inst.gen_setcover(seed=5, n=300, m=150, k=6), inst.gen_setcover(seed=6, n=1300, m=700, k=8)]
+    seen = []
+    for limit in (20_000, 20_000_000_000):
+        b = chap.BatchChains(probs, [0, 1, 1], [10, 10, 3])
+        res, seconds = b.run(max_iters=limit, stop_at_feasible=True)
+        assert all(r.final_nviol == 0 and 0 < r.feasible_iter < 20_000 for r in res) and seconds < 2.0
+        seen.append([(r.iters, r.moves) for r in res])
+        b.close()
+    assert seen[0] == seen[1]
+
+
+def test_a_done_chain_does_not_end_the_others(chap):
+    """One chain feasible at the start of the second launch, one that never is:
+    the run goes on to its limit."""
+    easy = inst.gen_setcover(seed=5, n=300, m=150, k=6)
+    never = inst.from_triplets("never", 2, 2, [0, 0, 1, 1], [0, 1, 0, 1], [1.0] * 4, np.zeros(2), np.ones(2), np.ones(2),
+                               np.array([3.0, 1.0]), np.full(2, inst.VAR_BIN), [inst.ROW_GE, inst.ROW_LE], x0=np.zeros(2))
+    b = chap.BatchChains([easy, never], [0, 1], [10, 2])
+    res, _ = b.run(max_iters=20_000, stop_at_feasible=True)
+    assert res[0].final_nviol == 0 and res[0].iters < 8192 and res[1].iters == 20_000
+    r, _ = single_run(chap, never, 2, 20_000, True)
+    assert (res[1].moves, res[1].best_nviol) == (r.moves, r.best_nviol)
+    b.close()
