@@ -1457,7 +1457,8 @@ __device__ __noinline__ void sr_evaluate(const Dev &d, const Search &S, const Sr
 // general MIP of 200k variables 35 us against 142, of 21k variables near a
 // feasible point 31 us against 110, 2M skewed columns with 50 dense ones (every
 // move a dense one, done by the whole GPU) 205 us against 410 (16 CTAs).
-template <bool MIX>
+// FPROWS: there may be non-integral rows.
+template <bool MIX, bool FPROWS>
 __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int nct, int max_launch,
                                             unsigned char *sr_smem)
 {
@@ -1708,7 +1709,7 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
             if (!pending) {
                 finish(true, dnv);
                 if (!done) sr_walk_local<MIX>(d, S, T, L, gw, nw, W);
-                if (f1 > f0 && (!MIX || b.q < S.bc)) sr_reverse_rows(d, sh, nI, len, f0, up);
+                if (FPROWS && f1 > f0 && (!MIX || b.q < S.bc)) sr_reverse_rows(d, sh, nI, len, f0, up);
             }
         } else if (!move && !pending) {
             finish(false, 0);
@@ -1740,8 +1741,8 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
             d.x[b.var] = xnew;
             (xnew > xold ? d.tabu_dec : d.tabu_inc)[b.var] = (int)stamp;
             if (!MIX || b.q < S.bc) {
-                S.kS[b.q] = sh.rev - b.s;
-                S.kD[b.q] = sh.revc - dc;
+                S.kS[b.q] = (FPROWS ? sh.rev : 0) - b.s;
+                S.kD[b.q] = (FPROWS ? sh.revc : 0) - dc;
                 d.bup[b.q] = up ? 0 : 1;
                 if (pending) L.stale[own >> T.lg] = 1;
             } else {
@@ -1755,7 +1756,7 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
                 }
             }
         }
-        if (threadIdx.x == kSrThreads - 1) {
+        if (FPROWS && threadIdx.x == kSrThreads - 1) {
             sh.rev = 0;
             sh.revc = 0;
         }
@@ -1798,7 +1799,7 @@ template <bool MIX>
 __global__ void __launch_bounds__(kSrThreads, 1) k_search(Dev d, Search S, int nct, int max_launch)
 {
     extern __shared__ __align__(16) unsigned char sr_smem[];
-    search_body<MIX>(d, S, nct, max_launch, sr_smem);
+    search_body<MIX, true>(d, S, nct, max_launch, sr_smem);
 }
 
 // Many independent searches (the chains of a batch), one CTA each: no barrier
@@ -1815,7 +1816,7 @@ __global__ void __launch_bounds__(kSrThreads, 1) k_search_chains(const ChainSear
     for (int i = threadIdx.x; i < (int)(sizeof(ChainSearch) / sizeof(int)); i += kSrThreads)
         reinterpret_cast<int *>(&c)[i] = src[i];
     __syncthreads();
-    search_body<false>(c.d, c.S, 1, max_launch, sr_smem);
+    search_body<false, false>(c.d, c.S, 1, max_launch, sr_smem);
 }
 
 // Kept values of every chain that is not done: blockIdx.y = chain.
