@@ -410,13 +410,16 @@ __global__ void k_batch_begin(BDev d, long long max_iters, int stop_at_feasible)
     if (ctl->done) atomicAdd(d.n_done, 1u);
 }
 
-// Initial row states of every chain from its instance's (blockIdx.y = chain).
+// Initial row states of every chain from its instance's (grid.y strides over
+// the chains, as below: a grid has 65,535 rows at most).
 __global__ void k_batch_reset_rows(BDev d, const BRow *rows0, const long long *inst_row0)
 {
-    const int c = blockIdx.y, k = d.ch_inst[c];
-    const int4 *src = reinterpret_cast<const int4 *>(rows0 + inst_row0[k]);
-    int4 *dst = reinterpret_cast<int4 *>(d.rs + d.ch_roff[c]);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.inst_m[k]; i += gridDim.x * blockDim.x) dst[i] = src[i];
+    for (int c = blockIdx.y; c < d.n_chains; c += gridDim.y) {
+        const int k = d.ch_inst[c];
+        const int4 *src = reinterpret_cast<const int4 *>(rows0 + inst_row0[k]);
+        int4 *dst = reinterpret_cast<int4 *>(d.rs + d.ch_roff[c]);
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.inst_m[k]; i += gridDim.x * blockDim.x) dst[i] = src[i];
+    }
 }
 
 // The search's row store of one instance from its column store: entry of
@@ -441,11 +444,10 @@ __global__ void k_chain_entries(int n, const int *cptr, const int *crow, const i
         head[(size_t)q * chap::kSrHead + t] = e0 + t < e1 ? make_int2(crow[e0 + t], cval[e0 + t]) : make_int2(0, 0);
 }
 
-// Chain states from the batch's: row states, x as doubles and flip bytes, the
-// control block (blockIdx.y = chain).
-__global__ void k_chain_load(BDev d, const chap::ChainSearch *chains)
+// A chain's state from the batch's: row states, x as doubles and flip bytes, the
+// control block.
+__device__ __forceinline__ void chain_load(const BDev &d, const chap::ChainSearch *chains, int c)
 {
-    const int c = blockIdx.y;
     const BCtl &b = d.ctl[c];
     const chap::Dev &D = chains[c].d;
     const long long xoff = d.ch_xoff[c];
@@ -477,6 +479,11 @@ __global__ void k_chain_load(BDev d, const chap::ChainSearch *chains)
     }
 }
 
+__global__ void k_chain_load(BDev d, const chap::ChainSearch *chains)
+{
+    for (int c = blockIdx.y; c < d.n_chains; c += gridDim.y) chain_load(d, chains, c);
+}
+
 // Chains whose own search is done.
 __global__ void k_chain_count(int n, const chap::ChainSearch *chains, unsigned *count)
 {
@@ -485,9 +492,8 @@ __global__ void k_chain_count(int n, const chap::ChainSearch *chains, unsigned *
 }
 
 // And back.
-__global__ void k_chain_store(BDev d, const chap::ChainSearch *chains)
+__device__ __forceinline__ void chain_store(const BDev &d, const chap::ChainSearch *chains, int c)
 {
-    const int c = blockIdx.y;
     BCtl &b = d.ctl[c];
     const chap::Dev &D = chains[c].d;
     const long long xoff = d.ch_xoff[c];
@@ -516,6 +522,11 @@ __global__ void k_chain_store(BDev d, const chap::ChainSearch *chains)
         const int4 v = *reinterpret_cast<const int4 *>(D.rs + i);
         *reinterpret_cast<int4 *>(rs + i) = v;
     }
+}
+
+__global__ void k_chain_store(BDev d, const chap::ChainSearch *chains)
+{
+    for (int c = blockIdx.y; c < d.n_chains; c += gridDim.y) chain_store(d, chains, c);
 }
 
 }  // namespace
@@ -813,7 +824,7 @@ void make_chains(chap_batch *b, const chap_problem *probs, const std::vector<int
 
 cudaError_t launch_chains_load(const chap_batch *b)
 {
-    k_chain_load<<<dim3(8, b->n_chains), 256, 0, b->st>>>(b->dev, b->chains);
+    k_chain_load<<<dim3(8, chap::chain_rows(b->n_chains)), 256, 0, b->st>>>(b->dev, b->chains);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = chap::launch_chain_keep(b->chains, b->n_chains, b->max_n, b->st);
     return e;
@@ -821,7 +832,7 @@ cudaError_t launch_chains_load(const chap_batch *b)
 
 cudaError_t launch_chains_store(const chap_batch *b)
 {
-    k_chain_store<<<dim3(8, b->n_chains), 256, 0, b->st>>>(b->dev, b->chains);
+    k_chain_store<<<dim3(8, chap::chain_rows(b->n_chains)), 256, 0, b->st>>>(b->dev, b->chains);
     return cudaGetLastError();
 }
 
@@ -833,7 +844,7 @@ chap_status upload_state(chap_batch *b)
     BCK(b, cudaMemsetAsync(b->dev.bar, 0, sizeof(GridBar), b->st), "reset barrier");
     BCK(b, cudaMemsetAsync(b->dev.tinc, 0, sizeof(int) * std::max<long long>(b->total_x, 1), b->st), "reset tabu");
     BCK(b, cudaMemsetAsync(b->dev.tdec, 0, sizeof(int) * std::max<long long>(b->total_x, 1), b->st), "reset tabu");
-    k_batch_reset_rows<<<dim3(8, b->n_chains), 256, 0, b->st>>>(b->dev, b->rows0, b->inst_row0);
+    k_batch_reset_rows<<<dim3(8, chap::chain_rows(b->n_chains)), 256, 0, b->st>>>(b->dev, b->rows0, b->inst_row0);
     BCK(b, cudaGetLastError(), "reset row states");
     BCK(b, cudaMemcpyAsync(b->dev.ctl, b->ctl0.data(), sizeof(BCtl) * b->ctl0.size(), cudaMemcpyHostToDevice, b->st),
         "upload control");

@@ -527,6 +527,7 @@ cudaError_t launch_search(const Dev &d, const Search &S, int max_launch, cudaStr
 // CTA), kept values, up to max_launch iterations.  max_n: most variables of a
 // chain; smem: most shared memory.
 bool chain_shape(Search &S);
+inline int chain_rows(int n) { return n < 65535 ? n : 65535; }   // grid.y of a kernel over n chains
 cudaError_t launch_chain_keep(const ChainSearch *chains, int n, int max_n, cudaStream_t st);
 cudaError_t launch_chain_search(const ChainSearch *chains, int n, int smem, int max_launch, cudaStream_t st);
 // Chooses S.nct (one CTA, or the largest cluster that fits the current device)

@@ -3919,7 +3919,7 @@ cudaError_t launch_chain_keep(const ChainSearch *chains, int n, int max_n, cudaS
 {
     // 4 lanes a column, a few CTAs per chain
     const int gx = std::max(1, std::min(16, (max_n + 2047) / 2048));
-    k_keep_chains<4><<<dim3(gx, n), kEvalThreads, 0, st>>>(chains);
+    k_keep_chains<4><<<dim3(gx, chain_rows(n)), kEvalThreads, 0, st>>>(chains, n);
     return cudaGetLastError();
 }
 

@@ -1819,15 +1819,17 @@ __global__ void __launch_bounds__(kSrThreads, 1) k_search_chains(const ChainSear
     search_body<false, false>(c.d, c.S, 1, max_launch, sr_smem);
 }
 
-// Kept values of every chain that is not done: blockIdx.y = chain.
+// Kept values of every chain that is not done (grid.y strides over the chains).
 template <int G>
-__global__ void __launch_bounds__(kEvalThreads) k_keep_chains(const ChainSearch *chains)
+__global__ void __launch_bounds__(kEvalThreads) k_keep_chains(const ChainSearch *chains, int n)
 {
-    const ChainSearch &c = chains[blockIdx.y];
-    if (c.d.ctl->done) return;
-    keep_bin<G>(c.d, c.S);
-    for (int b = blockIdx.x; b < c.S.nvb; b += gridDim.x) keep_rows(c.d, c.S, b);
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < c.S.nblk; b += gridDim.x * blockDim.x) c.S.bdirty[b] = 1;
+    for (int k = blockIdx.y; k < n; k += gridDim.y) {
+        const ChainSearch &c = chains[k];
+        if (c.d.ctl->done) continue;
+        keep_bin<G>(c.d, c.S);
+        for (int b = blockIdx.x; b < c.S.nvb; b += gridDim.x) keep_rows(c.d, c.S, b);
+        for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < c.S.nblk; b += gridDim.x * blockDim.x) c.S.bdirty[b] = 1;
+    }
 }
 
 // ------------------------------------- an iteration applied by the whole GPU

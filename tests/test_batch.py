@@ -179,3 +179,22 @@ def test_a_done_chain_does_not_end_the_others(chap):
     r, _ = single_run(chap, never, 2, 20_000, True)
     assert (res[1].moves, res[1].best_nviol) == (r.moves, r.best_nviol)
     b.close()
+
+
+def test_more_chains_than_a_grid_has_rows(chap):
+    """70,000 chains on the default schedule: created, run, reset and run again;
+    chains of one instance and tenure agree wherever they lie."""
+    probs = [inst.gen_setcover(seed=3, n=24, m=20, k=4), binary_mixed(4, 20, 12, k=3)]
+    n = 70_000
+    b = chap.BatchChains(probs, [k % 2 for k in range(n)], [(0, 0, 5, 5)[k % 4] for k in range(n)])
+    for _ in range(2):
+        res, _ = b.run(max_iters=40, stop_at_feasible=False)
+        got = np.array([(r.iters, r.moves, r.final_nviol, r.best_nviol) for r in res])
+        for c in range(4):
+            assert (got[c::4] == got[c]).all()
+            _, st = single_run(chap, probs[c % 2], (0, 0, 5, 5)[c], 40, False)
+            assert got[c].tolist() == [40, st["moves"], st["nviol"], st["best_nviol"]]
+            for far in (c, 65_532 + c, n - 4 + c):
+                assert np.array_equal(b.x(far), st["x"])
+        b.reset()
+    b.close()
