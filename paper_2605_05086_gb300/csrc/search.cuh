@@ -1826,6 +1826,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_keep_chains(const ChainSearch 
     for (int k = blockIdx.y; k < n; k += gridDim.y) {
         const ChainSearch &c = chains[k];
         if (c.d.ctl->done) continue;
+        if (c.S.nvb == 0 && blockIdx.x == 0 && threadIdx.x == 0) *c.S.sc = SrCtl{};   // keep_rows does it where there are rows
         keep_bin<G>(c.d, c.S);
         for (int b = blockIdx.x; b < c.S.nvb; b += gridDim.x) keep_rows(c.d, c.S, b);
         for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < c.S.nblk; b += gridDim.x * blockDim.x) c.S.bdirty[b] = 1;

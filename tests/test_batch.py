@@ -198,3 +198,25 @@ def test_more_chains_than_a_grid_has_rows(chap):
                 assert np.array_equal(b.x(far), st["x"])
         b.reset()
     b.close()
+
+
+def test_instance_without_rows(chap):
+    """A row-less instance beside another, on device memory that held other data:
+    nothing is violated, no flip has a score, every iteration is a weight update."""
+    import torch
+    junk = torch.full((1 << 28,), 0x01010101, dtype=torch.int32, device="cuda")
+    del junk
+    torch.cuda.empty_cache()
+    empty = inst.from_triplets("rowless", 40, 0, [], [], [], np.zeros(40), np.ones(40), np.ones(40), [],
+                               np.full(40, inst.VAR_BIN), [], x0=np.zeros(40))
+    other = inst.gen_setcover(seed=3, n=24, m=20, k=4)
+    b = chap.BatchChains([other, empty], [0, 1, 1], [0, 0, 5])
+    for again in range(2):
+        res, _ = b.run(max_iters=25, stop_at_feasible=False)
+        for c in (1, 2):
+            assert (res[c].iters, res[c].moves, res[c].final_nviol, res[c].best_nviol) == (25 * (again + 1), 0, 0, 0)
+            assert not b.x(c).any()
+    b.reset()
+    res, _ = b.run(max_iters=25, stop_at_feasible=True)
+    assert [r.iters for r in res[1:]] == [0, 0] and [r.feasible_iter for r in res[1:]] == [0, 0]
+    b.close()
