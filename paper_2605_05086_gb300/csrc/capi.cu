@@ -1158,8 +1158,8 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     in.n_long_cols = (int)(lcols.size() + rcols.size());
     in.n_cta_cols = n_tc;
     // evaluation kernels (they also select the move), a selection kernel only
-    // when none runs, the move apply and the weight bump
-    in.launches_per_step = (n_tb > 0) + (bin_blk ? 1 : 0) + (n_tn > 0) + (n_tc > 0) + (!tiles_hist.empty()) + (n_bb == 0) + 2 +
+    // when none runs, and the apply kernel (move or weight update)
+    in.launches_per_step = (n_tb > 0) + (bin_blk ? 1 : 0) + (n_tn > 0) + (n_tc > 0) + (!tiles_hist.empty()) + (n_bb == 0) + 1 +
                            (lazy ? 2 : 0) +   // kept binary scores: the scan and the marking kernel
                            (has_long ? 3 + long_rounds : 0) + (rcols.empty() ? 0 : 2);   // long lists: generation, merges, tile sums, scan
     // algorithmic bytes of one pass: every nonzero once (row + coefficient),
