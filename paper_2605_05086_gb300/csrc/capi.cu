@@ -645,7 +645,8 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     }
     // long lists: runs of kLongRun sorted entries per chunk of kLongChunk
     // nonzeros, padded to a power of two runs per column
-    // (columns of at most kRkMaxRuns runs of kRkChunk nonzeros are ranked)
+    // (columns of at most rank_max_runs runs of kRkChunk nonzeros are ranked)
+    const int max_rank_runs = rank_max_runs(kind_base[T_NB_LONG + 1] - kind_base[T_NB_LONG]);
     std::vector<LongCol> lcols;
     std::vector<RankCol> rcols;
     std::vector<Tile> tiles_rgen;
@@ -659,7 +660,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         lc.e_mid = ci_ptr[q + 1] - ci_ptr[q];
         lc.e_end = lc.e_mid + (cf_ptr[q + 1] - cf_ptr[q]);
         const int rk = (lc.e_end + kRkChunk - 1) / kRkChunk;
-        if (rk <= kRkMaxRuns) {
+        if (rk <= max_rank_runs) {
             RankCol rc{};
             rc.pos = q;
             rc.len = lc.e_end;

@@ -547,7 +547,14 @@ constexpr int kRbThreads = 1024;
 constexpr int kRkChunk = 508;          // nonzeros of a ranked run: <= 4 entries each, + 2 bounds
 constexpr int kRkRun = 2048;           // entries of a ranked run at most (power of two)
 constexpr int kRkThreads = 512;
-constexpr int kRkMaxRuns = 64;         // runs of a ranked column at most (longer columns are merged)
+// Runs of a ranked column at most (longer columns are merged): 47 and one for
+// every long column, up to kRkMaxRuns.  A ranked column's time grows with its
+// runs, a merged one's with the number of columns: one column of 20,000 / 24,000 /
+// 28,000 / 32,000 entries 160 / 179 / 195 / 212 us a pass ranked and 179 at all four
+// merged; 8 columns 275 / 305 / 364 / 407 against 375 to 385; 24 columns 515 / 627 /
+// 815 / 960 against 970.
+constexpr int kRkMaxRuns = 64;
+inline int rank_max_runs(int columns) { return columns < kRkMaxRuns - 47 ? 47 + columns : kRkMaxRuns; }
 constexpr int kLongChunk = 1020;       // nonzeros per generating CTA: <= 4 entries each, + 2 bounds
 constexpr int kLongRun = 4096;         // entries of one sorted run (power of two)
 constexpr int kLongThreads = 512;

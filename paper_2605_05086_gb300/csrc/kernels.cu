@@ -2473,7 +2473,7 @@ __global__ void __launch_bounds__(kLongThreads) k_long_eval(Dev d, const SEntry 
     finish_pass(d);
 }
 
-// -------------------------------------- ranked long lists (up to kRkMaxRuns runs)
+// -------------------------------------- ranked long lists (up to rank_max_runs)
 //
 // The same lists without a merge: k_rank_gen (one CTA per kRkChunk nonzeros)
 // sorts its entries in registers and writes the run with the prefix sums of
@@ -2482,9 +2482,7 @@ __global__ void __launch_bounds__(kLongThreads) k_long_eval(Dev d, const SEntry 
 // shared memory).  Two launches, 34 and 57 us, instead of a generation, log2
 // of the runs merge rounds, tile sums and a scan: 7 columns of 9,000 rows, 221
 // -> 131 us a pass.  The searches grow with entries x runs and the merge rounds
-// with entries x log(runs): at 64 runs (32,512 nonzeros) a thread's searches
-// are 700 steps in shared memory against 8 launches of 13 dependent loads from
-// L2; longer columns are merged.
+// with entries x log(runs): columns of more than rank_max_runs runs are merged.
 
 // Strict order of two entries of a ranked run: (t, class, entry), one
 // comparison for both partners of an exchange.

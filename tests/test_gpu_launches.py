@@ -20,13 +20,13 @@ def chap():
     return c
 
 
-def long_column(rows):
-    """One continuous column in every row, beside 40 others."""
+def long_column(rows, count=1):
+    """`count` continuous columns in every row, beside 40 others."""
     rng = np.random.default_rng(rows)
-    n = 41
-    r = np.repeat(np.arange(rows), 2)
-    c = np.stack([np.zeros(rows, int), rng.integers(1, n, size=rows)], axis=1).ravel()
-    return inst.from_triplets("long", n, rows, r, c, rng.standard_normal(2 * rows), np.zeros(n), np.full(n, 50.0), np.ones(n),
+    n = count + 40
+    r = np.repeat(np.arange(rows), count + 1)
+    c = np.concatenate([np.tile(np.arange(count), (rows, 1)), rng.integers(count, n, size=(rows, 1))], axis=1).ravel()
+    return inst.from_triplets("long", n, rows, r, c, rng.standard_normal(len(r)), np.zeros(n), np.full(n, 50.0), np.ones(n),
                               rng.standard_normal(rows) * 20, np.full(n, inst.VAR_CONT), np.zeros(rows, np.uint8))
 
 
@@ -38,6 +38,11 @@ CASES = {
     "counting": (lambda: inst.gen_skewed(seed=6, n=40_000, m=20_000, n_dense=6, dense_len=6_000), {}, 5),
     "ranked": (lambda: long_column(9_000), {}, 4),
     "merged": (lambda: long_column(40_000), {}, 11),   # 40 chunks: 6 merge rounds
+    # 48 runs are ranked where there is one long column, 64 where there are 17
+    "ranked_longest": (lambda: long_column(24_384), {}, 4),
+    "merged_shortest": (lambda: long_column(24_385), {}, 10),
+    "ranked_longest_17": (lambda: long_column(32_512, 17), {}, 4),
+    "merged_shortest_17": (lambda: long_column(32_513, 17), {}, 10),
 }
 
 

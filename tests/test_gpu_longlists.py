@@ -152,10 +152,11 @@ def _integer_column_best(prob, x, j):
     return (cand[k], int(s[k]), int(n[k])) if s[k] > 0 else (xb, 0, 0)
 
 
-@pytest.mark.parametrize("rows", [9_000, 32_512, 32_513])
+@pytest.mark.parametrize("rows", [9_000, 24_384, 24_385, 32_512, 32_513])
 def test_ranked_and_merged_lists(chap, rows):
-    """The longest list that is ranked (64 runs of 508 nonzeros), the shortest
-    that is merged, and an ordinary one."""
+    """The longest list of a single long column that is ranked (48 runs of 508
+    nonzeros), the shortest that is merged, two of 32 chunks and an ordinary
+    one."""
     prob = long_instance(9, [I], rows_per_long=rows, n_other=40, eq_frac=0.0)
     bs = chap.BestShift(prob, tenure=3, feas_tol=0.0)
     assert bs.info.n_long_cols == 1
