@@ -465,8 +465,8 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     }
     h->m_norm = mn;
 
-    // rows of the residual kernel: the short integral ones in index order (32 to a
-    // warp), the long ones by decreasing length (a warp each), then the others by
+    // rows of the residual kernel: the short integral ones, where there are many, in
+    // index order (32 to a warp), the long ones by decreasing length (a warp each), then the others by
     // decreasing length (32 rows of like length per CTA)
     std::vector<int> res_rows;
     res_rows.reserve(m);
@@ -474,7 +474,8 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         if (rint[i]) res_rows.push_back(i);
     const int n_res_int = (int)res_rows.size();
     auto row_len = [&](int i) { return p->row_ptr[i + 1] - p->row_ptr[i]; };
-    const auto res_long = std::stable_partition(res_rows.begin(), res_rows.end(), [&](int i) { return row_len(i) <= kResShort; });
+    const auto res_long = std::stable_partition(res_rows.begin(), res_rows.end(),
+                                                [&](int i) { return n_res_int > kResGroupMin && row_len(i) <= kResShort; });
     const int n_res_short = (int)(res_long - res_rows.begin());
     std::stable_sort(res_long, res_rows.end(), [&](int a, int b) { return row_len(a) > row_len(b); });
     for (int i = 0; i < m; ++i)

@@ -586,7 +586,13 @@ constexpr double kSrOneCtaTouched = 4096.0;
 constexpr long long kSrHistNnz = 2000000;
 constexpr int kSrHistNear = 16;
 constexpr int kCheckDevice = 1 << 14;    // variables from which a host state is checked on the device
-constexpr int kResShort = 64;            // entries up to which integral rows share a warp in the residual kernel
+constexpr int kResShort = 64;            // entries up to which integral rows share a warp in the residual kernel,
+// where there are more rows than its grid has warps (456 CTAs of 16): a row's
+// entries are then read in up to 8 rounds of 8 lanes instead of 2 of 32, which
+// only saves where warps are short (set_state of 5k / 8k / 16k general variables,
+// 1.2k to 4k integral rows, 69 / 74 / 101 us with shared warps, 56 / 64 / 91 without;
+// of 30k and more the same; 100,000 rows of 8 entries 12 us against 63).
+constexpr int kResGroupMin = 456 * 16;
 constexpr int kSrHead = 8;              // integral column entries addressed by position
 constexpr int kSrLaunchIters = 2048;    // iterations of one launch of the search
 constexpr int kSrBlkPos = 256;          // positions (and physical rows) of one summary block

@@ -972,13 +972,6 @@ __global__ void __launch_bounds__(kBlkFinThreads) k_bin_blk_final(Dev d, BinBlk 
     finish_pass(d);
 }
 
-// Flip direction of every binary position from x (after a new state).
-__global__ void k_bup_init(Dev d)
-{
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < d.n_bup; q += gridDim.x * blockDim.x)
-        d.bup[q] = __double_as_longlong(d.x[__ldg(d.var_list + q)]) == 0 ? 1 : 0;
-}
-
 // Selective re-evaluation of the binary flips.  k_eval_bin_lazy recomputes the
 // kept score and violation change of the queued positions (all of them when
 // lz_full); k_bin_scan applies tabu and aspiration to the kept values of every
@@ -3111,11 +3104,18 @@ __global__ void k_check_x(Dev d, const double *x, unsigned long long *bad)
 }
 
 // x_j + 0: a -0 from the caller is stored as +0, like every value the search
-// writes itself.
+// writes itself; with the flip direction of a binary variable (as a kernel of its
+// own 3 us of a small state's load).
 __global__ void k_canon_x(Dev d)
 {
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x)
-        d.x[j] = __dadd_rn(d.x[j], 0.0);
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x) {
+        const double x = __dadd_rn(d.x[j], 0.0);
+        d.x[j] = x;
+        if (d.n_bup > 0) {
+            const int q = __ldg(d.vpos + j);
+            if (q < d.n_bup) d.bup[q] = __double_as_longlong(x) == 0 ? 1 : 0;
+        }
+    }
 }
 
 constexpr int kResProd = 15;                      // producer warps of a residual CTA
@@ -3747,7 +3747,6 @@ cudaError_t launch_check_x(const Dev &d, const double *x, unsigned long long *ba
 cudaError_t launch_residuals(const Dev &d, const int *w, cudaStream_t st)
 {
     k_canon_x<<<grid_for(d.n, 256), 256, 0, st>>>(d);
-    if (d.n_bup > 0) k_bup_init<<<grid_for(d.n_bup, 256), 256, 0, st>>>(d);
     const int n_fp = d.m - d.n_res_int;
     const int fp_ctas = (n_fp + 31) / 32;
     const int tasks = d.n_res_int - d.n_res_short + (d.n_res_short + 31) / 32;

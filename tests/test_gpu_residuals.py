@@ -49,6 +49,35 @@ def test_residuals(chap, m, lens, fp_rows):
     bs.close()
 
 
+@pytest.mark.parametrize("m", [456 * 16, 456 * 16 + 1, 456 * 16 + 33])
+@pytest.mark.parametrize("lens", [(8,), (0, 1, 7, 8, 9, 63, 64, 65, 130)])
+def test_residuals_of_many_rows(chap, m, lens):
+    """Integral rows alone, one per warp and, from one row more than the grid has
+    warps, short ones 32 to a warp."""
+    rng = np.random.default_rng(m + len(lens))
+    n = 700
+    vt = rng.choice([inst.VAR_BIN, inst.VAR_INT], n)
+    ub = np.where(vt == inst.VAR_BIN, 1.0, 9.0)
+    k = np.array(lens)[np.arange(m) % len(lens)]
+    rows = np.repeat(np.arange(m), k)
+    at = np.arange(len(rows)) - np.repeat(np.cumsum(k) - k, k)
+    cols = (np.repeat(rng.integers(0, n, m), k) + 5 * at) % n     # distinct: 140 places before one comes again
+    prob = inst.from_triplets("many", n, m, rows, cols, rng.integers(1, 9, len(rows)) * rng.choice([-1.0, 1.0], len(rows)),
+                              np.zeros(n), ub, np.ones(n), rng.integers(-4, 5, m).astype(float), vt,
+                              rng.choice([inst.ROW_LE, inst.ROW_GE, inst.ROW_EQ], m))
+    orc = Oracle(prob)
+    bs = chap.BestShift(prob, tenure=3)
+    w = rng.integers(1, 9, size=bs.m_norm).astype(np.int32)
+    for _ in range(2):
+        x = np.floor(rng.random(n) * (ub + 1))
+        bs.set_state(x, w)
+        r, _, nv = orc.residuals(x)
+        assert np.array_equal(bs.residuals(), r)
+        st = bs.state()
+        assert st["nviol"] == nv and np.array_equal(st["w"], w)
+    bs.close()
+
+
 # the least sizes on either side of the device's check, and a last partial block
 @pytest.mark.parametrize("n", [16383, 16384, 20001])
 def test_refused_states(chap, n):
