@@ -151,6 +151,7 @@ typedef struct chap_tabu_result {
 typedef struct chap_info {
     int32_t n, m, m_norm;
     int32_t n_bin, n_int, n_cont, n_fixed;
+    int32_t kept_scores;      /* chap_tabu_run iterates on kept scores: 1; 2: from a nearly feasible start; 0: never */
     int64_t nnz, nnz_int_rows, nnz_fp_rows;
     int64_t bytes_per_pass;   /* algorithmic bytes one best-shift pass reads/writes */
     int32_t eval_blocks;      /* CTAs of one best-shift pass */
@@ -164,7 +165,7 @@ typedef struct chap_info {
     int64_t bytes_hist;       /* ... of the counting-sort kernel (long integer columns) */
     int32_t bin_lanes;        /* lanes that score one binary column (2, 4, 8 or 16) */
     int32_t nb_lanes;         /* lanes that score one short non-binary column (4, 8, 16 or 32) */
-    int32_t n_long_cols;      /* columns on the multi-CTA merge-sort path (lists over 8192 entries) */
+    int32_t n_long_cols;      /* columns on the multi-CTA paths of lists over 8192 entries (ranked or merge-sorted) */
     int32_t n_cta_cols;       /* columns on the one-CTA shared-memory sort path (129..8192 entries) */
     int32_t bin_rows;         /* 1: binary flips scored row-wise (clusters over column blocks) */
     int32_t bin_row_blocks;   /* > 0: binary flips row-blocked over this many row blocks (bin_kernel 3) */
@@ -336,14 +337,22 @@ CHAP_API chap_status chap_bs_step(struct chap_bs *h, chap_move *out);
  * stop_at_feasible) or opts->max_iters iterations have run in this call.
  * Iterations run on scores kept from one to the next inside the call
  * (evaluated from scratch at its start, then updated on the rows a move
- * changes; the same moves), in launches of many iterations.  Instances with
- * CTA- or merge-sorted columns, handles created with lazy_binary, bin_kernel 2
- * or 3 or static_scratch_only, handles whose device memory did not hold the
- * kept state, runs under an objective cutoff, and runs with counting-sorted
- * columns on fewer than 2M nonzeros that start with more than a 16th of the
- * rows violated evaluate every iteration from
- * scratch, recorded into a CUDA graph of opts->graph_iters iterations
- * (Sec. 3.1, "Kernel Specialization", last point) and replayed.
+ * changes; the same moves), in launches of many iterations.  Otherwise every
+ * iteration evaluates every column, recorded into a CUDA graph of
+ * opts->graph_iters iterations (Sec. 3.1, "Kernel Specialization", last point)
+ * and replayed:
+ *  - handles created with lazy_binary, bin_kernel 2 or 3, static_scratch_only or
+ *    as a column shard; instances without rows;
+ *  - instances with a column whose list one CTA sorts or that is longer
+ *    (chap_info n_cta_cols, n_long_cols);
+ *  - instances whose state one cluster's shared memory does not hold: more than
+ *    512 counting-sorted columns, more than 16.7M binary variables, or many short
+ *    non-binary ones (about 330,000 beside 0.8M binary ones);
+ *  - handles whose device memory did not hold the kept state at create;
+ *  - runs under an objective cutoff;
+ *  - runs with counting-sorted columns on fewer than 2M nonzeros that start with
+ *    more than a 16th of the rows violated (chosen once, at the call's start).
+ * chap_info kept_scores tells which holds for a handle.
  * opts may be NULL (the create options).  result (host) is filled on success.
  */
 CHAP_API chap_status chap_tabu_run(struct chap_bs *h, const chap_options *opts, chap_tabu_result *result);

@@ -81,7 +81,7 @@ class chap_cutoff_info(C.Structure):
 class chap_info(C.Structure):
     _fields_ = [("n", C.c_int32), ("m", C.c_int32), ("m_norm", C.c_int32),
                 ("n_bin", C.c_int32), ("n_int", C.c_int32), ("n_cont", C.c_int32), ("n_fixed", C.c_int32),
-                ("nnz", C.c_int64), ("nnz_int_rows", C.c_int64), ("nnz_fp_rows", C.c_int64),
+                ("kept_scores", C.c_int32), ("nnz", C.c_int64), ("nnz_int_rows", C.c_int64), ("nnz_fp_rows", C.c_int64),
                 ("bytes_per_pass", C.c_int64), ("eval_blocks", C.c_int32), ("n_hist_cols", C.c_int32),
                 ("launches_per_step", C.c_int32), ("grid_bin", C.c_int32), ("grid_nb", C.c_int32),
                 ("bytes_bin", C.c_int64), ("bytes_nb", C.c_int64), ("bytes_cta", C.c_int64),

@@ -1156,6 +1156,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     in.nnz = p->nnz; in.nnz_int_rows = nnz_int; in.nnz_fp_rows = p->nnz - nnz_int;
     in.eval_blocks = (bin_blk ? (int)blk_items.size() : n_tb) + n_tn + n_tc + (int)tiles_hist.size() + (int)tiles_lscan.size() +
                      (int)tiles_rgen.size();
+    in.kept_scores = !h->srch.on ? 0 : h->srch_dense ? 2 : 1;
     in.n_hist_cols = (int)hcols.size();
     in.n_long_cols = (int)(lcols.size() + rcols.size());
     in.n_cta_cols = n_tc;

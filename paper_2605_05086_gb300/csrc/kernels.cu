@@ -3877,9 +3877,13 @@ bool search_shape(Search &S, bool one_cta)
     // clusters of more than 8 CTAs are a size the device may or may not offer
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
     const int words = (S.bc + 31) / 32;
-    S.flip_words = words <= kSrFlipWords ? words : 0;
     if (S.nhist > kSrMaxHist) return false;
-    for (S.nct = one_cta && S.nblk <= kSrMaxTops ? 1 : kSrMaxCluster; S.nct >= 1; S.nct >>= 1) {
+    for (S.nct = one_cta && S.nblk <= kSrMaxTops ? 1 : kSrMaxCluster; S.nct >= 1; S.nct >>= 1)
+    for (int keep_flips = words <= kSrFlipWords ? 1 : 0; keep_flips >= 0; --keep_flips) {
+        // the flip bits go to global memory when there are many, and when the
+        // rest of the layout (of instances with many short non-binary columns)
+        // needs their place
+        S.flip_words = keep_flips ? words : 0;
         SrLocal L;
         S.smem = sr_layout(S, S.nct, nullptr, L);
         S.big_chunks = kSrBigWalk * kSrWarps * S.nct;

@@ -347,3 +347,38 @@ def test_reverse_flips_on_rounded_rows(chap, n, m, k, feas_tol):
         x = np.where(rng.random(n) < 0.05, 1.0 - prob.x0, prob.x0)
         w = rng.integers(1, 5, size=int(m + (prob.sense == 2).sum())).astype(np.int32)
         _run_equals_steps(chap, prob, (x, w), tenure=seed, feas_tol=feas_tol, iters=(1, 2, 37, 60))
+
+
+def wide_mixed(n, n_bin):
+    """n_bin binary, the rest integer in [0, 9], every variable in one row of 8."""
+    rng = np.random.default_rng(n)
+    m = n // 8
+    vt = np.where(np.arange(n) < n_bin, inst.VAR_BIN, inst.VAR_INT).astype(np.uint8)
+    ub = np.where(vt == inst.VAR_BIN, 1.0, 9.0)
+    cols = rng.permutation(n)[:8 * m]
+    a = rng.integers(1, 6, size=8 * m).astype(float)
+    return inst.from_triplets("wide", n, m, np.repeat(np.arange(m), 8), cols, a, np.zeros(n), ub, np.ones(n),
+                              np.ceil(0.3 * (a * ub[cols]).reshape(m, 8).sum(axis=1)), vt, np.full(m, inst.ROW_GE, np.uint8))
+
+
+# 70% binary up to where the flip bits and the candidate lists share a CTA's
+# memory, where only the lists fit, and past those; many integers
+@pytest.mark.parametrize("n,n_bin,kept", [(620_000, 434_000, 1), (700_000, 490_000, 1), (760_000, 532_000, 1),
+                                          (1_200_000, 840_000, 0), (400_000, 40_000, 0), (1_000, 700, 1)])
+def test_driver_by_size(chap, n, n_bin, kept):
+    """chap_info.kept_scores on both sides of what a cluster's shared memory
+    holds, and a run against steps on either driver."""
+    prob = wide_mixed(n, n_bin)
+    bs = chap.BestShift(prob, tenure=3)
+    assert bs.info.kept_scores == kept
+    bs.close()
+    _run_equals_steps(chap, prob, (prob.x0,), tenure=3, iters=(1, 12))
+
+
+def test_driver_of_other_handles(chap):
+    cover = inst.gen_setcover(seed=1, n=257, m=257, k=6)
+    hubs = integers_long_columns(4)
+    assert chap.BestShift(cover).info.kept_scores == 1
+    assert chap.BestShift(hubs).info.kept_scores == 2
+    for opts in (dict(lazy_binary=1), dict(bin_kernel=2), dict(static_scratch_only=1)):
+        assert chap.BestShift(cover, **opts).info.kept_scores == 0
