@@ -123,7 +123,9 @@ typedef struct chap_options {
     int32_t shard_count;         /* create time, default 0 or 1: the handle evaluates every column */
     int32_t bin_kernel;          /* create time: binary flips 0 automatic, 1 column-wise, 2 row-wise, 3 row-blocked */
     int32_t bin_block_rows;      /* create time: rows of one row block of bin_kernel 3 (0: 8192; 1..8192) */
-    int32_t reserved;
+    int32_t run_scores;          /* create time: scores of chap_tabu_run's iterations: 0 automatic, 1 kept from one
+                                    iteration to the next wherever the instance allows it, 2 from scratch (any
+                                    other value: automatic) */
 } chap_options;
 
 /* One move.  var = -1 means "no admissible variable has a positive score": the
@@ -151,7 +153,7 @@ typedef struct chap_tabu_result {
 typedef struct chap_info {
     int32_t n, m, m_norm;
     int32_t n_bin, n_int, n_cont, n_fixed;
-    int32_t kept_scores;      /* chap_tabu_run iterates on kept scores: 1; 2: from a nearly feasible start; 0: never */
+    int32_t kept_scores;      /* chap_tabu_run iterates on kept scores: 1; 2: from a nearly feasible state; 0: never */
     int64_t nnz, nnz_int_rows, nnz_fp_rows;
     int64_t bytes_per_pass;   /* algorithmic bytes one best-shift pass reads/writes */
     int32_t eval_blocks;      /* CTAs of one best-shift pass */
@@ -341,8 +343,8 @@ CHAP_API chap_status chap_bs_step(struct chap_bs *h, chap_move *out);
  * iteration evaluates every column, recorded into a CUDA graph of
  * opts->graph_iters iterations (Sec. 3.1, "Kernel Specialization", last point)
  * and replayed:
- *  - handles created with lazy_binary, bin_kernel 2 or 3, static_scratch_only or
- *    as a column shard; instances without rows;
+ *  - handles created with lazy_binary, bin_kernel 2 or 3, static_scratch_only,
+ *    run_scores 2 or as a column shard; instances without rows;
  *  - instances with a column whose list one CTA sorts or that is longer
  *    (chap_info n_cta_cols, n_long_cols);
  *  - instances whose state one cluster's shared memory does not hold: more than
@@ -350,8 +352,11 @@ CHAP_API chap_status chap_bs_step(struct chap_bs *h, chap_move *out);
  *    non-binary ones (about 330,000 beside 0.8M binary ones);
  *  - handles whose device memory did not hold the kept state at create;
  *  - runs under an objective cutoff;
- *  - runs with counting-sorted columns on fewer than 2M nonzeros that start with
- *    more than a 16th of the rows violated (chosen once, at the call's start).
+ *  - unless run_scores is 1, where a full pass costs less: runs that start with
+ *    more than a 16th of the rows violated (chosen once, at the call's start) with
+ *    counting-sorted columns on fewer than 2M nonzeros, or with non-binary columns
+ *    on fewer than 5,000; and all runs with non-binary columns on fewer than
+ *    200,000 nonzeros of which a move meets more than a 20th.
  * chap_info kept_scores tells which holds for a handle.
  * opts may be NULL (the create options).  result (host) is filled on success.
  */

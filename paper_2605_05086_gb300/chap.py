@@ -51,7 +51,7 @@ class chap_options(C.Structure):
     _fields_ = [("feas_tol", C.c_double), ("tenure", C.c_int32), ("graph_iters", C.c_int32),
                 ("max_iters", C.c_int64), ("stop_at_feasible", C.c_int32), ("lazy_binary", C.c_int32),
                 ("static_scratch_only", C.c_int32), ("shard_rank", C.c_int32), ("shard_count", C.c_int32),
-                ("bin_kernel", C.c_int32), ("bin_block_rows", C.c_int32), ("reserved", C.c_int32)]
+                ("bin_kernel", C.c_int32), ("bin_block_rows", C.c_int32), ("run_scores", C.c_int32)]
 
 
 class chap_move(C.Structure):

@@ -1137,8 +1137,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
         delete h;
         return CHAP_E_CUDA;
     }
-    if (keep) {
-        h->srch_dense = kind_base[T_NB_HIST] != kind_base[T_NB_HIST + 1] && p->nnz < kSrHistNnz;
+    if (keep && h->opt.run_scores != 2) {
         const std::vector<int> hist_vars(var_list.begin() + kind_base[T_NB_HIST], var_list.begin() + kind_base[T_NB_HIST + 1]);
         // mean entries a move's walk meets: sum of len^2 over the rows, per column
         double touched = 0.0;
@@ -1146,7 +1145,11 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
             const double len = (double)(p->row_ptr[i + 1] - p->row_ptr[i]);
             touched += len * len;
         }
-        search_create(h, bin_cols, nb_cols, hist_vars, p->nnz, touched / std::max(1, n));
+        touched /= std::max(1, n);
+        const SrUse use = h->opt.run_scores == 1 ? SrUse::always
+                                                 : search_use(nb_cols > 0, !hist_vars.empty(), p->nnz, touched);
+        h->srch_near = use == SrUse::near;
+        if (use != SrUse::never) search_create(h, bin_cols, nb_cols, hist_vars, p->nnz, touched);
     }
     pl.apply_blocks = (int)std::min<int64_t>(152, std::max<int64_t>(1, ((int64_t)std::max(max_col, m) + kApplyThreads - 1) / kApplyThreads));
 
@@ -1156,7 +1159,7 @@ chap_status chap_bs_create(const chap_problem *p, const chap_options *opts, void
     in.nnz = p->nnz; in.nnz_int_rows = nnz_int; in.nnz_fp_rows = p->nnz - nnz_int;
     in.eval_blocks = (bin_blk ? (int)blk_items.size() : n_tb) + n_tn + n_tc + (int)tiles_hist.size() + (int)tiles_lscan.size() +
                      (int)tiles_rgen.size();
-    in.kept_scores = !h->srch.on ? 0 : h->srch_dense ? 2 : 1;
+    in.kept_scores = !h->srch.on ? 0 : h->srch_near ? 2 : 1;
     in.n_hist_cols = (int)hcols.size();
     in.n_long_cols = (int)(lcols.size() + rcols.size());
     in.n_cta_cols = n_tc;
@@ -1534,7 +1537,7 @@ chap_status chap_tabu_run(chap_bs *h, const chap_options *opts, chap_tabu_result
         return fail(h, CHAP_E_UNSUPPORTED, "iteration counter would exceed the 32-bit tabu stamps");
     Dev &d = h->dev;
     CK(h, launch_begin_run(d, o.max_iters, o.stop_at_feasible, h->st), "begin run");
-    if (h->srch.on && !h->h_ctl->cut_on && !(h->srch_dense && h->h_ctl->nviol * kSrHistNear > h->m)) {
+    if (h->srch.on && !h->h_ctl->cut_on && !(h->srch_near && h->h_ctl->nviol * kSrNear > h->m)) {
         s = search_run(h);
         if (s != CHAP_OK) return s;
     } else {

@@ -23,7 +23,7 @@ struct chap_bs {
     std::vector<void *> allocs;
     Dev dev{};
     LaunchPlan plan{};
-    bool srch_dense = false;    // counting-sorted columns on a small matrix: search only near feasibility
+    bool srch_near = false;      // the kept-score search runs only from nearly feasible states
     chap::Search srch{};        // kept-score search of chap_tabu_run (srch.on: in use)
     // device scratch for host-memory outputs
     double *t_xhat = nullptr;

@@ -582,9 +582,32 @@ constexpr double kSrOneCtaTouched = 4096.0;
 // for the iteration graph, of 300k (2.3M) 3.8 against 4.8, 64 of 2M (20M) 10.3
 // against 26.  Near feasibility (few violated rows) the search wins at 60k too
 // (1.9 against 4.1).  The graph runs below the first with more than a row in
-// kSrHistNear violated at the start of the call.
+// kSrNear violated at the start of the call.
 constexpr long long kSrHistNnz = 2000000;
-constexpr int kSrHistNear = 16;
+constexpr int kSrNear = 16;
+// Mixed instances without counting-sorted columns: the cluster costs 20 to 30 us
+// an iteration that moves at any size (8 where most iterations only raise
+// weights), a full pass 15 to 23 us up to a few thousand nonzeros, and where a
+// move changes a large share of a small matrix the walk does the pass's work
+// again.  us an iteration (200 of them), search / graph: general 200 variables (0.6k
+// nonzeros) 28 / 19, 1,000 (3k) 26 / 23, from near 28 / 19 and, where weight updates
+// prevail, 7 / 17; general 2,000 (10k) 28 / 24 and 8 / 22 from near, 5,000 (25k) 27 / 19
+// and 10 / 18.  Rows over 5,000 variables of which a move meets 6% (29k) 26 / 18, from
+// near 38 / 19; 18% (91k) 36 / 25, 59 / 29, on integral rows 11 / 21; 33% (165k) 39 /
+// 25, 77 / 32; over 20,000 variables 10% (229k) 24 / 28, 44 / 35; 33% (791k) 39 / 33,
+// 86 / 118; over 100,000 18% (2.2M) 28 / 53, 131 / 107.
+constexpr long long kSrTinyNnz = 5000;      // below: the graph from a far state
+constexpr long long kSrDenseNnz = 200000;   // below, and above a share of the entries met of
+constexpr int kSrDenseShare = 20;           // one in kSrDenseShare: the graph
+// Use of the search: never (the graph), from nearly feasible states, always.
+enum class SrUse { never, near, always };
+inline SrUse search_use(bool short_nb, bool hist, long long nnz, double touched)
+{
+    if (hist) return nnz < kSrHistNnz ? SrUse::near : SrUse::always;
+    if (!short_nb) return SrUse::always;
+    if (nnz < kSrTinyNnz) return SrUse::near;
+    return nnz < kSrDenseNnz && touched * kSrDenseShare > (double)nnz ? SrUse::never : SrUse::always;
+}
 constexpr int kCheckDevice = 1 << 14;    // variables from which a host state is checked on the device
 constexpr int kResShort = 64;            // entries up to which integral rows share a warp in the residual kernel,
 // where there are more rows than its grid has warps (456 CTAs of 16): a row's

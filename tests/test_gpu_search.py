@@ -102,8 +102,8 @@ INSTANCES.update({
     "hubs": lambda: integers_long_columns(4),
     "hubs_700": lambda: integers_long_columns(5, n_hub=3, rows_per=700),
     "skewed": lambda: inst.gen_skewed(seed=6, n=40_000, m=20_000, n_dense=6, dense_len=6_000),
-    # the two forms in which a search with counting-sorted columns starts: many
-    # nonzeros, or few violated rows (else the iteration graph runs)
+    # the two forms in which a search with counting-sorted columns starts by
+    # itself: many nonzeros, or few violated rows (else the iteration graph runs)
     "skewed_many_nonzeros": lambda: inst.gen_skewed(seed=6, n=320_000, m=160_000, n_dense=6, dense_len=20_000),
     "skewed_near": lambda: nearly_feasible(inst.gen_skewed(seed=6, n=40_000, m=20_000, n_dense=6, dense_len=6_000)),
     "hubs_near": lambda: nearly_feasible(integers_long_columns(4)),
@@ -118,11 +118,14 @@ def _same_state(a, b):
         assert a[k] == b[k], k
 
 
+# 1: the search whatever the size and the state, 0: the library's choice
+@pytest.mark.parametrize("run_scores", [1, 0])
 @pytest.mark.parametrize("which", sorted(INSTANCES))
 @pytest.mark.parametrize("tenure", [0, 25])
-def test_search_equals_steps(chap, which, tenure):
+def test_search_equals_steps(chap, which, tenure, run_scores):
     prob = INSTANCES[which]()
-    a = chap.BestShift(prob, tenure=tenure)
+    a = chap.BestShift(prob, tenure=tenure, run_scores=run_scores)
+    assert a.info.kept_scores == 1 or not run_scores
     b = chap.BestShift(prob, tenure=tenure)
     rng = np.random.default_rng(11)
     lo, hi = np.maximum(prob.lb, -5.0), np.minimum(prob.ub, 40.0)
@@ -165,7 +168,7 @@ def test_checkpointed_tabu_and_aspiration(chap, mixed):
     results of columns with a tabu direction not used), and a best count that
     lets aspiration through."""
     prob = integers_long_columns(12) if mixed else binary_rows(12, 700, 400, 6, fp=True)
-    a = chap.BestShift(prob, tenure=5)
+    a = chap.BestShift(prob, tenure=5, run_scores=1)
     b = chap.BestShift(prob, tenure=5)
     rng = np.random.default_rng(3)
     for slack in (0, 3, 1000):
@@ -241,9 +244,10 @@ def test_short_column_lanes_fill_the_gpu(chap, n, lanes):
     bs.close()
 
 
-def _run_equals_steps(chap, prob, start, tenure=0, feas_tol=1e-9, iters=(1, 2, 9, 30)):
-    """Runs and single steps from `start` (x, w) give the same state."""
-    a = chap.BestShift(prob, tenure=tenure, feas_tol=feas_tol)
+def _run_equals_steps(chap, prob, start, tenure=0, feas_tol=1e-9, iters=(1, 2, 9, 30), kept=1):
+    """Runs of the search and single steps from `start` (x, w) give the same state."""
+    a = chap.BestShift(prob, tenure=tenure, feas_tol=feas_tol, run_scores=1)
+    assert a.info.kept_scores == kept
     b = chap.BestShift(prob, tenure=tenure, feas_tol=feas_tol)
     a.set_state(*start)
     b.set_state(*start)
@@ -364,7 +368,7 @@ def wide_mixed(n, n_bin):
 # 70% binary up to where the flip bits and the candidate lists share a CTA's
 # memory, where only the lists fit, and past those; many integers
 @pytest.mark.parametrize("n,n_bin,kept", [(620_000, 434_000, 1), (700_000, 490_000, 1), (760_000, 532_000, 1),
-                                          (1_200_000, 840_000, 0), (400_000, 40_000, 0), (1_000, 700, 1)])
+                                          (1_200_000, 840_000, 0), (400_000, 40_000, 0), (5_000, 3_500, 1)])
 def test_driver_by_size(chap, n, n_bin, kept):
     """chap_info.kept_scores on both sides of what a cluster's shared memory
     holds, and a run against steps on either driver."""
@@ -372,13 +376,40 @@ def test_driver_by_size(chap, n, n_bin, kept):
     bs = chap.BestShift(prob, tenure=3)
     assert bs.info.kept_scores == kept
     bs.close()
-    _run_equals_steps(chap, prob, (prob.x0,), tenure=3, iters=(1, 12))
+    _run_equals_steps(chap, prob, (prob.x0,), tenure=3, iters=(1, 12), kept=kept)
 
 
 def test_driver_of_other_handles(chap):
-    cover = inst.gen_setcover(seed=1, n=257, m=257, k=6)
-    hubs = integers_long_columns(4)
-    assert chap.BestShift(cover).info.kept_scores == 1
-    assert chap.BestShift(hubs).info.kept_scores == 2
-    for opts in (dict(lazy_binary=1), dict(bin_kernel=2), dict(static_scratch_only=1)):
-        assert chap.BestShift(cover, **opts).info.kept_scores == 0
+    """kept_scores by option and by kind and size of the instance: tiny mixed ones
+    and those with counting-sorted columns from nearly feasible states, small
+    dense mixed ones never, large or sparse ones always."""
+    def kept(prob, **opts):
+        bs = chap.BestShift(prob, **opts)
+        k = bs.info.kept_scores
+        bs.close()
+        return k
+
+    cover, hubs = inst.gen_setcover(seed=1, n=257, m=257, k=6), integers_long_columns(4)
+    for opts, want in [({}, 1), (dict(run_scores=1), 1), (dict(run_scores=2), 0), (dict(run_scores=7), 1),
+                       (dict(lazy_binary=1), 0), (dict(bin_kernel=2), 0), (dict(static_scratch_only=1), 0)]:
+        assert kept(cover, **opts) == want, opts
+    assert (kept(hubs), kept(hubs, run_scores=1), kept(hubs, run_scores=2)) == (2, 1, 0)
+    # 4,992 and 5,000 nonzeros
+    assert (kept(wide_mixed(4_992, 3_000)), kept(wide_mixed(5_000, 3_000))) == (2, 1)
+    sparse = inst.gen_general(seed=1, n=6_000, m=3_000, len_cap=300)
+    assert kept(sparse) == 1
+    rng = np.random.default_rng(0)
+    n, m, k = 2_000, 60, 300   # 18,000 nonzeros, a move meets an eighth of them
+    cols = np.concatenate([np.sort(rng.choice(n, size=k, replace=False)) for _ in range(m)])
+    vt = np.where(np.arange(n) % 2, inst.VAR_INT, inst.VAR_BIN).astype(np.uint8)
+    dense = inst.from_triplets("dense_mixed", n, m, np.repeat(np.arange(m), k), cols, rng.integers(1, 9, m * k).astype(float),
+                               np.zeros(n), np.where(vt == inst.VAR_BIN, 1.0, 9.0), np.ones(n), np.full(m, 900.0), vt,
+                               np.full(m, inst.ROW_GE, np.uint8))
+    assert (kept(dense), kept(dense, run_scores=1)) == (0, 1)
+    a, b = chap.BestShift(dense, tenure=3), chap.BestShift(dense, tenure=3)
+    a.run(max_iters=50, stop_at_feasible=0)
+    for _ in range(50):
+        b.step()
+    assert np.array_equal(a.state()["x"], b.state()["x"])
+    a.close()
+    b.close()
