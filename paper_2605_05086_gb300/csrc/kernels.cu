@@ -2697,8 +2697,7 @@ __global__ void __launch_bounds__(kRkThreads) k_rank_eval(Dev d, const Tile *til
             naux[u] = i < n ? __ldg(d.raux + b + i) : make_aux(kClsPost, 0);
         }
     };
-    int n = __ldg(d.rcnt + rc.run0);
-    fetch(0, n);
+    fetch(0, __ldg(d.rcnt + rc.run0));
     for (int r = 0; r < rc.runs; ++r) {
         __syncthreads();
 #pragma unroll
@@ -2711,7 +2710,9 @@ __global__ void __launch_bounds__(kRkThreads) k_rank_eval(Dev d, const Tile *til
         const int nn = r + 1 < rc.runs ? __ldg(d.rcnt + rc.run0 + r + 1) : 0;
         fetch(min(r + 1, rc.runs - 1), nn);
         // entries that count at key: those below it, and at it the pre entries
-        // (pads past the end are post entries of the largest key)
+        // (pads past the end are post entries of the largest key, and a run is
+        // never full, so the search need not tell its last two places apart)
+        static_assert(4 * kRkChunk + 2 < kRkRun, "a run ends with a pad");
         int lo[PER];
 #pragma unroll
         for (int u = 0; u < PER; ++u) lo[u] = 0;
@@ -2726,14 +2727,10 @@ __global__ void __launch_bounds__(kRkThreads) k_rank_eval(Dev d, const Tile *til
         }
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
-            // the last entry of a full run
-            if (lo[u] == kRkRun - 1 && n == kRkRun &&
-                (skey[kRkRun - 1] < key[u] || (skey[kRkRun - 1] == key[u] && spost[kRkRun - 1] == 0))) lo[u] = kRkRun;
             if (lo[u] == 0 || !cand[u]) continue;
             s[u] += __ldg(d.rsum + b + lo[u] - 1);
             dc[u] += __ldg(d.rsumc + b + lo[u] - 1);
         }
-        n = nn;
     }
 #pragma unroll
     for (int u = 0; u < PER; ++u)
