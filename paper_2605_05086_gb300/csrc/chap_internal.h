@@ -439,9 +439,9 @@ struct LaunchPlan {
     int bin_cols;              // binary columns: positions [0, bin_cols)
     int n_bin;                 // CTAs of the persistent binary kernel (0: no binary column)
     int bin_G;                 // lanes per binary column (2, 4 or 8, from the mean column length)
-    int nb_q0, nb_cols;        // positions of the short non-binary columns (<= kWarpSortMax entries)
+    int nb_q0, nb_cols;        // positions of the short non-binary columns (<= kWarpSortMax or kWarpListMax entries)
     int nb_grid;               // CTAs of the persistent short-column kernel (0: no such column)
-    int nb_G;                  // lanes per short non-binary column (4 or 8, from the mean column length)
+    int nb_G;                  // lanes per short non-binary column (4 or 8 from the mean column length, up to 32 where columns are few)
     const Tile *tiles_cta;
     int n_cta;
     int cta_smem;              // dynamic shared memory of the CTA-sort kernel
@@ -622,13 +622,18 @@ constexpr int kSrBlkPos = 256;          // positions (and physical rows) of one 
 constexpr int kSrMaxRows = 512;         // column entries (and threads) of one CTA's records
 constexpr int kApplyThreads = 1024;
 constexpr int kLazyMaxRows = 2048;      // longer moved columns re-evaluate every kept binary score
-constexpr int kWarpSortMax = 128;       // longest list of an integer short column (one warp sorts it, K <= 4)
-constexpr int kWarpListMax = 256;       // ... of a continuous short column (a delta and a marker per half, K <= 8)
+constexpr int kWarpSortMax = 128;       // longest list of an integer short column (a warp scores it by counting)
+constexpr int kWarpListMax = 256;       // ... of a continuous short column (a delta and a marker per half)
 constexpr double kBinG2MaxLen = 6.0;    // mean binary column length up to which 2 lanes score a column
 constexpr int kBinG2MinCols = 32768;    // (and only with this many binary columns: small instances are latency-bound)
 constexpr double kBinG4MaxLen = 16.0;   // ... up to which 4 lanes do
 constexpr double kBinG8MaxLen = 1.0e30; // ... up to which 8 lanes do (16 above)
-constexpr int kNbWideMin = 1024;        // short non-binary columns from which more than 8 lanes may score one
+// Short non-binary columns from which more than 8 lanes may score one.  Measured
+// on both sides of it, an iteration of the graph over general variables: 1,020
+// columns 23 us with 4 lanes and 18 with 32, 600 columns 22 to 31 and 17, 300 columns
+// 21 and 16, 18 columns 17 and 15.  So the line could lie lower: nothing measured
+// argues for 4 or 8 lanes at any number of columns below it.
+constexpr int kNbWideMin = 1024;
 constexpr double kNbG4MaxLen = 16.0;    // mean short non-binary column length up to which 4 lanes score a column (8 above)
 
 }  // namespace chap

@@ -3475,7 +3475,7 @@ int nb_lanes(int ncols, int G)
     // more lanes per column while the columns leave warps of one resident wave
     // without work (6.3k columns near a feasible point, most on the whole-warp
     // path: 8 in turn on each of 790 warps with 4 lanes, 140 us; 2 on 3,150
-    // with 16); a handful of columns is latency either way
+    // with 16); the line below which they are not is argued at kNbWideMin
     if (ncols < kNbWideMin) return G;
     const long long warps = (long long)nb_grid_size(INT_MAX, G) * kNbWarps;
     while (G < 32 && (long long)ncols * (2 * G) / 32 <= warps) G *= 2;
