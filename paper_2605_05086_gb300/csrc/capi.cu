@@ -269,7 +269,6 @@ void search_create(chap_bs *h, int bin_cols, int nb_cols, const std::vector<int>
         S.kR = dalloc<long long>(h, nb_cols);
         S.nctx = dalloc<NbCtx>(h, nb_cols);
         S.side = dalloc<unsigned char>(h, nb_cols);
-        S.clean = dalloc<unsigned char>(h, nx);
         S.kU = dalloc<long long>(h, nb_cols);
         S.cS = dalloc<long long>(h, nx);
         S.cX = dalloc<double>(h, nx);
@@ -279,7 +278,7 @@ void search_create(chap_bs *h, int bin_cols, int nb_cols, const std::vector<int>
         S.hctx = dalloc<KeepCtx>(h, hist_cols);
         long long *ho = dalloc<long long>(h, hist_cols);
         S.hoff = ho;
-        mix_ok = S.kL && S.kR && S.nctx && S.side && S.clean && S.kU && S.cS && S.cX && S.cD && S.hb && S.ha && S.hctx && ho &&
+        mix_ok = S.kL && S.kR && S.nctx && S.side && S.kU && S.cS && S.cX && S.cD && S.hb && S.ha && S.hctx && ho &&
                  h2d(ho, hoff.data(), hoff.size(), h->st) == cudaSuccess &&
                  cudaStreamSynchronize(h->st) == cudaSuccess;
     }

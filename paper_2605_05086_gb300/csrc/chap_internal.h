@@ -399,10 +399,9 @@ struct Search {
     long long *kL, *kR;      // short: bound of the score left and right of xbar
     NbCtx *nctx;
     unsigned char *side;     // bit 0: x above its lower bound, bit 1: below its upper
-    unsigned char *clean;    // cS, cX, cD are the column's best shift regardless of tabu
     long long *kU;           // short: bound of the score of every value of the column
-    long long *cS;           // score of the best shift (0: none)
-    double *cX;
+    long long *cS;           // score of the best shift regardless of tabu (0: none positive; kSrStale: not known)
+    double *cX;              // its value and violation change
     int *cD;
     HBin *hb;                // counting-sorted: kept bins (column k from hoff[k], an even number), scalars, contexts
     const long long *hoff;

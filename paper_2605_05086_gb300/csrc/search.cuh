@@ -283,9 +283,9 @@ struct SrTerm {
 };
 
 // Half with magnitude |m| of its margin (m = eps - r; |r| on an integral row),
-// violated V, coefficient sign P (a > 0) and magnitude |a|; tf: |r| where a
-// satisfied half has a tight point, else |m|; ok: the magnitudes are usable
-// floats.
+// violated V, coefficient sign P (a > 0) and magnitude |a|; tf: of a satisfied
+// half, at most |m| and, where it has a tight point, |r|; ok: the magnitudes are
+// usable floats.
 __device__ __forceinline__ SrTerm sr_term(bool V, bool P, float mf, float tf, float af, bool ok, const NbCtx &c)
 {
     const float to = V == P ? c.dl : c.dh;        // distance to the bound the breakpoint lies towards
@@ -318,12 +318,12 @@ __device__ __forceinline__ SrTerms sr_terms(long long rb, double eps, int w1, in
 {
     SrTerms o;
     bool ok = true, P;
-    float m1, m2, t1, t2, af;
+    float m1, m2, af;
     if (!FP) {
         o.v1 = rb > 0;
         o.v2 = rb < 0;
         P = a > 0;
-        m1 = m2 = t1 = t2 = fabsf((float)rb);
+        m1 = m2 = fabsf((float)rb);
         af = fabsf((float)(int)a);
     } else {
         const double rr = __longlong_as_double(rb), b1 = __dsub_rn(eps, rr), b2 = __dadd_rn(eps, rr);
@@ -333,16 +333,15 @@ __device__ __forceinline__ SrTerms sr_terms(long long rb, double eps, int w1, in
         m1 = fabsf(approx_f(b1, ok));
         m2 = fabsf(approx_f(b2, ok));
         af = fabsf(approx_f(__longlong_as_double(a), ok));
-        t1 = m1;
-        t2 = m2;
-        if (!c.isint && (o.v1 || o.v2)) t1 = t2 = fabsf(approx_f(rr, ok));
     }
-    const SrTerm t = sr_term(o.v1, P, m1, t1, af, ok, c);
+    // |r| - eps, where a satisfied half has a tight point: nearer than it and than its margin
+    const float tf = fminf(m1, m2);
+    const SrTerm t = sr_term(o.v1, P, m1, tf, af, ok, c);
     o.l = (long long)t.l * w1;
     o.r = (long long)t.r * w1;
     o.decided = t.decided;
     if (w2 < 0) return o;
-    const SrTerm u = sr_term(o.v2, !P, m2, t2, af, ok, c);
+    const SrTerm u = sr_term(o.v2, !P, m2, tf, af, ok, c);
     o.l += (long long)u.l * w2;
     o.r += (long long)u.r * w2;
     o.decided = o.decided && u.decided;
@@ -482,6 +481,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_keep_bin(Dev d, Search S)
 }
 
 constexpr long long kSrNoBound = kNoScore;   // kU of a column never evaluated
+constexpr long long kSrStale = -1;           // cS of a column whose kept result no longer holds
 
 // Contexts and bounds of the short non-binary columns: 8 lanes per column.
 __global__ void __launch_bounds__(kEvalThreads) k_keep_nb(Dev d, Search S)
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_keep_nb(Dev d, Search S)
             S.kU[p] = kSrNoBound;
             S.nctx[p] = c;
             S.side[p] = (x > lb ? 1 : 0) | (x < ub ? 2 : 0);
-            S.clean[p] = 0;
+            S.cS[p] = kSrStale;
         }
     }
 }
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(kHistThreads) k_keep_hist(Dev d, Search S, con
     }
     if (tl.aux == 0 && threadIdx.x == 0) {
         S.hctx[tl.begin] = sr_histctx(c.xb, __ldg(d.lb + c.j), __ldg(d.ub + c.j));
-        S.clean[S.nnb + tl.begin] = 0;
+        S.cS[S.nnb + tl.begin] = kSrStale;
     }
 }
 
@@ -715,7 +715,7 @@ __device__ __noinline__ void sr_entry_hist(const Search &S, const SrRec &r, int 
     if (an.alpha) atomicAdd(reinterpret_cast<unsigned long long *>(&ha->alpha), (unsigned long long)an.alpha);
     if (an.beta_c) atomicAdd(&ha->beta_c, an.beta_c);
     if (an.alpha_c) atomicAdd(&ha->alpha_c, an.alpha_c);
-    if (ch || an.beta || an.alpha || an.beta_c || an.alpha_c) S.clean[S.nnb + k] = 0;
+    if (ch || an.beta || an.alpha || an.beta_c || an.alpha_c) S.cS[S.nnb + k] = kSrStale;
 }
 
 __device__ __forceinline__ void sr_own_add(const Search &S, const SrWalk &W, SrOwn &own)
@@ -753,20 +753,6 @@ __device__ __forceinline__ void sr_reverse(const SrRec &r, double a, bool up, lo
 {
     sr_flip<true>(r.r0, r.eps, r.w1, r.w2, __double_as_longlong(a), up, s, dc);
     sr_flip<true>(r.r1, r.eps, r.w1, r.w2, __double_as_longlong(a), !up, s, dc);
-}
-
-// The same over the moved column's records in shared memory, into sh.rev and
-// sh.revc (apart from the search's body: its live ranges cost the iterations
-// without such rows 1% otherwise).
-__device__ __noinline__ void sr_reverse_rows(const Dev &d, SrShared &sh, int nI, int len, int f0, bool up)
-{
-    const int v = threadIdx.x;
-    if (v < nI || v >= len) return;
-    long long s = 0;
-    int dc = 0;
-    sr_reverse(sh.rec[v], __ldg(d.cf_val + f0 + (v - nI)), up, s, dc);
-    if (s) atomicAdd(reinterpret_cast<unsigned long long *>(&sh.rev), (unsigned long long)s);
-    if (dc) atomicAdd(&sh.revc, dc);
 }
 
 // One entry of a binary column.  The moved column's own sums are not walked:
@@ -814,7 +800,7 @@ __device__ __forceinline__ void sr_entry_nb(const Search &S, const SrTeam *T, co
     long long up = sr_rise(o.v1, n.v1, falls, r.w1, i1);
     if (r.w2 >= 0) up += sr_rise(o.v2, n.v2, rises, r.w2, i2);
     if (up) atomicAdd(reinterpret_cast<unsigned long long *>(S.kU + p), (unsigned long long)up);
-    S.clean[p] = 0;
+    S.cS[p] = kSrStale;
     sr_nmark(T, L, p);
 }
 
@@ -1294,11 +1280,10 @@ __device__ __forceinline__ void sr_refresh(const Dev &d, const Search &S, const 
     long long top;
     VCand v = sr_eval_column(d, S, L, p, true, iter, nviol, bestnv, xh, top);
     if (lane == 0) {
-        S.cS[p] = v.valid ? v.s : 0;
+        S.cS[p] = v.valid && v.s > 0 ? v.s : 0;
         if (p < S.nnb) S.kU[p] = top;
         S.cX[p] = xh;
         S.cD[p] = v.dc;
-        S.clean[p] = 1;
     }
     bool ok = v.valid && v.s > 0;
     if (!ok) return;
@@ -1326,27 +1311,25 @@ __device__ __forceinline__ void sr_load_nb(const Search &S, int gb, SrNbBlock &B
     constexpr int PER = kSrBlk / 32;
     const int lane = threadIdx.x & 31;
     long long kl[PER], kr[PER], ku[PER], cs[PER];
-    int sd[PER], cl[PER];
+    int sd[PER];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int p = gb * kSrBlk + 32 * k + lane;
         kl[k] = kr[k] = ku[k] = cs[k] = 0;
         sd[k] = 0;
-        cl[k] = 1;
         if (p < S.nnb) {
             kl[k] = __ldcg(S.kL + p);
             kr[k] = __ldcg(S.kR + p);
             ku[k] = __ldcg(S.kU + p);
             cs[k] = __ldcg(S.cS + p);
             sd[k] = __ldcg(S.side + p);
-            cl[k] = __ldcg(S.clean + p);
         }
     }
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const long long a = (sd[k] & 1) ? kl[k] : 0, b = (sd[k] & 2) ? kr[k] : 0;
-        B.s[k] = cl[k] && cs[k] > 0 ? cs[k] : 0;
-        B.u[k] = cl[k] ? 0u : sr_sat(min(max(a, b), ku[k]));
+        B.s[k] = max(cs[k], 0LL);
+        B.u[k] = cs[k] >= 0 ? 0u : sr_sat(min(max(a, b), ku[k]));
     }
 }
 
@@ -1531,7 +1514,7 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
         for (int h = threadIdx.x; h < S.nhist; h += kSrThreads) L.hc[h] = S.hctx[h];
         for (int kk = threadIdx.x; kk * nct + T.rank < S.nhist; kk += kSrThreads) {
             const int p = S.nnb + kk * nct + T.rank;
-            const long long s = S.clean[p] ? S.cS[p] : 0;
+            const long long s = S.cS[p];
             L.htops[kk] = s > 0 ? SrBest{s, d.var_list[S.bc + p], S.bc + p} : SrBest{0, kNoVar, 0};
         }
         if (threadIdx.x == 0) sh.ncand = 0;
@@ -1600,15 +1583,14 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
             }
             for (int kk = warp; kk * nct + T.rank < S.nhist; kk += kSrWarps) {
                 const int p = S.nnb + kk * nct + T.rank;
-                if (!__ldcg(S.clean + p)) {
+                if (__ldcg(S.cS + p) < 0) {
                     double xh;
                     long long top;
                     const VCand v = sr_eval_column(d, S, L, p, true, iter, nviol, bestnv, xh, top);
                     if (lane == 0) {
-                        S.cS[p] = v.valid ? v.s : 0;
+                        S.cS[p] = v.valid && v.s > 0 ? v.s : 0;
                         S.cX[p] = xh;
                         S.cD[p] = v.dc;
-                        S.clean[p] = 1;
                         L.htops[kk] = v.valid && v.s > 0 ? SrBest{v.s, __ldg(d.var_list + S.bc + p), S.bc + p}
                                                          : SrBest{0, kNoVar, 0};
                     }
@@ -1702,6 +1684,13 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
                 ch = sr_move_row(d, S, row, ai, af, dl, di, rec, integ);
                 sh.rec[threadIdx.x] = rec;
                 n = sr_chunks(rec);
+                if (FPROWS && !integ && (!MIX || b.q < S.bc)) {
+                    long long rs = 0;
+                    int rd = 0;
+                    sr_reverse(rec, af, up, rs, rd);
+                    if (rs) atomicAdd(reinterpret_cast<unsigned long long *>(&sh.rev), (unsigned long long)rs);
+                    if (rd) atomicAdd(&sh.revc, rd);
+                }
             }
             sr_count_chunks(sh, n);
             const int dnv = T.add_cta(ch);
@@ -1710,7 +1699,6 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
             if (!pending) {
                 finish(true, dnv);
                 if (!done) sr_walk_local<MIX>(d, S, T, L, gw, nw, W);
-                if (FPROWS && f1 > f0 && (!MIX || b.q < S.bc)) sr_reverse_rows(d, sh, nI, len, f0, up);
             }
         } else if (!move && !pending) {
             finish(false, 0);
@@ -1742,12 +1730,13 @@ __device__ __forceinline__ void search_body(const Dev &d, const Search &S, int n
             d.x[b.var] = xnew;
             (xnew > xold ? d.tabu_dec : d.tabu_inc)[b.var] = (int)stamp;
             if (!MIX || b.q < S.bc) {
-                S.kS[b.q] = (FPROWS ? sh.rev : 0) - b.s;
-                S.kD[b.q] = (FPROWS ? sh.revc : 0) - dc;
+                // (the whole GPU adds a pending move's own in k_search_put)
+                S.kS[b.q] = (FPROWS && !pending ? sh.rev : 0) - b.s;
+                S.kD[b.q] = (FPROWS && !pending ? sh.revc : 0) - dc;
                 d.bup[b.q] = up ? 0 : 1;
                 if (pending) L.stale[own >> T.lg] = 1;
             } else {
-                S.clean[place] = 0;
+                S.cS[place] = kSrStale;
                 if (hist) {
                     S.hctx[place - S.nnb] = sh.mc.h[1];
                 } else {
