@@ -1437,8 +1437,8 @@ __device__ __noinline__ void sr_evaluate(const Dev &d, const Search &S, const Sr
 // entries, lists and summaries in shared memory, reductions by redux.  Measured
 // per iteration, against a full pass, apply and weight update as graph nodes:
 // set cover of 2k / 200k variables 4.2 / 6 us against 11 / 18.7 (one CTA);
-// general MIP of 200k variables 40 us against 142, of 21k variables near a
-// feasible point 28 to 45 us (by instance) against 110 to 140, 2M skewed columns
+// general MIP of 200k variables 38 us against 142, of 21k variables near a
+// feasible point 26 to 43 us (by instance) against 110 to 140, 2M skewed columns
 // with 50 dense ones (every move a dense one, done by the whole GPU) 155 us against
 // 410 (16 CTAs).
 // FPROWS: there may be non-integral rows.
